@@ -12,6 +12,7 @@
 #include <string>
 #include <tuple>
 
+#include "vc_implicit.cuh"
 #include "vc_internal.cuh"
 #include "vc_krylov.cuh"
 
@@ -57,7 +58,7 @@ static int alloc_work(Mdp* m) {
     };
     const Part parts[] = {
         {(void**)&m->Vb, 4 * S},
-        {(void**)&m->U32, implicit ? 4 * S : 0},
+        {(void**)&m->U32, implicit ? 4 * (S + kUPad) : 0},
         {(void**)&m->U32s, implicit ? 4 * S : 0},
         {(void**)&m->U64, m->has_model ? 8 * S : 0},
         {(void**)&m->V64a, 8 * S},
@@ -228,7 +229,27 @@ static int loop32(Mdp* m, float* buf0, float* buf1, double tol, long long max_sw
     return VC_OK;
 }
 
-// FP64 policy evaluation V <- R_pi + gamma P_pi V until the sweep change is below tol.
+// The value-iteration loop of an implicit handle in resident launches (vc_loop.cu): the same
+// sweeps, test and control block as loop32, one host read per launch.  *launched = false
+// if the device cannot hold the grid (the caller then uses loop32).
+static int loop32_resident(Mdp* m, float* buf0, float* buf1, double tol, long long max_sweeps, int self_loop,
+                           cudaStream_t st, int* final_idx, bool* launched) {
+    Ctl& h = *m->ctl_host;
+    reset_ctl(h, tol, max_sweeps, m->spin_polls);
+    VC_CUDA(cudaMemcpyAsync(m->ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
+    int rc;
+    for (;;) {
+        if ((rc = launch_vi_loop(m, buf0, buf1, self_loop, st, launched)) || !*launched) return rc;
+        if ((rc = read_ctl(m, st))) return rc;
+        if (h.error & kErrTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
+        if (h.error & kErrBounds) return fail(VC_ERR_CUDA, "a device bounds check failed (bounds-checking build)");
+        if (h.done) break;
+        VC_CUDA(cudaMemsetAsync(&m->ctl->arrivals, 0, sizeof(unsigned int), st));
+    }
+    *final_idx = h.final_buf;
+    return VC_OK;
+}
+
 // One FP64 Bellman backup V_in -> V_out with argmax pi_out; returns max|V_out - V_in| and
 // the number of states whose argmax differs from pi_ref (if given).
 static int cert64(Mdp* m, const double* V_in, double* V_out, int32_t* pi_out, double* qgap,
@@ -802,11 +823,14 @@ int vc_value_iterate(vc_mdp* mh, float* V, double* V64_out, int32_t* pi_out, dou
             rc = fail(VC_ERR_ARG, "VC_ITER_BLOCK needs a VC_IMPLICIT handle");
             goto out;
         }
-        rc = loop32(m, V, m->Vb, tol, max_sweeps, st, &fin, [&](const float* in, float* o, SweepCtl sc) {
-            sc.self_loop = self_loop;
-            sc.block = block;
-            return launch_sweep32(m, in, o, nullptr, nullptr, sc, st);
-        });
+        bool resident = (m->fmt & 0xF) == VC_IMPLICIT && !block;
+        if (resident) rc = loop32_resident(m, V, m->Vb, tol, max_sweeps, self_loop, st, &fin, &resident);
+        if (!rc && !resident)
+            rc = loop32(m, V, m->Vb, tol, max_sweeps, st, &fin, [&](const float* in, float* o, SweepCtl sc) {
+                sc.self_loop = self_loop;
+                sc.block = block;
+                return launch_sweep32(m, in, o, nullptr, nullptr, sc, st);
+            });
     }
     if (rc) goto out;
     if (fin == 1) VC_CUDA(cudaMemcpyAsync(V, m->Vb, 4 * S, cudaMemcpyDeviceToDevice, st));

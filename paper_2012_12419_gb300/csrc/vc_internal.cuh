@@ -258,7 +258,7 @@ struct Ctl {
     unsigned long long changes;         // policy entries that differ from a reference policy
     unsigned long long cert64;          // FP64 residual bits of a standalone Bellman backup
     int error;                          // bit flags raised by kernels (infeasible policy, bad input)
-    int pad2_;
+    unsigned int arrivals;              // grid barrier of the loop kernel: arrivals since the launch
     long long spin_limit;               // polls + 1 of each bounded pipeline wait (0 = the default)
 };
 
@@ -749,6 +749,12 @@ int autotune_csr(Mdp* m, int reps, cudaStream_t st, double* best_us);
 
 // Grid of the persistent state-parallel kernels.
 int state_grid(const Mdp* m);
+
+// FP32 value-iteration loop of an implicit handle in one resident kernel (vc_loop.cu): enqueues
+// up to a bounded number of sweeps on the reset control block (buf0 / buf1 ping-pong,
+// starting from the sweeps done so far).  *launched is false when the device cannot hold the
+// grid at once (nothing was enqueued; the caller launches sweep by sweep).
+int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
 
 // Inner hosts and block size of the in-block iteration of an implicit handle.
 int block_shape(const Mdp* m, int* h_out, int* B_out);

@@ -12,13 +12,14 @@
 
 #include <mutex>
 
+#include "vc_implicit.cuh"
 #include "vc_internal.cuh"
 
 namespace vc {
 
 constexpr int kNoAllocMaxStates = 1 << 20;  // 1,048,576 states: 4 MiB of float scratch
 
-static __device__ __align__(256) float g_noalloc_U[kNoAllocMaxStates];
+static __device__ __align__(256) float g_noalloc_U[kNoAllocMaxStates + kUPad];
 static __device__ __align__(256) unsigned int g_noalloc_res[64];
 static __device__ __align__(256) Ctl g_noalloc_ctl;
 

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "vc_implicit.cuh"
 #include "vc_internal.cuh"
 #include "vc_krylov.cuh"
 
@@ -105,64 +106,11 @@ __device__ __forceinline__ T post_reward(const Model& md, const Coef<T>& c, cons
     return c.w_occ * T(occ_sum) + c.w_q * T(d.q) + loss;
 }
 
-// Defer's backup with its self-transition solved, W of post_and_defer, computed on its
-// own: in the single-instance pass 1 this form, next to the plain expect_next, timed
-// faster (93 against 108 us per sweep of the 2.5 M-state instance) than the fused one,
-// which the batched pass uses.
-// (the same from gathered values, as expect_from)
-template <int MH>
-__device__ __forceinline__ float defer_from(const Model& md, const Coef<float>& c, const Digits& d, const float* v1,
-                                           const float* v0, float va, float vf, float rx) {
-    float sm = 0.0f, pm = 0.0f;
-#pragma unroll
-    for (int k = 0; k < MH; k++) {
-        if (k < md.H) {
-            const int o = d.occ[k];
-            if (o == 1) {
-                const float p = c.pc[k] + c.pd[k];
-                sm = fmaf(p, v1[k], sm);
-                pm += p;
-            } else if (o > 1) {
-                const float p1 = c.pc[k] * (float)o;
-                sm = fmaf(p1, v1[k], sm);
-                sm = fmaf(c.pd[k], v0[k], sm);
-                pm += p1;
-                pm += c.pd[k];
-            }
-        }
-    }
-    if (d.q < md.Q) {
-        sm = fmaf(c.pa, va, sm);
-        pm += c.pa;
-    }
-    const float pf = d.ph ? c.pf1 : c.pf0;
-    sm = fmaf(pf, vf, sm);
-    pm += pf;
-    return __fdiv_rn(fmaf(c.gamma, sm, rx), fmaf(c.gamma, pm, 1.0f - c.gamma));
-}
-
-template <int MH>
-__device__ __forceinline__ float defer_self_loop(const Model& md, const Coef<float>& c, const float* __restrict__ V,
-                                                 int x, const Digits& d, float rx) {
-    float v1[MH], v0[MH];
-#pragma unroll
-    for (int k = 0; k < MH; k++) {
-        const int o = d.occ[k];
-        v1[k] = (k < md.H && o > 0) ? V[x - md.stride[k]] : 0.0f;
-        v0[k] = (k < md.H && o > 1) ? V[x - o * md.stride[k]] : 0.0f;
-    }
-    const float va = (d.q < md.Q) ? V[x + 2] : 0.0f;
-    const float vf = V[d.ph ? x - 1 : x + 1];
-    return defer_from<MH>(md, c, d, v1, v0, va, vf, rx);
-}
-
 // ---------------------------------------------------------------- implicit: pass 1
-// SL (FP32 only): also U2(x) = defer's backup with the self-transition solved.
-template <int MH, typename T, bool SL>
+// One state per thread, any precision (the FP64 backups of the refinement).
+template <int MH, typename T>
 __global__ void __launch_bounds__(kThreads) k_post(Model md, Coef<T> c, const T* __restrict__ V, T* __restrict__ U,
-                                                   T* __restrict__ U2, SweepCtl sc) {
-    static_assert(!SL || std::is_same<T, float>::value, "self-transition solve in FP32 sweeps only");
-    if (loop_done(sc)) return;
+                                                   SweepCtl sc) {
     for (int x = blockIdx.x * kThreads + threadIdx.x; x < md.S; x += gridDim.x * kThreads) {
         Digits d;
         decode<MH>(md, x, d);
@@ -171,67 +119,24 @@ __global__ void __launch_bounds__(kThreads) k_post(Model md, Coef<T> c, const T*
 #endif
         const T rx = post_reward<MH>(md, c, d);
         U[x] = rx + c.gamma * expect_next<MH>(md, c, V, x, d);
-        if constexpr (SL) U2[x] = defer_self_loop<MH>(md, c, V, x, d, rx);
     }
 }
 
-// FP32 pass 1 over pairs of states: x (even, channel phase 0) and x + 1 (phase 1) share
-// their digits and their reward (the phase does not enter it), and every value the two
-// read comes in 8-byte-aligned pairs (the strides are even): V(x - o s_k) and
-// V(x + 1 - o s_k) are adjacent, and each state's phase flip reads the other's V.  One
-// decode, one reward and half the loads and stores per state; each state's arithmetic is
-// expect_from's (and defer_from's), so U and W are those of k_post bit for bit.
-template <int MH, bool SL>
-__global__ void __launch_bounds__(kThreads) k_post_pair(Model md, Coef<float> c, const float* __restrict__ V,
-                                                        float* __restrict__ U, float* __restrict__ U2, SweepCtl sc) {
+// FP32 pass 1 over items of VW consecutive states (vc_implicit.cuh).
+template <int MH, int VW, bool SL>
+__global__ void __launch_bounds__(kThreads) k_post_vec(Model md, Coef<float> c, const float* __restrict__ V,
+                                                       float* __restrict__ U, float* __restrict__ W, SweepCtl sc) {
     if (loop_done(sc)) return;
-    const int npairs = md.S >> 1;  // S = 2 (Q + 1) (C + 1)^H is even
-    for (int t = blockIdx.x * kThreads + threadIdx.x; t < npairs; t += gridDim.x * kThreads) {
-        const int x = 2 * t;
-        Digits d0;
-        decode<MH>(md, x, d0);  // phase 0
-        Digits d1 = d0;
-        d1.ph = 1;
-#ifdef VC_DEBUG_BOUNDS
-        if (!successors_in_range<MH>(md, x, d0, sc.ctl) || !successors_in_range<MH>(md, x + 1, d1, sc.ctl)) continue;
-#endif
-        const float rx = post_reward<MH>(md, c, d0);
-        const float2 vx = *reinterpret_cast<const float2*>(V + x);
-        float v1a[MH], v1b[MH], v0a[MH], v0b[MH];
-#pragma unroll
-        for (int k = 0; k < MH; k++) {
-            const int o = d0.occ[k];
-            const float2 p1 = (k < md.H && o > 0) ? *reinterpret_cast<const float2*>(V + x - md.stride[k])
-                                                  : make_float2(0.0f, 0.0f);
-            const float2 p0 = (k < md.H && o > 1) ? *reinterpret_cast<const float2*>(V + x - o * md.stride[k])
-                                                  : make_float2(0.0f, 0.0f);
-            v1a[k] = p1.x;
-            v1b[k] = p1.y;
-            v0a[k] = p0.x;
-            v0b[k] = p0.y;
-        }
-        const float2 va = (d0.q < md.Q) ? *reinterpret_cast<const float2*>(V + x + 2) : make_float2(0.0f, 0.0f);
-        // the phase flip of x lands on x + 1, that of x + 1 on x
-        const float e0 = expect_from<MH, float>(md, c, d0, vx.x, v1a, v0a, va.x, vx.y);
-        const float e1 = expect_from<MH, float>(md, c, d1, vx.y, v1b, v0b, va.y, vx.x);
-        *reinterpret_cast<float2*>(U + x) = make_float2(rx + c.gamma * e0, rx + c.gamma * e1);
-        if constexpr (SL) {
-            const float w0 = defer_from<MH>(md, c, d0, v1a, v0a, va.x, vx.y, rx);
-            const float w1 = defer_from<MH>(md, c, d1, v1b, v0b, va.y, vx.x, rx);
-            *reinterpret_cast<float2*>(U2 + x) = make_float2(w0, w1);
-        }
-    }
+    const int items = md.S / VW;
+    for (int t = blockIdx.x * kThreads + threadIdx.x; t < items; t += gridDim.x * kThreads)
+        post_item<MH, VW, SL>(md, c, V, VW * t, U, W, sc.ctl);
 }
 
 // ---------------------------------------------------------------- implicit: pass 2
-// SL: defer takes U2(s) (its backup with the self-transition solved) instead of U(s).
-template <int MH, typename T, bool SL>
-__global__ void __launch_bounds__(kThreads) k_max(Model md, const T* __restrict__ U, const T* __restrict__ U2,
-                                                  const T* __restrict__ V_in,
+template <int MH, typename T>
+__global__ void __launch_bounds__(kThreads) k_max(Model md, const T* __restrict__ U, const T* __restrict__ V_in,
                                                   T* __restrict__ V_out, int32_t* __restrict__ pi,
                                                   T* __restrict__ qgap, SweepCtl sc) {
-    if (loop_done(sc)) return;
-    const long long sweep = loop_sweep(sc);
     T res = T(0), vabs = T(0);
     for (int s = blockIdx.x * kThreads + threadIdx.x; s < md.S; s += gridDim.x * kThreads) {
         Digits d;
@@ -247,7 +152,7 @@ __global__ void __launch_bounds__(kThreads) k_max(Model md, const T* __restrict_
                            VC_IN_BOUNDS(sc.ctl, s + md.stride[k] - 2 >= 0 && s + md.stride[k] - 2 < md.S);
             uk[k] = f ? U[s + md.stride[k] - 2] : T(-INFINITY);
         }
-        const T u = SL ? U2[s] : U[s];  // defer: the post-decision state is s itself; highest index, so ties keep lower ones
+        const T u = U[s];  // defer: the post-decision state is s itself; highest index, so ties keep lower ones
 #pragma unroll
         for (int k = 0; k < MH; k++) {
             if (uk[k] > best) {
@@ -275,7 +180,7 @@ __global__ void __launch_bounds__(kThreads) k_max(Model md, const T* __restrict_
     if (sc.mode == kModeNone) return;
     res = block_max<T, kThreads>(res);
     vabs = block_max<T, kThreads>(vabs);
-    finish_block<T>(sc, res, vabs, sweep);
+    finish_block<T>(sc, res, vabs, 0);
 }
 
 // ------------------------------------------------------- implicit: in-block iteration
@@ -301,145 +206,32 @@ __global__ void __launch_bounds__(kBlockThreads, 3) k_block(Model md, Coef<float
     finish_block<float>(sc, res, vabs, sweep);
 }
 
-// FP32 pass 2 with two states per thread and loop step: both states' gathers are issued
-// before either maximum is taken, so twice as many independent loads are in flight per
-// warp (the pass waits on the L2 latency of its gathers).  Same arithmetic and order as
-// k_max, so the same results bit for bit.
-template <int MH, bool SL>
-__global__ void __launch_bounds__(kThreads) k_max2(Model md, const float* __restrict__ U, const float* __restrict__ U2,
-                                                   const float* __restrict__ V_in, float* __restrict__ V_out,
-                                                   int32_t* __restrict__ pi, float* __restrict__ qgap, SweepCtl sc) {
+// FP32 pass 2 over the same items, with policy and Q-gap when asked for.
+template <int MH, int VW, bool SL, bool ARG>
+__global__ void __launch_bounds__(kThreads) k_max_vec(Model md, const float* __restrict__ U,
+                                                      const float* __restrict__ W, const float* __restrict__ V_in,
+                                                      float* __restrict__ V_out, int32_t* __restrict__ pi,
+                                                      float* __restrict__ qgap, SweepCtl sc) {
     if (loop_done(sc)) return;
     const long long sweep = loop_sweep(sc);
     float res = 0.0f, vabs = 0.0f;
-    const int step = gridDim.x * kThreads;
-    for (int s0 = blockIdx.x * kThreads + threadIdx.x; s0 < md.S; s0 += 2 * step) {
-        float uk[2][MH], ud[2], vin[2];
-        int sv[2];
-        bool live[2];
+    const int items = md.S / VW;
+    for (int t = blockIdx.x * kThreads + threadIdx.x; t < items; t += gridDim.x * kThreads) {
+        const int s = VW * t;
+        float vin[VW], best[VW], second[VW];
+        int arg[VW];
+        ldv<VW>(V_in + s, vin);
+        max_item<MH, VW, SL, ARG>(md, U, W, s, best, second, arg, sc.ctl);
+        if (V_out) stv<VW>(V_out + s, best);
 #pragma unroll
-        for (int t = 0; t < 2; t++) {
-            const int s = s0 + t * step;
-            sv[t] = s;
-            live[t] = s < md.S;
-            Digits d;
-            decode<MH>(md, live[t] ? s : 0, d);
-#pragma unroll
-            for (int k = 0; k < MH; k++) {
-                const bool f = live[t] && d.q >= 1 && k < md.H && d.occ[k] < md.C && (k == md.H - 1 || d.ph == 1) &&
-                               VC_IN_BOUNDS(sc.ctl, s + md.stride[k] - 2 >= 0 && s + md.stride[k] - 2 < md.S);
-                uk[t][k] = f ? U[s + md.stride[k] - 2] : -INFINITY;
+        for (int j = 0; j < VW; j++) {
+            if constexpr (ARG) {
+                if (pi) pi[s + j] = arg[j];
+                if (qgap) qgap[s + j] = second[j] == -INFINITY ? INFINITY : best[j] - second[j];
             }
-            ud[t] = live[t] ? (SL ? U2[s] : U[s]) : -INFINITY;
-            vin[t] = live[t] ? V_in[s] : 0.0f;
+            res = fmaxf(res, fabsf(best[j] - vin[j]));
+            vabs = fmaxf(vabs, fabsf(best[j]));
         }
-#pragma unroll
-        for (int t = 0; t < 2; t++) {
-            if (!live[t]) continue;
-            float best = -INFINITY, second = -INFINITY;
-            int arg = md.H;
-#pragma unroll
-            for (int k = 0; k < MH; k++) {
-                if (uk[t][k] > best) {
-                    second = best;
-                    best = uk[t][k];
-                    arg = k;
-                } else if (uk[t][k] > second) {
-                    second = uk[t][k];
-                }
-            }
-            const float u = ud[t];
-            if (u > best) {
-                second = best;
-                best = u;
-                arg = md.H;
-            } else if (u > second) {
-                second = u;
-            }
-            const int s = sv[t];
-            if (V_out) V_out[s] = best;
-            if (pi) pi[s] = arg;
-            if (qgap) qgap[s] = (second == -INFINITY) ? INFINITY : best - second;
-            res = fmaxf(res, fabsf(best - vin[t]));
-            vabs = fmaxf(vabs, fabsf(best));
-        }
-    }
-    if (sc.mode == kModeNone) return;
-    res = block_max<float, kThreads>(res);
-    vabs = block_max<float, kThreads>(vabs);
-    finish_block<float>(sc, res, vabs, sweep);
-}
-
-// Max over actions in order, lowest index on ties, for one state: its placements uk[] and
-// defer's value u (the highest index).
-template <int MH>
-__device__ __forceinline__ void max_actions(const Model& md, const float* uk, float u, float& best, float& second,
-                                            int& arg) {
-    best = -INFINITY;
-    second = -INFINITY;
-    arg = md.H;
-#pragma unroll
-    for (int k = 0; k < MH; k++) {
-        if (uk[k] > best) {
-            second = best;
-            best = uk[k];
-            arg = k;
-        } else if (uk[k] > second) {
-            second = uk[k];
-        }
-    }
-    if (u > best) {
-        second = best;
-        best = u;
-        arg = md.H;
-    } else if (u > second) {
-        second = u;
-    }
-}
-
-// Pass 2 over pairs of states s (even, channel phase 0) and s + 1 (phase 1): one decode,
-// and one 8-byte load per action serves both, since their post-decision states of a
-// placement are adjacent (s + s_k - 2 is even) and every placement feasible in phase 0
-// (the RSU) is feasible in phase 1; outputs are written as pairs.  Each state's maximum,
-// argmax and gap are k_max2's.
-template <int MH, bool SL>
-__global__ void __launch_bounds__(kThreads) k_max_pair(Model md, const float* __restrict__ U,
-                                                       const float* __restrict__ U2, const float* __restrict__ V_in,
-                                                       float* __restrict__ V_out, int32_t* __restrict__ pi,
-                                                       float* __restrict__ qgap, SweepCtl sc) {
-    if (loop_done(sc)) return;
-    const long long sweep = loop_sweep(sc);
-    float res = 0.0f, vabs = 0.0f;
-    const int npairs = md.S >> 1;
-    for (int t = blockIdx.x * kThreads + threadIdx.x; t < npairs; t += gridDim.x * kThreads) {
-        const int s = 2 * t;
-        Digits d;
-        decode<MH>(md, s, d);  // phase 0; s + 1 has the same queue and occupancies
-        float uk0[MH], uk1[MH];
-#pragma unroll
-        for (int k = 0; k < MH; k++) {
-            // phase 1: every host with a free slot; phase 0: the RSU (host H - 1) only
-            const bool f1 = d.q >= 1 && k < md.H && d.occ[k] < md.C &&
-                            VC_IN_BOUNDS(sc.ctl, s + md.stride[k] - 2 >= 0 && s + md.stride[k] - 1 < md.S);
-            const bool f0 = f1 && k == md.H - 1;
-            const float2 u2 = f1 ? *reinterpret_cast<const float2*>(U + s + md.stride[k] - 2)
-                                 : make_float2(-INFINITY, -INFINITY);
-            uk0[k] = f0 ? u2.x : -INFINITY;
-            uk1[k] = f1 ? u2.y : -INFINITY;
-        }
-        const float2 ud = *reinterpret_cast<const float2*>((SL ? U2 : U) + s);
-        const float2 vin = *reinterpret_cast<const float2*>(V_in + s);
-        float b0, c0, b1, c1;
-        int a0, a1;
-        max_actions<MH>(md, uk0, ud.x, b0, c0, a0);
-        max_actions<MH>(md, uk1, ud.y, b1, c1, a1);
-        if (V_out) *reinterpret_cast<float2*>(V_out + s) = make_float2(b0, b1);
-        if (pi) *reinterpret_cast<int2*>(pi + s) = make_int2(a0, a1);
-        if (qgap)
-            *reinterpret_cast<float2*>(qgap + s) =
-                make_float2(c0 == -INFINITY ? INFINITY : b0 - c0, c1 == -INFINITY ? INFINITY : b1 - c1);
-        res = fmaxf(res, fmaxf(fabsf(b0 - vin.x), fabsf(b1 - vin.y)));
-        vabs = fmaxf(vabs, fmaxf(fabsf(b0), fabsf(b1)));
     }
     if (sc.mode == kModeNone) return;
     res = block_max<float, kThreads>(res);
@@ -609,8 +401,9 @@ static int launch_block(Mdp* m, const float* V_in, float* V_out, SweepCtl sc, cu
             m->blk_grid = std::max(1, per_sm) * (m->num_sms > 0 ? m->num_sms : 148);
         }
         const int ntiles = (m->S + T - 1) / T;
-        k_post_pair<MH, true><<<g, kThreads, 0, st>>>(m->md, m->c32, V_in, m->U32, m->U32s, sc1);
-        kern<<<std::min(ntiles, m->blk_grid), threads, smem, st>>>(m->md, m->c32, T, m->blk_passes, V_in, m->U32,
+        float* U = m->U32 + kUShift;
+        k_post_vec<MH, 2, true><<<g, kThreads, 0, st>>>(m->md, m->c32, V_in, U, m->U32s, sc1);
+        kern<<<std::min(ntiles, m->blk_grid), threads, smem, st>>>(m->md, m->c32, T, m->blk_passes, V_in, U,
                                                                    m->U32s, V_out, sc);
         VC_CUDA(cudaGetLastError());
         return (int)VC_OK;
@@ -627,16 +420,30 @@ int launch_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* 
     const int g = state_grid(m);
     SweepCtl sc1 = sc;
     if (sc1.mode != kModeLoop32) sc1.mode = kModeNone;
+    float* U = m->U32 + kUShift;
+    const bool aligned16 = (((uintptr_t)V_in | (uintptr_t)V_out) & 15) == 0;
     count_launches(2);
     by_h(m, [&](auto mh) {
         constexpr int MH = decltype(mh)::value;
-        if (sc.self_loop) {
-            k_post_pair<MH, true><<<g, kThreads, 0, st>>>(m->md, m->c32, V_in, m->U32, m->U32s, sc1);
-            k_max_pair<MH, true><<<g, kThreads, 0, st>>>(m->md, m->U32, m->U32s, V_in, V_out, pi, qgap, sc);
-        } else {
-            k_post_pair<MH, false><<<g, kThreads, 0, st>>>(m->md, m->c32, V_in, m->U32, nullptr, sc1);
-            k_max_pair<MH, false><<<g, kThreads, 0, st>>>(m->md, m->U32, nullptr, V_in, V_out, pi, qgap, sc);
-        }
+        auto go = [&](auto vw, auto sl) {
+            constexpr int VW = decltype(vw)::value;
+            constexpr bool SL = decltype(sl)::value;
+            k_post_vec<MH, VW, SL><<<g, kThreads, 0, st>>>(m->md, m->c32, V_in, U, m->U32s, sc1);
+            if (pi || qgap)
+                k_max_vec<MH, VW, SL, true><<<g, kThreads, 0, st>>>(m->md, U, m->U32s, V_in, V_out, pi, qgap, sc);
+            else
+                k_max_vec<MH, VW, SL, false><<<g, kThreads, 0, st>>>(m->md, U, m->U32s, V_in, V_out, pi, qgap, sc);
+        };
+        auto by_vw = [&](auto sl) {
+            if (MH <= 8 && aligned16 && wide_rows(m->md))
+                go(std::integral_constant<int, MH <= 8 ? 4 : 2>(), sl);
+            else
+                go(std::integral_constant<int, 2>(), sl);
+        };
+        if (sc.self_loop)
+            by_vw(std::true_type());
+        else
+            by_vw(std::false_type());
         return 0;
     });
     VC_CUDA(cudaGetLastError());
@@ -652,8 +459,8 @@ int launch_bellman64(Mdp* m, const double* V_in, double* V_out, int32_t* pi, dou
     count_launches(2);
     by_h(m, [&](auto mh) {
         constexpr int MH = decltype(mh)::value;
-        k_post<MH, double, false><<<g, kThreads, 0, st>>>(m->md, m->c64, V_in, m->U64, nullptr, none);
-        k_max<MH, double, false><<<g, kThreads, 0, st>>>(m->md, m->U64, nullptr, V_in, V_out, pi, qgap, sc);
+        k_post<MH, double><<<g, kThreads, 0, st>>>(m->md, m->c64, V_in, m->U64, none);
+        k_max<MH, double><<<g, kThreads, 0, st>>>(m->md, m->U64, V_in, V_out, pi, qgap, sc);
         return 0;
     });
     VC_CUDA(cudaGetLastError());
@@ -668,7 +475,7 @@ int launch_resid64(Mdp* m, const int32_t* pi, const double* V64, float* r, Sweep
     count_launches(2);
     by_h(m, [&](auto mh) {
         constexpr int MH = decltype(mh)::value;
-        k_post<MH, double, false><<<g, kThreads, 0, st>>>(m->md, m->c64, V64, m->U64, nullptr, none);
+        k_post<MH, double><<<g, kThreads, 0, st>>>(m->md, m->c64, V64, m->U64, none);
         k_resid64<MH><<<g, kThreads, 0, st>>>(m->md, pi, m->U64, V64, r, sc);
         return 0;
     });

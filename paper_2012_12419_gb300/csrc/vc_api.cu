@@ -68,8 +68,9 @@ static int alloc_work(Mdp* m) {
         {(void**)&m->Rres, 4 * S},
         {(void**)&m->pi, 4 * S},
         {(void**)&m->pi2, 4 * S},
-        {(void**)&m->kr, 20 * S},
-        {(void**)&m->kr_part, 24 * (size_t)state_grid(m)},
+        {(void**)&m->kr, 20 * krylov_stride(m->S)},
+        {(void**)&m->post, m->has_model ? 4 * S : 0},
+        {(void**)&m->kr_part, 24 * (size_t)std::max(state_grid(m), m->num_sms > 0 ? m->num_sms : 148)},
         {(void**)&m->kctl, sizeof(KrylovCtl)},
         {(void**)&m->ctl, sizeof(Ctl)},
     };

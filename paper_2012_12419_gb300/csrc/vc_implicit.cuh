@@ -22,6 +22,63 @@ namespace vc {
 constexpr int kUShift = 2;   // U(0) is element kUShift of its buffer
 constexpr int kUPad = 8;     // floats of an U buffer beyond S
 
+// ------------------------------------------------------------------ model arithmetic
+// E[V(next) | x] = V(x) + sum_e p_e (V(y_e) - V(x)) from the gathered values (vx = V(x),
+// v1 / v0 the completion / departure targets of each host, va the arrival, vf the phase
+// flip): the self-loop probability is never formed, so rounding scales with value
+// differences, not with |V|.  The sum runs in a fixed order.
+template <int MH, typename T>
+__device__ __forceinline__ T expect_from(const Model& md, const Coef<T>& c, const Digits& d, T vx, const T* v1,
+                                         const T* v0, T va, T vf) {
+    T acc = T(0);
+#pragma unroll
+    for (int k = 0; k < MH; k++) {
+        if (k < md.H) {
+            const int o = d.occ[k];
+            if (o > 0) {
+                if (o == 1) {
+                    acc += (c.pc[k] + c.pd[k]) * (v1[k] - vx);  // completion and departure both empty the host
+                } else {
+                    acc += c.pc[k] * T(o) * (v1[k] - vx) + c.pd[k] * (v0[k] - vx);
+                }
+            }
+        }
+    }
+    if (d.q < md.Q) acc += c.pa * (va - vx);
+    acc += (d.ph ? c.pf1 : c.pf0) * (vf - vx);
+    return vx + acc;
+}
+
+template <int MH, typename T>
+__device__ __forceinline__ T expect_next(const Model& md, const Coef<T>& c, const T* V, int x,
+                                         const Digits& d) {
+    // every gather first (independent loads in flight together), then the sum
+    const T vx = V[x];
+    T v1[MH], v0[MH];
+#pragma unroll
+    for (int k = 0; k < MH; k++) {
+        const int o = d.occ[k];
+        v1[k] = (k < md.H && o > 0) ? V[x - md.stride[k]] : T(0);
+        v0[k] = (k < md.H && o > 1) ? V[x - o * md.stride[k]] : T(0);
+    }
+    const T va = (d.q < md.Q) ? V[x + 2] : T(0);
+    const T vf = V[d.ph ? x - 1 : x + 1];
+    return expect_from<MH, T>(md, c, d, vx, v1, v0, va, vf);
+}
+
+#ifdef VC_DEBUG_BOUNDS
+// Every state expect_next reads from post-decision state x lies in [0, S).
+template <int MH>
+__device__ __forceinline__ bool successors_in_range(const Model& md, int x, const Digits& d, Ctl* ctl) {
+    bool ok = x >= 0 && x < md.S && (d.ph ? x - 1 : x + 1) >= 0 && (d.ph ? x - 1 : x + 1) < md.S &&
+              (d.q >= md.Q || x + 2 < md.S);
+#pragma unroll
+    for (int k = 0; k < MH; k++)
+        if (k < md.H && d.occ[k] > 0) ok = ok && x - d.occ[k] * md.stride[k] >= 0 && x - md.stride[k] >= 0;
+    return VC_IN_BOUNDS(ctl, ok);
+}
+#endif
+
 // Whether rows of 2(Q + 1) codes are whole items of four (VW = 4 also needs 16-byte-aligned
 // value arrays; hosts beyond 8 keep VW = 2, whose gathered values fit the registers).
 inline bool wide_rows(const Model& md) { return (md.Q & 1) != 0; }
@@ -34,6 +91,8 @@ __device__ __forceinline__ void ldv(const float* p, float* v) {
         v[1] = t.y;
         v[2] = t.z;
         v[3] = t.w;
+    } else if constexpr (VW == 1) {
+        v[0] = *p;
     } else {
         const float2 t = *reinterpret_cast<const float2*>(p);
         v[0] = t.x;
@@ -45,6 +104,8 @@ template <int VW>
 __device__ __forceinline__ void stv(float* p, const float* v) {
     if constexpr (VW == 4)
         *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (VW == 1)
+        *p = v[0];
     else
         *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
 }
@@ -56,9 +117,9 @@ __device__ __forceinline__ bool has_host(const Model& md, int k) {
 }
 
 // Pass 1 of one item: U(x) = R(x) + gamma E[V(next) | x] of its VW states and, with SL,
-// defer's value with its self-transition solved.  Each state's arithmetic is expect_from's
-// (and defer_from's) in the same order.
-template <int MH, int VW, bool SL>
+// defer's value with its self-transition solved; EXPECT: E[V(next) | x] alone, into U.  Each
+// state's arithmetic is expect_from's (and defer_from's) in the same order.
+template <int MH, int VW, bool SL, bool EXPECT = false>
 __device__ __forceinline__ void post_item(const Model& md, const Coef<float>& c, const float* V, int x, float* U,
                                           float* W, Ctl* ctl) {
     Digits d;
@@ -139,7 +200,7 @@ __device__ __forceinline__ void post_item(const Model& md, const Coef<float>& c,
             if (room) a += c.pa * (va - vx[j]);
             a += pf * (vf - vx[j]);
             const float e = vx[j] + a;
-            u[j] = rx + c.gamma * e;
+            u[j] = EXPECT ? e : rx + c.gamma * e;
             if constexpr (SL) {
                 float s = sm[j], p = pm[i];
                 if (room) {
@@ -151,8 +212,9 @@ __device__ __forceinline__ void post_item(const Model& md, const Coef<float>& c,
                 w[j] = __fdiv_rn(fmaf(c.gamma, s, rx), fmaf(c.gamma, p, 1.0f - c.gamma));
             }
         }
-        stv<2>(U + (x + 2 * i), u + 2 * i);
+        if constexpr (!EXPECT) stv<2>(U + (x + 2 * i), u + 2 * i);
     }
+    if constexpr (EXPECT) stv<VW>(U + x, u);
     if constexpr (SL) stv<VW>(W + x, w);
 }
 

@@ -694,7 +694,8 @@ struct Mdp {
     float* Rres = nullptr;      // FP32 copy of the FP64 policy residual
     int32_t* pi = nullptr;      // policy under refinement
     int32_t* pi2 = nullptr;
-    float* kr = nullptr;        // BiCGSTAB vectors of the correction solve: r, p, v, s, t ([5][S])
+    float* kr = nullptr;        // BiCGSTAB vectors of the correction solve: r, p, v, s, t ([5][krylov_stride(S)])
+    int32_t* post = nullptr;    // post-decision states of the policy under refinement (model handles)
     double* kr_part = nullptr;  // BiCGSTAB per-block partials ([3][grid])
     KrylovCtl* kctl = nullptr;  // BiCGSTAB scalars (device) and their pinned mirror
     KrylovCtl* kctl_host = nullptr;

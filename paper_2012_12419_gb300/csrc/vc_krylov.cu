@@ -1,68 +1,514 @@
 // vc_krylov.cu -- BiCGSTAB for the correction equation (I - gamma P_pi) e = r of the
-// mixed-precision refinement (single handle): the element-wise kernels of one iteration
-// and the host driver.  The two products by the matrix are launch_apply32 (implicit model
-// or stored rows).  Iterations are enqueued in chunks sized from the observed rate of
-// decrease; the host reads the control block between chunks only.
+// mixed-precision refinement (single handle), one resident kernel for the whole solve.
+//
+// Launched kernel by kernel an iteration is five launches, 1,216 blocks' tickets on the
+// control block and FP64 block sums (two FP64 multiply-adds per SM and cycle on this chip), with
+// host reads in between.  Here at most one CTA per SM stays for the whole solve: a CTA owns the
+// same states in every vector, so only p and s cross CTAs; a grid barrier separates the five
+// steps; the threads' dot products are added as FP32 pairs (sum and error term), so FP64 is
+// left with one partial per CTA; and every CTA adds the same partials in the same order and
+// advances its own copy of the scalars.
+//
+// A dot product is a sum of FP32 chains, chain c over the states c, c + chains, c + 2 chains, ..
+// with `chains` fixed by the model's size and the device (state_grid x kThreads), and the
+// chains are added in about twice FP32's precision; so neither the width of an item nor the
+// number of CTAs changes a solve.
+//
+// The product by A = I - gamma P_pi has three forms: from the stored rows; from the implicit
+// model state by state (2H + 3 scalar gathers around x_pi(s)); and, for large models, in two
+// passes as a sweep does it: E[x(next) | .] of every post-decision state by items of four
+// (two) states, then one gather per state.  The two-pass form trades a grid barrier (1.5 us)
+// for a quarter of the load instructions.
+//
+// Bound: L2 latency of the gathers and of five short vector steps, and five (seven) barriers an
+// iteration.  Whole calls, launched kernels against this one: evaluation of a policy of
+// 524,288 states 8.6 -> 3.6 ms, gradient step of 343,750 states 12.3 -> 8.6 ms, solves of
+// 2.5 M states 10.1 -> 8.0 ms and of 640 states 0.74 -> 0.46 ms.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
+#include "vc_grid.cuh"
+#include "vc_implicit.cuh"
 #include "vc_krylov.cuh"
 
 namespace vc {
 
-// r = b, x = 0, with <b, b> and max |b|.
-__global__ void __launch_bounds__(kThreads) k_kr_init(KrylovArgs k) {
-    if (kr_done(k)) return;
-    float d0 = 0.0f, mx = 0.0f;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < k.n; i += gridDim.x * kThreads) {
-        const float b = k.b[i];
-        k.r[i] = b;
-        k.x[i] = 0.0f;
-        d0 = fmaf(b, b, d0);
-        mx = fmaxf(mx, fabsf(b));
+constexpr int kKrThreads = 512;
+constexpr int kKrOneCta = 2048;     // unknowns up to which one CTA solves alone (no grid barrier)
+constexpr int kKrItems = 128;       // least items of a CTA otherwise
+
+// Vectors of one solve (FP32, n entries each) and the reduction scratch.
+struct KrylovArgs {
+    KrylovCtl* kc;
+    Ctl* ctl;          // the handle's control block (error flags of the bounds-checking build)
+    double* part;      // [3][gridDim.x]: two partial sums and a partial max per CTA
+    const float* b;    // right-hand side and shadow residual
+    float *x, *r, *p, *v, *s, *t;
+    float* e;          // E[x(next) | .] of the two-pass product
+    int32_t* post;     // x_pi(s) of every state (implicit model; -1: infeasible, a row of the identity)
+    int n;
+    int chains;        // FP32 chains of a dot product (a multiple of 4, or at least n)
+};
+
+// Scalars of the stage, from the grid totals (one thread).
+__device__ inline void kr_advance(KrylovCtl* c, int stage, double d0, double d1, double mx) {
+    if (stage == kKrInit) {
+        c->rho = d0;  // <b, r0> with r0 = b
+        c->rmax = (float)mx;
+        // one FP32 solve reduces the residual by 2^-18 at most (the refinement's next
+        // FP64 round takes it further), so the target never asks for more
+        c->target = fmax(c->target, ldexp(mx, -18));
+        c->alpha = c->omega = 1.0;
+        c->beta = 0.0;
+        c->iter = 0;
+        if (mx < c->target) c->done = 1;
+        else if (!(d0 > 0.0)) c->done = 5;
+    } else if (stage == kKrV) {
+        // alpha = rho / <b, v>
+        if (d0 == 0.0 || !isfinite(d0)) {
+            c->done = 5;
+        } else {
+            c->alpha = c->rho / d0;
+        }
+    } else if (stage == kKrT) {
+        // omega = <t, s> / <t, t>; t = 0 means s = 0 (A is non-singular): omega = 0 and
+        // the x / r update below ends the solve with r = s = 0
+        c->omega = (d1 > 0.0) ? d0 / d1 : 0.0;
+        if (!isfinite(c->omega)) c->done = 5;
+    } else {
+        // after x += alpha p + omega s, r = s - omega t
+        c->rmax = (float)mx;
+        c->iter += 1;
+        if (mx < c->target) {
+            c->done = 1;
+        } else if (c->iter >= c->max_iter) {
+            c->done = 2;
+        } else if (c->omega == 0.0 || c->rho == 0.0 || !isfinite(mx)) {
+            c->done = 5;
+        } else {
+            c->beta = (d0 / c->rho) * (c->alpha / c->omega);
+            c->rho = d0;
+            if (!isfinite(c->beta) || d0 == 0.0) c->done = 5;
+        }
     }
-    kr_finish<kThreads>(k, kKrInit, d0, 0.0f, mx);
 }
 
-// p = r (first iteration), else p = r + beta (p - omega v).
-__global__ void __launch_bounds__(kThreads) k_kr_p(KrylovArgs k) {
-    if (kr_done(k)) return;
-    const bool first = k.kc->iter == 0;
-    const float beta = (float)k.kc->beta, omega = (float)k.kc->omega;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < k.n; i += gridDim.x * kThreads)
-        k.p[i] = first ? k.r[i] : fmaf(beta, fmaf(-omega, k.v[i], k.p[i]), k.r[i]);
-}
-
-// s = r - alpha v.
-__global__ void __launch_bounds__(kThreads) k_kr_s(KrylovArgs k) {
-    if (kr_done(k)) return;
-    const float alpha = (float)k.kc->alpha;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < k.n; i += gridDim.x * kThreads)
-        k.s[i] = fmaf(-alpha, k.v[i], k.r[i]);
-}
-
-// x += alpha p + omega s; r = s - omega t, with <b, r> and max |r|.
-__global__ void __launch_bounds__(kThreads) k_kr_x(KrylovArgs k) {
-    if (kr_done(k)) return;
-    const float alpha = (float)k.kc->alpha, omega = (float)k.kc->omega;
-    float d0 = 0.0f, mx = 0.0f;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < k.n; i += gridDim.x * kThreads) {
-        const float s = k.s[i];
-        k.x[i] += fmaf(alpha, k.p[i], omega * s);
-        const float r = fmaf(-omega, k.t[i], s);
-        k.r[i] = r;
-        d0 = fmaf(k.b[i], r, d0);
-        mx = fmaxf(mx, fabsf(r));
+// A sum of FP32 values as an unevaluated pair, every addition split exactly (Knuth's two-sum;
+// T. Ogita, S. M. Rump, S. Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26(6),
+// 2005), so it comes out as if summed in about twice FP32's precision.
+struct PairSum {
+    float s = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void add(float p) {
+        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+        c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
+        s = t;
     }
-    kr_finish<kThreads>(k, kKrX, d0, 0.0f, mx);
+    __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float os = __shfl_down_sync(0xffffffffu, s, o), oc = __shfl_down_sync(0xffffffffu, c, o);
+            add(os);
+            c += oc;
+        }
+    }
+};
+
+struct KrShared {
+    KrylovCtl c;                           // this CTA's copy of the scalars
+    float2 d0[kKrThreads / 32], d1[kKrThreads / 32];
+    unsigned int mx;                       // bits of the CTA's max |r|
+    double tot[3];
+    int fail;
+};
+
+// CTA totals -> grid totals -> scalars of `stage` in every CTA's copy.  False once a barrier
+// wait gave up.  D1, MX: whether the stage has a second dot product, a maximum.
+template <bool D1, bool MX>
+__device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, GridBarrier& bar, int stage, PairSum a0,
+                                          PairSum a1, float mx) {
+    const int w = (int)threadIdx.x >> 5, l = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
+    a0.warp_sum();
+    if (D1) a1.warp_sum();
+    const unsigned int mb = MX ? __reduce_max_sync(0xffffffffu, fbits(mx)) : 0u;
+    if (l == 0) {
+        sh.d0[w] = make_float2(a0.s, a0.c);
+        if (D1) sh.d1[w] = make_float2(a1.s, a1.c);
+        if (MX) atomicMax(&sh.mx, mb);
+    }
+    __syncthreads();
+    const int G = (int)gridDim.x;
+    if (w == 0) {
+        PairSum t0, t1;
+        if (l < nw) {
+            t0.s = sh.d0[l].x;
+            t0.c = sh.d0[l].y;
+            if (D1) {
+                t1.s = sh.d1[l].x;
+                t1.c = sh.d1[l].y;
+            }
+        }
+        t0.warp_sum();
+        if (D1) t1.warp_sum();
+        if (l == 0) {
+            const double v0 = (double)t0.s + (double)t0.c, v1 = (double)t1.s + (double)t1.c;
+            const double vm = MX ? (double)__uint_as_float(sh.mx) : 0.0;
+            if (MX) sh.mx = 0u;
+            if (G == 1) {
+                sh.tot[0] = v0;
+                sh.tot[1] = v1;
+                sh.tot[2] = vm;
+            } else {
+                k.part[blockIdx.x] = v0;
+                if (D1) k.part[G + blockIdx.x] = v1;
+                if (MX) k.part[2 * G + blockIdx.x] = vm;
+            }
+        }
+    }
+    if (!bar.arrive_and_wait()) return false;
+    if (w == 0) {
+        double v0 = 0.0, v1 = 0.0, vm = 0.0;
+        if (G > 1) {
+            for (int i = l; i < G; i += 32) {
+                v0 += __ldcg(k.part + i);
+                if (D1) v1 += __ldcg(k.part + G + i);
+                if (MX) vm = fmax(vm, __ldcg(k.part + 2 * G + i));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+                if (D1) v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+                if (MX) vm = fmax(vm, __shfl_xor_sync(0xffffffffu, vm, o));
+            }
+        } else if (l == 0) {
+            v0 = sh.tot[0];
+            v1 = sh.tot[1];
+            vm = sh.tot[2];
+        }
+        if (l == 0) kr_advance(&sh.c, stage, v0, v1, vm);
+    }
+    __syncthreads();
+    return true;
+}
+
+// ------------------------------------------------------------------------- products
+// Implicit model, one state at a time: y(s) = x(s) - gamma E[x(next) | x_pi(s)].  The policy
+// was checked feasible by the residual pass; an infeasible entry acts as the identity.
+template <int MH>
+struct ModelProduct {
+    static constexpr int kWidth = 1;
+    static constexpr bool kTwoPass = false;
+    Model md;
+    Coef<float> c;
+    const int32_t* pi;
+    __device__ __forceinline__ void setup(const KrylovArgs& k, int s) const {
+        Digits d;
+        decode<MH>(md, s, d);
+        int x = s;
+        k.post[s] = apply_action<MH>(md, s, pi[s], d, x) ? x : -1;
+    }
+    __device__ __forceinline__ void first(const KrylovArgs&, const float*, int) const {}
+    __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
+        y[0] = xin[s];
+        const int x = k.post[s];
+        if (x < 0) return;
+        Digits d;
+        decode<MH>(md, x, d);
+#ifdef VC_DEBUG_BOUNDS
+        if (!successors_in_range<MH>(md, x, d, k.ctl)) return;
+#endif
+        y[0] -= c.gamma * expect_next<MH>(md, c, xin, x, d);
+    }
+};
+
+// Implicit model in two passes over items of VW states.
+template <int MH, int VW>
+struct ModelProduct2 {
+    static constexpr int kWidth = VW;
+    static constexpr bool kTwoPass = true;
+    Model md;
+    Coef<float> c;
+    const int32_t* pi;
+    __device__ __forceinline__ void setup(const KrylovArgs& k, int s0) const {
+        for (int j = 0; j < VW; j++) {
+            Digits d;
+            decode<MH>(md, s0 + j, d);
+            int x = s0 + j;
+            k.post[s0 + j] = apply_action<MH>(md, s0 + j, pi[s0 + j], d, x) ? x : -1;
+        }
+    }
+    __device__ __forceinline__ void first(const KrylovArgs& k, const float* xin, int s) const {
+        post_item<MH, VW, false, true>(md, c, xin, s, k.e, nullptr, k.ctl);
+    }
+    __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
+        int x[VW];
+        ldv<VW>(xin + s, y);
+#pragma unroll
+        for (int j = 0; j < VW; j += 2) {
+            const int2 t = *reinterpret_cast<const int2*>(k.post + s + j);
+            x[j] = t.x;
+            x[j + 1] = t.y;
+        }
+#pragma unroll
+        for (int j = 0; j < VW; j++)
+            if (x[j] >= 0 && VC_IN_BOUNDS(k.ctl, x[j] < k.n)) y[j] -= c.gamma * k.e[x[j]];
+    }
+};
+
+// Stored rows of pi (pi = nullptr: action 0, the one row of a single-action system such as
+// the adjoint's): y(s) = x(s) - gamma (scale) sum_j val_j x[col_j], fused multiply-adds in
+// column order; the gathers of eight entries are in flight before the first of them is added.
+template <typename VT>
+struct RowProduct {
+    static constexpr int kWidth = 1;
+    static constexpr bool kTwoPass = false;
+    int A;
+    float gamma;
+    const int64_t* row_ptr;
+    const int32_t* col;
+    const VT* val;
+    const float* scale;
+    const int32_t* pi;
+    static __device__ __forceinline__ float value(const VT* p) {
+        if constexpr (sizeof(VT) == 4) return __ldg(p);
+        else return __uint_as_float((uint32_t)__ldg(p) << 16);
+    }
+    __device__ __forceinline__ void setup(const KrylovArgs&, int) const {}
+    __device__ __forceinline__ void first(const KrylovArgs&, const float*, int) const {}
+    __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
+        y[0] = xin[s];
+        const int act = pi ? pi[s] : 0;
+        if (act < 0 || act >= A) return;
+        const int64_t r = (int64_t)s * A + act;
+        const int64_t lo = __ldg(row_ptr + r);
+        const int n = (int)(__ldg(row_ptr + r + 1) - lo);
+        float acc = 0.0f;
+        for (int j0 = 0; j0 < n; j0 += 8) {
+            float w[8], g[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                w[u] = g[u] = 0.0f;
+                if (j0 + u < n) {
+                    w[u] = value(val + lo + j0 + u);
+                    const int cj = __ldg(col + lo + j0 + u);
+                    if (VC_IN_BOUNDS(k.ctl, cj >= 0 && cj < k.n)) g[u] = xin[cj];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (j0 + u < n) acc = fmaf(w[u], g[u], acc);
+        }
+        if (scale) acc *= __ldg(scale + r);
+        y[0] -= gamma * acc;
+    }
+};
+
+// ---------------------------------------------------------------------------- kernel
+template <typename Op>
+__global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, int budget) {
+    constexpr int VW = Op::kWidth;
+    __shared__ KrShared sh;
+    const int n = k.n, chains = k.chains, step = (int)blockDim.x;
+    // this CTA's items of the two-pass product's first pass: one contiguous range of states
+    const int per1 = (n / VW + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int f0 = (int)blockIdx.x * per1 + (int)threadIdx.x, f1 = min(n / VW, (int)(blockIdx.x + 1) * per1);
+    // its items of everything else: the states of one contiguous range of chains
+    const int vitems = min(n, chains) / VW;
+    const int per = (vitems + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int c0 = (int)blockIdx.x * per + (int)threadIdx.x, c1 = min(vitems, (int)(blockIdx.x + 1) * per);
+    if (threadIdx.x == 0) {
+        sh.c = *k.kc;
+        sh.mx = 0u;
+        sh.fail = 0;
+    }
+    __syncthreads();
+    GridBarrier bar{&k.kc->arrivals, gridDim.x, 0u, &sh.fail};
+    const bool resumed = sh.c.iter > 0;
+    const int stop = sh.c.iter + budget;
+    bool ok = true;
+    if (!resumed) {
+        // r = b, x = 0, with <b, b> and max |b|
+        PairSum a0;
+        float mx = 0.0f;
+        for (int v = c0; v < c1; v += step) {
+            float d0[VW] = {};
+            for (long long i = (long long)VW * v; i < n; i += chains) {
+                op.setup(k, (int)i);
+                float b[VW], z[VW] = {};
+                ldv<VW>(k.b + i, b);
+#pragma unroll
+                for (int j = 0; j < VW; j++) {
+                    d0[j] = fmaf(b[j], b[j], d0[j]);
+                    mx = fmaxf(mx, fabsf(b[j]));
+                }
+                stv<VW>(k.r + i, b);
+                stv<VW>(k.x + i, z);
+            }
+#pragma unroll
+            for (int j = 0; j < VW; j++) a0.add(d0[j]);
+        }
+        ok = kr_reduce<false, true>(k, sh, bar, kKrInit, a0, PairSum(), mx);
+    }
+    // y = A x over the owned states, with the dot products of the stage
+    auto product = [&](const float* xin, float* y, bool second) {
+        if (!bar.sync()) return false;  // x is complete
+        if constexpr (Op::kTwoPass) {
+            for (int t = f0; t < f1; t += step) op.first(k, xin, VW * t);
+            if (!bar.sync()) return false;
+        }
+        PairSum a0, a1;
+        for (int v = c0; v < c1; v += step) {
+            float d0[VW] = {}, d1[VW] = {};
+            for (long long i = (long long)VW * v; i < n; i += chains) {
+                float yv[VW], w[VW];
+                ldv<VW>((second ? xin : k.b) + i, w);
+                op.row(k, xin, (int)i, yv);
+                stv<VW>(y + i, yv);
+#pragma unroll
+                for (int j = 0; j < VW; j++) {
+                    d0[j] = fmaf(w[j], yv[j], d0[j]);
+                    d1[j] = fmaf(yv[j], yv[j], d1[j]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < VW; j++) {
+                a0.add(d0[j]);
+                a1.add(d1[j]);
+            }
+        }
+        return second ? kr_reduce<true, false>(k, sh, bar, kKrT, a0, a1, 0.0f)
+                      : kr_reduce<false, false>(k, sh, bar, kKrV, a0, a1, 0.0f);
+    };
+    while (ok && !sh.c.done && sh.c.iter < stop) {
+        // p = r (first iteration), else p = r + beta (p - omega v)
+        const bool first = sh.c.iter == 0;
+        const float beta = (float)sh.c.beta, omega0 = (float)sh.c.omega;
+        for (int v0 = c0; v0 < c1; v0 += step)
+            for (long long i = (long long)VW * v0; i < n; i += chains) {
+                float r[VW], p[VW], v[VW];
+                ldv<VW>(k.r + i, r);
+                if (!first) {
+                    ldv<VW>(k.p + i, p);
+                    ldv<VW>(k.v + i, v);
+#pragma unroll
+                    for (int j = 0; j < VW; j++) r[j] = fmaf(beta, fmaf(-omega0, v[j], p[j]), r[j]);
+                }
+                stv<VW>(k.p + i, r);
+            }
+        if (!(ok = product(k.p, k.v, false)) || sh.c.done) break;
+        // s = r - alpha v
+        const float alpha = (float)sh.c.alpha;
+        for (int v0 = c0; v0 < c1; v0 += step)
+            for (long long i = (long long)VW * v0; i < n; i += chains) {
+                float r[VW], v[VW];
+                ldv<VW>(k.r + i, r);
+                ldv<VW>(k.v + i, v);
+#pragma unroll
+                for (int j = 0; j < VW; j++) r[j] = fmaf(-alpha, v[j], r[j]);
+                stv<VW>(k.s + i, r);
+            }
+        if (!(ok = product(k.s, k.t, true)) || sh.c.done) break;
+        // x += alpha p + omega s; r = s - omega t, with <b, r> and max |r|
+        const float omega = (float)sh.c.omega;
+        PairSum a0;
+        float mx = 0.0f;
+        for (int v0 = c0; v0 < c1; v0 += step) {
+            float d0[VW] = {};
+            for (long long i = (long long)VW * v0; i < n; i += chains) {
+                float x[VW], p[VW], s[VW], t[VW], b[VW];
+                ldv<VW>(k.x + i, x);
+                ldv<VW>(k.p + i, p);
+                ldv<VW>(k.s + i, s);
+                ldv<VW>(k.t + i, t);
+                ldv<VW>(k.b + i, b);
+#pragma unroll
+                for (int j = 0; j < VW; j++) {
+                    x[j] += fmaf(alpha, p[j], omega * s[j]);
+                    s[j] = fmaf(-omega, t[j], s[j]);
+                    d0[j] = fmaf(b[j], s[j], d0[j]);
+                    mx = fmaxf(mx, fabsf(s[j]));
+                }
+                stv<VW>(k.x + i, x);
+                stv<VW>(k.r + i, s);
+            }
+#pragma unroll
+            for (int j = 0; j < VW; j++) a0.add(d0[j]);
+        }
+        ok = kr_reduce<false, true>(k, sh, bar, kKrX, a0, PairSum(), mx);
+    }
+    if (threadIdx.x != 0) return;
+    if (sh.fail) atomicOr(&k.kc->fault, 1);
+    if (blockIdx.x == 0) {
+        KrylovCtl* c = k.kc;
+        c->rho = sh.c.rho;
+        c->alpha = sh.c.alpha;
+        c->omega = sh.c.omega;
+        c->beta = sh.c.beta;
+        c->target = sh.c.target;
+        c->rmax = sh.c.rmax;
+        c->done = sh.c.done;
+        c->iter = sh.c.iter;
+    }
+}
+
+// Enqueues one launch.  The grid is at most one CTA per SM; where the device cannot hold it
+// at once (a partitioned GPU) it is halved until it can.
+template <typename Op>
+static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budget, cudaStream_t st) {
+    const int sms = m->num_sms > 0 ? m->num_sms : 148;
+    const int items = std::min(k.n, k.chains) / Op::kWidth;
+    int grid = k.n <= kKrOneCta ? 1 : std::max(1, std::min(sms, items / kKrItems));
+    for (;; grid = std::max(1, grid / 2)) {
+        const int per = (items + grid - 1) / grid;
+        const int threads = std::min(kKrThreads, std::max(32, (per + 31) / 32 * 32));
+        bool launched = false;
+        const int rc = launch_resident((const void*)k_krylov<Op>, (items + per - 1) / per, threads, 0, st, &launched,
+                                       op, k, budget);
+        if (rc || launched) return rc;
+        if (grid == 1) return fail(VC_ERR_CUDA, "the correction solve's kernel does not fit the device");
+    }
+}
+
+// States from which the two-pass product is the faster one.
+constexpr int kKrTwoPass = 600000;
+
+static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, int budget, cudaStream_t st) {
+    if (!m->has_model) {
+        if ((m->fmt & 0xF) == VC_CSR_BF16) {
+            RowProduct<uint16_t> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const uint16_t*)m->val, m->scale, pi};
+            return krylov_run(m, op, k, budget, st);
+        }
+        RowProduct<float> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const float*)m->val, m->scale, pi};
+        return krylov_run(m, op, k, budget, st);
+    }
+    const bool two = m->S >= kKrTwoPass;
+    auto go = [&](auto mh) -> int {
+        constexpr int MH = decltype(mh)::value;
+        if (two && MH <= 8 && wide_rows(m->md))
+            return krylov_run(m, ModelProduct2<MH, MH <= 8 ? 4 : 2>{m->md, m->c32, pi}, k, budget, st);
+        if (two) return krylov_run(m, ModelProduct2<MH, 2>{m->md, m->c32, pi}, k, budget, st);
+        return krylov_run(m, ModelProduct<MH>{m->md, m->c32, pi}, k, budget, st);
+    };
+    switch (m->md.H) {
+        case 1: return go(std::integral_constant<int, 1>());
+        case 2: return go(std::integral_constant<int, 2>());
+        case 3: return go(std::integral_constant<int, 3>());
+        case 4: return go(std::integral_constant<int, 4>());
+        case 5: return go(std::integral_constant<int, 5>());
+        case 6: return go(std::integral_constant<int, 6>());
+        case 7: return go(std::integral_constant<int, 7>());
+        case 8: return go(std::integral_constant<int, 8>());
+        default: return go(std::integral_constant<int, 16>());
+    }
 }
 
 int krylov_correct(Mdp* m, const int32_t* pi, const float* b, float* x, double target, long long max_iter,
                    cudaStream_t st, long long* products, bool* converged) {
     *products = 0;
     *converged = false;
-    const size_t S = (size_t)m->S;
+    const size_t S = krylov_stride(m->S);
     KrylovCtl& h = *m->kctl_host;
     memset(&h, 0, sizeof(KrylovCtl));
     h.target = target;
@@ -79,37 +525,20 @@ int krylov_correct(Mdp* m, const int32_t* pi, const float* b, float* x, double t
     k.v = m->kr + 2 * S;
     k.s = m->kr + 3 * S;
     k.t = m->kr + 4 * S;
+    k.e = m->E1;
+    k.post = m->post;
     k.n = m->S;
-    const int g = state_grid(m);
-    count_launches(1);
-    k_kr_init<<<g, kThreads, 0, st>>>(k);
-    VC_CUDA(cudaGetLastError());
+    k.chains = state_grid(m) * kThreads;
+    // iterations of one launch: about a quarter of a second
+    const int budget = (int)std::min<long long>(1 << 20, std::max<long long>(4, (long long)(1e10 / m->S)));
     int rc;
-    long long chunk = 4;
-    float r_prev = -1.0f;
     for (;;) {
-        for (long long i = 0; i < chunk; i++) {
-            count_launches(3);
-            k_kr_p<<<g, kThreads, 0, st>>>(k);
-            if ((rc = launch_apply32(m, pi, k.p, k.v, b, kKrV, k, st))) return rc;
-            k_kr_s<<<g, kThreads, 0, st>>>(k);
-            if ((rc = launch_apply32(m, pi, k.s, k.t, k.s, kKrT, k, st))) return rc;
-            k_kr_x<<<g, kThreads, 0, st>>>(k);
-            VC_CUDA(cudaGetLastError());
-        }
+        if ((rc = krylov_launch(m, pi, k, budget, st))) return rc;
         VC_CUDA(cudaMemcpyAsync(&h, m->kctl, sizeof(KrylovCtl), cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
+        if (h.fault) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
         if (h.done) break;
-        // next chunk: the iterations the last chunk's rate of decrease predicts (2 .. 64)
-        long long next = 2 * chunk;
-        if (r_prev > 0.0f && h.rmax > 0.0f && h.rmax < r_prev) {
-            const double rate = log((double)h.rmax / r_prev) / (double)chunk;  // < 0
-            next = (long long)ceil(log(h.target / (double)h.rmax) / rate);
-        }
-        r_prev = h.rmax;
-        chunk = std::min<long long>(std::max<long long>(next, 2), 64);
-        chunk = std::min<long long>(chunk, (long long)h.max_iter - h.iter);
-        if (chunk < 1) chunk = 1;
+        VC_CUDA(cudaMemsetAsync(&m->kctl->arrivals, 0, sizeof(unsigned int), st));
     }
     *products = 2LL * h.iter;
     *converged = (h.done == 1);

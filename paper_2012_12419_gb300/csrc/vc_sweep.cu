@@ -22,7 +22,6 @@
 
 #include "vc_implicit.cuh"
 #include "vc_internal.cuh"
-#include "vc_krylov.cuh"
 
 namespace vc {
 
@@ -31,63 +30,6 @@ int state_grid(const Mdp* m) {
     const long long cap = (long long)(m->num_sms > 0 ? m->num_sms : 148) * 8;
     return (int)(need < cap ? need : cap);
 }
-
-// ------------------------------------------------------------------ model arithmetic
-// E[V(next) | x] = V(x) + sum_e p_e (V(y_e) - V(x)) from the gathered values (vx = V(x),
-// v1 / v0 the completion / departure targets of each host, va the arrival, vf the phase
-// flip): the self-loop probability is never formed, so rounding scales with value
-// differences, not with |V|.  The sum runs in a fixed order.
-template <int MH, typename T>
-__device__ __forceinline__ T expect_from(const Model& md, const Coef<T>& c, const Digits& d, T vx, const T* v1,
-                                         const T* v0, T va, T vf) {
-    T acc = T(0);
-#pragma unroll
-    for (int k = 0; k < MH; k++) {
-        if (k < md.H) {
-            const int o = d.occ[k];
-            if (o > 0) {
-                if (o == 1) {
-                    acc += (c.pc[k] + c.pd[k]) * (v1[k] - vx);  // completion and departure both empty the host
-                } else {
-                    acc += c.pc[k] * T(o) * (v1[k] - vx) + c.pd[k] * (v0[k] - vx);
-                }
-            }
-        }
-    }
-    if (d.q < md.Q) acc += c.pa * (va - vx);
-    acc += (d.ph ? c.pf1 : c.pf0) * (vf - vx);
-    return vx + acc;
-}
-
-template <int MH, typename T>
-__device__ __forceinline__ T expect_next(const Model& md, const Coef<T>& c, const T* __restrict__ V, int x,
-                                         const Digits& d) {
-    // every gather first (independent loads in flight together), then the sum
-    const T vx = V[x];
-    T v1[MH], v0[MH];
-#pragma unroll
-    for (int k = 0; k < MH; k++) {
-        const int o = d.occ[k];
-        v1[k] = (k < md.H && o > 0) ? V[x - md.stride[k]] : T(0);
-        v0[k] = (k < md.H && o > 1) ? V[x - o * md.stride[k]] : T(0);
-    }
-    const T va = (d.q < md.Q) ? V[x + 2] : T(0);
-    const T vf = V[d.ph ? x - 1 : x + 1];
-    return expect_from<MH, T>(md, c, d, vx, v1, v0, va, vf);
-}
-
-#ifdef VC_DEBUG_BOUNDS
-// Every state expect_next reads from post-decision state x lies in [0, S).
-template <int MH>
-__device__ __forceinline__ bool successors_in_range(const Model& md, int x, const Digits& d, Ctl* ctl) {
-    bool ok = x >= 0 && x < md.S && (d.ph ? x - 1 : x + 1) >= 0 && (d.ph ? x - 1 : x + 1) < md.S &&
-              (d.q >= md.Q || x + 2 < md.S);
-#pragma unroll
-    for (int k = 0; k < MH; k++)
-        if (k < md.H && d.occ[k] > 0) ok = ok && x - d.occ[k] * md.stride[k] >= 0 && x - md.stride[k] >= 0;
-    return VC_IN_BOUNDS(ctl, ok);
-}
-#endif
 
 // Expected one-step reward of the post-decision state: occupancy, queue and losses
 // (departures lose their tasks, a full queue loses the arrival).
@@ -303,33 +245,6 @@ __global__ void __launch_bounds__(kThreads) k_correct32(Model md, Coef<float> c,
     finish_block<float>(sc, res, vabs, sweep);
 }
 
-// Product by the correction matrix for the BiCGSTAB solve: y(s) = x(s) - gamma
-// E[x(next) | x_pi(s)], with the stage's partial sums <w, y> and <y, y>.  The policy was
-// checked feasible by the residual pass; an infeasible entry would act as the identity.
-template <int MH>
-__global__ void __launch_bounds__(kThreads) k_apply32(Model md, Coef<float> c, const int32_t* __restrict__ pi,
-                                                      const float* __restrict__ xin, float* __restrict__ y,
-                                                      const float* __restrict__ w, int stage, KrylovArgs k) {
-    if (kr_done(k)) return;
-    float d0 = 0.0f, d1 = 0.0f;
-    for (int s = blockIdx.x * kThreads + threadIdx.x; s < md.S; s += gridDim.x * kThreads) {
-        Digits d;
-        decode<MH>(md, s, d);
-        int x = s;
-        float yv = xin[s];
-        if (apply_action<MH>(md, s, pi[s], d, x)) {
-#ifdef VC_DEBUG_BOUNDS
-            if (successors_in_range<MH>(md, x, d, k.ctl))
-#endif
-                yv -= c.gamma * expect_next<MH>(md, c, xin, x, d);
-        }
-        y[s] = yv;
-        d0 = fmaf(w[s], yv, d0);
-        d1 = fmaf(yv, yv, d1);
-    }
-    kr_finish<kThreads>(k, stage, d0, d1, 0.0f);
-}
-
 __global__ void k_axpy64(double* __restrict__ V, const float* __restrict__ e, int n) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) V[i] += (double)e[i];
 }
@@ -489,18 +404,6 @@ int launch_correct32(Mdp* m, const int32_t* pi, const float* r, const float* e_i
     count_launches(1);
     by_h(m, [&](auto mh) {
         k_correct32<decltype(mh)::value><<<state_grid(m), kThreads, 0, st>>>(m->md, m->c32, pi, r, e_in, e_out, sc);
-        return 0;
-    });
-    VC_CUDA(cudaGetLastError());
-    return VC_OK;
-}
-
-int launch_apply32(Mdp* m, const int32_t* pi, const float* x, float* y, const float* w, int stage,
-                   const KrylovArgs& k, cudaStream_t st) {
-    if (!m->has_model) return csr_apply32(m, pi, x, y, w, stage, k, st);
-    count_launches(1);
-    by_h(m, [&](auto mh) {
-        k_apply32<decltype(mh)::value><<<state_grid(m), kThreads, 0, st>>>(m->md, m->c32, pi, x, y, w, stage, k);
         return 0;
     });
     VC_CUDA(cudaGetLastError());

@@ -230,9 +230,9 @@ static int loop32(Mdp* m, float* buf0, float* buf1, double tol, long long max_sw
     return VC_OK;
 }
 
-// The value-iteration loop of an implicit handle in resident launches (vc_loop.cu): the same
-// sweeps, test and control block as loop32, one host read per launch.  *launched = false
-// if the device cannot hold the grid (the caller then uses loop32).
+// The value-iteration loop in resident launches (vc_loop.cu, vc_csr_loop.cu): the same sweeps,
+// test and control block as loop32, one host read per launch.  *launched = false if no
+// resident kernel serves the handle (the caller then uses loop32).
 static int loop32_resident(Mdp* m, float* buf0, float* buf1, double tol, long long max_sweeps, int self_loop,
                            cudaStream_t st, int* final_idx, bool* launched) {
     Ctl& h = *m->ctl_host;
@@ -240,7 +240,9 @@ static int loop32_resident(Mdp* m, float* buf0, float* buf1, double tol, long lo
     VC_CUDA(cudaMemcpyAsync(m->ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
     int rc;
     for (;;) {
-        if ((rc = launch_vi_loop(m, buf0, buf1, self_loop, st, launched)) || !*launched) return rc;
+        rc = (m->fmt & 0xF) == VC_IMPLICIT ? launch_vi_loop(m, buf0, buf1, self_loop, st, launched)
+                                           : launch_csr_loop(m, buf0, buf1, self_loop, st, launched);
+        if (rc || !*launched) return rc;
         if ((rc = read_ctl(m, st))) return rc;
         if (h.error & kErrTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
         if (h.error & kErrBounds) return fail(VC_ERR_CUDA, "a device bounds check failed (bounds-checking build)");
@@ -824,7 +826,7 @@ int vc_value_iterate(vc_mdp* mh, float* V, double* V64_out, int32_t* pi_out, dou
             rc = fail(VC_ERR_ARG, "VC_ITER_BLOCK needs a VC_IMPLICIT handle");
             goto out;
         }
-        bool resident = (m->fmt & 0xF) == VC_IMPLICIT && !block;
+        bool resident = !block;
         if (resident) rc = loop32_resident(m, V, m->Vb, tol, max_sweeps, self_loop, st, &fin, &resident);
         if (!rc && !resident)
             rc = loop32(m, V, m->Vb, tol, max_sweeps, st, &fin, [&](const float* in, float* o, SweepCtl sc) {

@@ -646,7 +646,7 @@ static int enumerate_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
         if (ts >= 4 && ts % 4 == 0) sizes.push_back(ts);
     }
     unsigned long long* dcap = nullptr;
-    unsigned long long hcap[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    unsigned long long hcap[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // by size; the last: chunks of 32 / A states
     VC_CUDA(cudaMallocAsync((void**)&dcap, sizeof(hcap), st));
     VC_CUDA(cudaMemsetAsync(dcap, 0, sizeof(hcap), st));
     for (size_t i = 0; i < sizes.size(); ++i) {
@@ -654,11 +654,16 @@ static int enumerate_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
         count_launches(1);
         k_tile_cap<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(m->row_ptr, m->S, m->A, sizes[i], nt, dcap + i);
     }
+    const int chunk = 32 / m->A;  // states of a chunk of the resident loop
+    const int64_t nchunks = ((int64_t)m->S + chunk - 1) / chunk;
+    count_launches(1);
+    k_tile_cap<<<(unsigned)((nchunks + 255) / 256), 256, 0, st>>>(m->row_ptr, m->S, m->A, chunk, nchunks, dcap + 7);
     VC_CUDA(cudaGetLastError());
     VC_CUDA(cudaMemcpyAsync(hcap, dcap, sizeof(hcap), cudaMemcpyDeviceToHost, st));
     VC_CUDA(cudaFreeAsync(dcap, st));
     VC_CUDA(cudaStreamSynchronize(st));
     for (size_t i = 0; i < sizes.size(); ++i) cands.push_back({sizes[i], (long long)hcap[i] + 16});
+    m->loop_cap = (int64_t)std::min<unsigned long long>(std::max(hcap[7], 1ull), 1ull << 20);
     // one attribute per kernel instance: allow the largest request, launches ask for less
     int dyn_limit = 0;
     cudaError_t e = bf16 ? set_tma_smem_any<uint16_t>(apad, smem_blk, &dyn_limit)
@@ -696,6 +701,8 @@ static int enumerate_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
 
 // Default plan: the first candidate (the direct kernel if none fits).
 int plan_csr(Mdp* m, cudaStream_t st) {
+    // the columns' tail padding: copies are rounded up to 16 bytes and may be read as columns
+    VC_CUDA(cudaMemsetAsync(m->col + m->nnz_stored, 0, 4 * 16, st));
     // a handle built with its sliced copy takes its plan from the sliced layout
     if (m->fmt & VC_SLICED) {
         m->plan = CsrPlan();

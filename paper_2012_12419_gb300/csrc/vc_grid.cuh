@@ -1,9 +1,12 @@
-// vc_grid.cuh -- grid barrier of the resident kernels and their launch.
+// vc_grid.cuh -- grid barrier of the resident kernels, their launch and the stopping test of
+// the value-iteration loops among them.
 //
 // The kernels are cooperative launches of at most the resident grid, so every block of a
 // barrier runs; each wait still has an iteration limit, after which the block gives up, the
 // kernel flags a timeout and returns.
 #pragma once
+
+#include <math.h>
 
 #include "vc_internal.cuh"
 
@@ -39,6 +42,40 @@ struct GridBarrier {
     __device__ __forceinline__ bool sync() {
         __syncthreads();
         return arrive_and_wait();
+    }
+};
+
+// Step 3's test on every thread of a CTA from the sweep's residual r and max|V'| vm:
+// finish_block's decision, in the same order.  4 ulp(vm) is a power of two, so for vm
+// above 2^-100 both sides of r < max(tol, 4 ulp) are compared in FP32 exactly (tol rounded
+// up to FP32: r < tol iff r < that).
+struct LoopVerdict {
+    double tol;
+    float tol32, best;
+    int since;
+    long long max_sweeps;
+    __device__ int operator()(float r, float vm, long long k) {
+        bool below;
+        if (vm >= 0x1p-100f) {
+            const float ulp4 = __uint_as_float((fbits(vm) & 0x7f800000u) - (21u << 23));
+            below = r < tol32 || r < ulp4;
+        } else {
+            int e = 0;
+            frexpf(vm, &e);
+            const double ulp = vm > 0.0f ? ldexp(1.0, e - 24) : 0.0;
+            below = (double)r < fmax(tol, 4.0 * ulp);
+        }
+        int done = 0;
+        if (below) {
+            done = 1;
+        } else if (r < best) {
+            best = r;
+            since = 0;
+        } else if (++since >= kStallSweeps) {
+            done = 3;
+        }
+        if (!done && k >= max_sweeps) done = 2;
+        return done;
     }
 };
 

@@ -671,6 +671,7 @@ struct Mdp {
     double* R64 = nullptr;      // FP64 rows without a register generator); the FP64 steps use them
     double* rate_tab = nullptr; // rates.occ_tab (device, owned)
     CsrPlan plan;
+    int64_t loop_cap = 0;       // most entries of 32 / A consecutive states' rows (the resident loop's chunks)
     std::string tune_report;    // candidates and times of the last autotune
     // sliced copy of the stored matrix (SELL-C-sigma, C = 32 states per slice): one
     // 128-byte-aligned record per slice in a byte slab (header, state map, R / scale,
@@ -756,6 +757,10 @@ int state_grid(const Mdp* m);
 // starting from the sweeps done so far).  *launched is false when the device cannot hold the
 // grid at once (nothing was enqueued; the caller launches sweep by sweep).
 int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
+
+// The same loop over a stored matrix that stays in L2 (vc_csr_loop.cu); *launched is also
+// false when the matrix or its schedule is not one the loop serves.
+int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
 
 // Inner hosts and block size of the in-block iteration of an implicit handle.
 int block_shape(const Mdp* m, int* h_out, int* B_out);

@@ -14,8 +14,6 @@
 // instructions), then two barriers of ~1.5 us.  Measured per sweep, launched kernels
 // against this loop: 45 -> 28 us at 2.5 M states (H = 7), 18.3 -> 8.4 us at 343,750 states
 // with the self-transition solve (VW = 2), whole solves of 640 states 2.89 -> 0.76 ms.
-#include <math.h>
-
 #include <algorithm>
 #include <type_traits>
 
@@ -31,40 +29,6 @@ constexpr int kLoopThreads = 512;
 // round trips); four arrays of 8,192 floats also fit beside the L1's needs.
 constexpr int kLoopOneCta = 8192;
 constexpr int kLoopItems = 256;    // least items of a CTA of the multi-CTA loop
-
-// Step 3's test on every thread of a CTA from the sweep's residual r and max|V'| vm:
-// finish_block's decision, in the same order.  4 ulp(vm) is a power of two, so for vm
-// above 2^-100 both sides of r < max(tol, 4 ulp) are compared in FP32 exactly (tol rounded
-// up to FP32: r < tol iff r < that).
-struct LoopVerdict {
-    double tol;
-    float tol32, best;
-    int since;
-    long long max_sweeps;
-    __device__ int operator()(float r, float vm, long long k) {
-        bool below;
-        if (vm >= 0x1p-100f) {
-            const float ulp4 = __uint_as_float((fbits(vm) & 0x7f800000u) - (21u << 23));
-            below = r < tol32 || r < ulp4;
-        } else {
-            int e = 0;
-            frexpf(vm, &e);
-            const double ulp = vm > 0.0f ? ldexp(1.0, e - 24) : 0.0;
-            below = (double)r < fmax(tol, 4.0 * ulp);
-        }
-        int done = 0;
-        if (below) {
-            done = 1;
-        } else if (r < best) {
-            best = r;
-            since = 0;
-        } else if (++since >= kStallSweeps) {
-            done = 3;
-        }
-        if (!done && k >= max_sweeps) done = 2;
-        return done;
-    }
-};
 
 // SMEM: one CTA, V's two buffers, U and W in shared memory (4 S + kUPad floats); else W, U
 // are the handle's buffers and V the caller's pair.

@@ -64,6 +64,14 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
+// The same copy with the L2's default policy (data that every sweep reads again).
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+
 // Poll limit of the pipeline waits of one sweep: the handle's cap when one was set (a
 // host-side fault-injection hook), else kSpinLimit.  Drains of in-flight copies always
 // use kSpinLimit.

@@ -2,7 +2,8 @@
 // of the placement MDP solved together (each by Algorithm 3 with its own gamma, its own
 // convergence test and its own sweep count).
 //
-// Layout: the instances' state ranges are concatenated; a tile table cuts every range into
+// Layout: the instances' state ranges are concatenated (inside the handle each starts on 256
+// bytes; the caller's arrays are packed); a tile table cuts every range into
 // tiles of at most `ts` states that never straddle two instances.  Every sweep kernel is
 // persistent (a few CTAs per SM, grid-stride over the tile table); a tile of an instance
 // that has terminated returns at once.  Per sweep and instance, each tile folds its
@@ -11,16 +12,19 @@
 // FP32 stall, max_sweeps) and retires the instance from the active count.  All active
 // instances advance one sweep per launch, so a launch's parity names the ring slot.
 //
-// The FP32 loop is one CUDA graph: a conditional WHILE node whose body is two sweeps (the
-// ping-pong pair) and a one-thread kernel that keeps the loop running while any instance is
-// active and the sweep budget lasts.  There are no inter-CTA waits anywhere: instances only
-// couple through their per-sweep tickets.
+// The FP32 loop is one resident kernel (vc_batch_loop.cu) where it serves the batch, else one
+// CUDA graph: a conditional WHILE node whose body is two sweeps (the ping-pong pair) and a
+// one-thread kernel that keeps the loop running while any instance is active and the sweep
+// budget lasts.  There are no inter-CTA waits in the graph: instances only couple through
+// their per-sweep tickets.
 #include <math.h>
 
 #include <algorithm>
 #include <type_traits>
 #include <vector>
 
+#include "vc_batch.cuh"
+#include "vc_implicit.cuh"
 #include "vc_internal.cuh"
 #include "vc_krylov.cuh"
 
@@ -33,41 +37,6 @@ namespace vc {
         const cudaError_t le_ = cudaGetLastError();                        \
         if (le_ != cudaSuccess) return vc::cuda_fail(le_, "launch: " what); \
     } while (0)
-
-struct InstDesc {
-    Model md;
-    Coef<float> c32;
-    Coef<double> c64;
-    long long off;  // first state in the concatenated arrays
-    int S;
-    int blk_h;      // inner hosts of the in-block iteration's blocks (2(Q+1)(C+1)^blk_h states)
-};
-
-struct BatchTile {
-    int inst;
-    int start;  // first state, relative to the instance
-    int count;
-    int pad_;
-};
-
-// Device-side control of the batched loops (SoA over instances).
-struct BatchCtl {
-    int* done;                 // 0 running, 1 converged, 2 max sweeps, 3 FP32 stall
-    int* sweeps;
-    int* ticket;
-    const int* tiles_of;       // tiles per instance (constant)
-    int* final_buf;            // buffer of the last iterate (0: A, 1: B)
-    int* since_best;
-    float* best_res;
-    unsigned int* res32;       // [2n] ring of two slots
-    unsigned int* vmax32;      // [2n]
-    unsigned long long* res64; // [n] FP64 residual of a certificate / residual pass
-    int* active;               // instances still running
-    long long* iters;          // sweeps launched by the graph loop
-    const long long* max_sweeps; // loop parameters in device memory, so one captured graph
-    const double* tol;           // serves every call
-    const float* tol_scale;      // per-instance factor on tol (nullptr: 1)
-};
 
 // Instance descriptor of a tile, staged in shared memory once per tile.
 __device__ __forceinline__ void load_desc(const InstDesc* __restrict__ descs, int inst, InstDesc& sd) {
@@ -939,18 +908,32 @@ __global__ void k_bkr_reset(BatchKrylov K, int n, double target, const float* to
     }
 }
 
-// Per-instance selection of the final ping-pong buffer into out (float or double).
-template <typename TI, typename TO>
-__global__ void k_bselect(const InstDesc* __restrict__ descs, const BatchTile* __restrict__ tiles, int ntiles,
-                          const int* __restrict__ final_buf, const TI* __restrict__ A, const TI* __restrict__ B,
-                          TO* __restrict__ out) {
+// The caller's packed array into the handle's, and back.
+template <typename T, bool kImport>
+__global__ void k_bcopy(const InstDesc* __restrict__ descs, const BatchTile* __restrict__ tiles, int ntiles,
+                        const T* __restrict__ in, T* __restrict__ out) {
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const BatchTile tl = tiles[t];
-        const long long off = descs[tl.inst].off;
-        const TI* src = final_buf[tl.inst] ? B : A;
+        const long long mine = descs[tl.inst].off + tl.start, theirs = descs[tl.inst].eoff + tl.start;
         for (int j = threadIdx.x; j < tl.count; j += blockDim.x) {
-            const long long g = off + tl.start + j;
-            out[g] = (TO)src[g];
+            if (kImport) out[mine + j] = in[theirs + j];
+            else out[theirs + j] = in[mine + j];
+        }
+    }
+}
+
+// Per-instance selection of the final ping-pong buffer into the caller's array and into A.
+__global__ void k_bselect(const InstDesc* __restrict__ descs, const BatchTile* __restrict__ tiles, int ntiles,
+                          const int* __restrict__ final_buf, float* __restrict__ A, const float* __restrict__ B,
+                          float* __restrict__ out) {
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const BatchTile tl = tiles[t];
+        const long long mine = descs[tl.inst].off + tl.start, theirs = descs[tl.inst].eoff + tl.start;
+        const bool second = final_buf[tl.inst] != 0;
+        for (int j = threadIdx.x; j < tl.count; j += blockDim.x) {
+            const float v = second ? B[mine + j] : A[mine + j];
+            if (second) A[mine + j] = v;
+            out[theirs + j] = v;
         }
     }
 }
@@ -1012,7 +995,8 @@ static void by_mh(int mh, F&& f) {
 // ------------------------------------------------------------------------ batch handle
 struct Batch {
     int n = 0;
-    long long total = 0;
+    long long total = 0;   // states, as in the caller's arrays
+    long long padded = 0;  // entries of the handle's concatenated arrays
     int mh = 8;
     int ts = 4096;    // states per tile (default: the fastest measured on the 512-instance batch)
     int bps = 8;      // blocks per SM of the persistent grid
@@ -1032,6 +1016,7 @@ struct Batch {
     unsigned int *res32 = nullptr, *vmax32 = nullptr;
     unsigned long long* res64 = nullptr;
     long long* iters = nullptr;
+    unsigned int* bar = nullptr;  // the resident loop's barrier counter and fault flag
     long long* max_d = nullptr;
     double* tol_d = nullptr;
     float* tol_scale = nullptr;  // per-instance factor of the correction loop's tolerance
@@ -1109,7 +1094,7 @@ static BatchCtl ctl_of(Batch* b, bool scaled = false) {
 
 static BatchKrylov kry_of(Batch* b) {
     BatchKrylov K;
-    const size_t T = (size_t)b->total;
+    const size_t T = (size_t)b->padded;
     K.rho = b->kr_rho;
     K.alpha = b->kr_alpha;
     K.omega = b->kr_omega;
@@ -1508,6 +1493,42 @@ static int reset_loop(Batch* b, double tol, long long max_sweeps, cudaStream_t s
     return VC_OK;
 }
 
+// The FP32 loop by vc_batch_loop.cu.  Its instances advance in step, one grid barrier after each
+// pass, so the small ones ride along (a few percent of the work) and the side streams of
+// the whole-instance path stay empty; a batch of small instances only, which needs no
+// barrier, keeps that path, and the in-block iteration keeps its graph.
+static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, cudaStream_t st, bool* resident) {
+    *resident = false;
+    if ((flags & VC_ITER_BLOCK) || b->n_small == b->n) return VC_OK;
+    int rc = reset_loop(b, tol, max_sweeps, st);
+    if (rc) return rc;
+    BatchLoopArgs a;
+    a.descs = b->d_desc;
+    a.n = b->n;
+    a.c = ctl_of(b);
+    a.V0 = b->Va;
+    a.V1 = b->Vb;
+    a.U = b->U + kUShift;
+    a.U2 = b->U2;
+    a.arrivals = b->bar;
+    a.fault = (int*)b->bar + 1;
+    a.first = 0;
+    // sweeps of one launch: about a quarter of a second
+    a.budget = (int)std::min<long long>(1 << 20, std::max<long long>(16, (long long)(2e10 / (double)b->padded)));
+    for (;;) {
+        int h[2] = {0, 0};  // active instances, fault
+        VC_CUDA(cudaMemsetAsync(b->bar, 0, 8, st));
+        if ((rc = launch_batch_loop(a, b->mh, b->num_sms, (flags & VC_ITER_SELF_LOOP) != 0, st, resident))) return rc;
+        if (!*resident) return VC_OK;
+        VC_CUDA(cudaMemcpyAsync(&h[0], b->active, 4, cudaMemcpyDeviceToHost, st));
+        VC_CUDA(cudaMemcpyAsync(&h[1], a.fault, 4, cudaMemcpyDeviceToHost, st));
+        VC_CUDA(cudaStreamSynchronize(st));
+        if (h[1]) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
+        if (h[0] <= 0) return VC_OK;
+        a.first += a.budget;
+    }
+}
+
 template <int MH>
 static void enqueue_extract(Batch* b, const float* V, int32_t* pi, cudaStream_t st) {
     if (pairs_ok<MH>(b))
@@ -1567,13 +1588,16 @@ int vc_build_batch(const vc_params* p, int32_t n, void* stream, vc_batch** out) 
         d.md = tmp.md;
         d.c32 = tmp.c32;
         d.c64 = tmp.c64;
-        d.off = b->total;
+        d.off = b->padded;
+        d.eoff = b->total;
         d.S = tmp.S;
         b->h_desc.push_back(d);
         b->total += tmp.S;
+        b->padded += (tmp.S + 63LL) & ~63LL;
         maxH = std::max(maxH, tmp.md.H);
     }
     if (!rc && b->total >= (1LL << 31)) rc = fail(VC_ERR_ARG, "total states must be < 2^31");
+    if (!rc && b->padded >= (1LL << 31)) rc = fail(VC_ERR_ARG, "total states (each instance rounded up to 64) must be < 2^31");
     if (rc) {
         delete b;
         return rc;
@@ -1582,11 +1606,11 @@ int vc_build_batch(const vc_params* p, int32_t n, void* stream, vc_batch** out) 
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t T = (size_t)b->total, N = (size_t)n;
+    const size_t T = (size_t)b->padded, N = (size_t)n;
     void** f4[] = {(void**)&b->Va, (void**)&b->Vb, (void**)&b->U, (void**)&b->U2, (void**)&b->E0, (void**)&b->E1,
                    (void**)&b->Rr, (void**)&b->pi, (void**)&b->pi2};
     for (void** pp : f4)
-        if (!rc) rc = balloc(b, pp, 4 * T);
+        if (!rc) rc = balloc(b, pp, 4 * (T + kUPad));
     void** f8[] = {(void**)&b->V64, (void**)&b->V64b, (void**)&b->U64};
     for (void** pp : f8)
         if (!rc) rc = balloc(b, pp, 8 * T);
@@ -1600,6 +1624,7 @@ int vc_build_batch(const vc_params* p, int32_t n, void* stream, vc_batch** out) 
     if (!rc) rc = balloc(b, (void**)&b->active, 16);
     if (!rc) rc = balloc(b, (void**)&b->err, 16);
     if (!rc) rc = balloc(b, (void**)&b->iters, 16);
+    if (!rc) rc = balloc(b, (void**)&b->bar, 16);
     if (!rc) rc = balloc(b, (void**)&b->max_d, 16);
     if (!rc) rc = balloc(b, (void**)&b->tol_d, 16);
     if (!rc) rc = balloc(b, (void**)&b->tol_scale, 4 * N);
@@ -1666,7 +1691,7 @@ int vc_batch_offsets(const vc_batch* bh, int64_t* offsets) {
     set_error("");
     if (!bh || !offsets) return fail(VC_ERR_ARG, "NULL argument");
     const Batch* b = (const Batch*)bh;
-    for (int i = 0; i < b->n; i++) offsets[i] = b->h_desc[i].off;
+    for (int i = 0; i < b->n; i++) offsets[i] = b->h_desc[i].eoff;
     offsets[b->n] = b->total;
     return VC_OK;
 }
@@ -1686,27 +1711,30 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
         if (pe != cudaSuccess) return cuda_fail(pe, "an earlier CUDA call left an error pending");
     }
     if (!graphs_ready(b)) return fail(VC_ERR_CUDA, "the batch's loop graphs are not built (a schedule change failed)");
-    // ---- FP32 value iteration of every instance: one graph launch
-    VC_CUDA(cudaMemcpyAsync(b->Va, V, 4 * T, cudaMemcpyDeviceToDevice, st));
-    if ((rc = reset_loop(b, tol, max_sweeps, st, b->n_small))) return rc;
-    {
+    // ---- FP32 value iteration of every instance: the resident loop or one graph launch
+    count_launches(1);
+    k_bcopy<float, true><<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, V, b->Va);
+    VC_LAUNCHED("k_bcopy");
+    bool resident = false;
+    if ((rc = resident_loop(b, tol, max_sweeps, flags, st, &resident))) return rc;
+    long long vi_iters = 0, corr_iters = 0;
+    if (!resident) {
+        if ((rc = reset_loop(b, tol, max_sweeps, st, b->n_small))) return rc;
         const bool sl = (flags & (VC_ITER_SELF_LOOP | VC_ITER_BLOCK)) != 0;
         int rs = VC_OK;
         by_mh(b->mh, [&](auto m) { rs = launch_small<decltype(m)::value>(b, sl, st); });
         if (rs) return rs;
-    }
-    VC_CUDA(cudaGraphLaunch((flags & VC_ITER_BLOCK) ? b->x_vi_blk : (flags & VC_ITER_SELF_LOOP) ? b->x_vi_sl : b->x_vi,
-                            st));
-    {
+        VC_CUDA(cudaGraphLaunch((flags & VC_ITER_BLOCK)       ? b->x_vi_blk
+                                : (flags & VC_ITER_SELF_LOOP) ? b->x_vi_sl
+                                                              : b->x_vi,
+                                st));
         const cudaError_t ge = cudaGetLastError();
         if (ge != cudaSuccess) return cuda_fail(ge, "after the FP32 loop graph launch");
+        if ((rc = join_small(b, st))) return rc;
+        VC_CUDA(cudaMemcpyAsync(&vi_iters, b->iters, 8, cudaMemcpyDeviceToHost, st));
     }
-    if ((rc = join_small(b, st))) return rc;
-    long long vi_iters = 0, corr_iters = 0;
-    VC_CUDA(cudaMemcpyAsync(&vi_iters, b->iters, 8, cudaMemcpyDeviceToHost, st));
     count_launches(1);
-    k_bselect<float, float><<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, b->final_buf, b->Va,
-                                                          b->Vb, V);
+    k_bselect<<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, b->final_buf, b->Va, b->Vb, V);
     VC_LAUNCHED("k_bselect");
     std::vector<int> done(N), sweeps(N), csweeps(N, 0), cert(N, 0), rounds(N, 0);
     std::vector<double> r64(N, INFINITY);
@@ -1719,10 +1747,10 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
         // ---- refinement of every instance: argmax policy, FP64 residual, FP32 correction
         // by BiCGSTAB (one graph launch; fixed-point sweeps as the fallback), FP64 update,
         // FP64 Bellman certificate; repeat on failures.
-        by_mh(b->mh, [&](auto m) { enqueue_extract<decltype(m)::value>(b, V, b->pi, st); });
+        by_mh(b->mh, [&](auto m) { enqueue_extract<decltype(m)::value>(b, b->Va, b->pi, st); });
         VC_LAUNCHED("policy extraction");
         count_launches(3);
-        k_f32_to_f64_n<<<b->grid, kThreads, 0, st>>>(V, b->V64, (long long)T);
+        k_f32_to_f64_n<<<b->grid, kThreads, 0, st>>>(b->Va, b->V64, b->padded);
         VC_LAUNCHED("k_f32_to_f64_n");
         const long long eval_max = std::max<long long>(100000, max_sweeps);
         // Per-instance target of the FP64 residual: tol, or, in accuracy mode,
@@ -1769,12 +1797,12 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
                     cs[i] = 2 * ki[i];
                     solved = solved && kd[i] == 1;
                 }
-                if (solved && (rc = launch_axpy64(b->V64, b->E0, (int)T, st))) return rc;
+                if (solved && (rc = launch_axpy64(b->V64, b->E0, (int)b->padded, st))) return rc;
             }
             if (!solved) {
                 // fixed-point correction sweeps (VC_ITER_PLAIN_CORRECTION, or BiCGSTAB broke
                 // down for an instance): e <- r + gamma P_pi e from e = 0 for every instance
-                VC_CUDA(cudaMemsetAsync(b->E0, 0, 4 * T, st));
+                VC_CUDA(cudaMemsetAsync(b->E0, 0, 4 * (size_t)b->padded, st));
                 if ((rc = reset_loop(b, 0.5 * tol, eval_max, st))) return rc;
                 VC_CUDA(cudaGraphLaunch(b->x_corr, st));
                 VC_CUDA(cudaMemcpyAsync(&corr_iters, b->iters, 8, cudaMemcpyDeviceToHost, st));
@@ -1795,8 +1823,8 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
             VC_LAUNCHED("FP64 certificate");
             std::vector<unsigned long long> rb(N);
             VC_CUDA(cudaMemcpyAsync(rb.data(), b->res64, 8 * N, cudaMemcpyDeviceToHost, st));
-            VC_CUDA(cudaMemcpyAsync(b->V64, b->V64b, 8 * T, cudaMemcpyDeviceToDevice, st));
-            VC_CUDA(cudaMemcpyAsync(b->pi, b->pi2, 4 * T, cudaMemcpyDeviceToDevice, st));
+            VC_CUDA(cudaMemcpyAsync(b->V64, b->V64b, 8 * (size_t)b->padded, cudaMemcpyDeviceToDevice, st));
+            VC_CUDA(cudaMemcpyAsync(b->pi, b->pi2, 4 * (size_t)b->padded, cudaMemcpyDeviceToDevice, st));
             VC_CUDA(cudaStreamSynchronize(st));
             if (herr) return fail(VC_ERR_CUDA, "internal: batched refinement policy infeasible");
             all_cert = true;
@@ -1815,10 +1843,21 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
             VC_CUDA(cudaMemcpyAsync(b->certified, skip_h.data(), 4 * N, cudaMemcpyHostToDevice, st));
             skipped = b->certified;
         }
-        if (V64_out) VC_CUDA(cudaMemcpyAsync(V64_out, b->V64, 8 * T, cudaMemcpyDeviceToDevice, st));
-        if (pi_out) VC_CUDA(cudaMemcpyAsync(pi_out, b->pi, 4 * T, cudaMemcpyDeviceToDevice, st));
+        if (V64_out) {
+            count_launches(1);
+            k_bcopy<double, false><<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, b->V64, V64_out);
+        }
+        if (pi_out) {
+            count_launches(1);
+            k_bcopy<int32_t, false><<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, b->pi, pi_out);
+        }
+        VC_LAUNCHED("result copies");
     } else {
-        if (pi_out) by_mh(b->mh, [&](auto m) { enqueue_extract<decltype(m)::value>(b, V, pi_out, st); });
+        if (pi_out) {
+            by_mh(b->mh, [&](auto m) { enqueue_extract<decltype(m)::value>(b, b->Va, b->pi, st); });
+            count_launches(1);
+            k_bcopy<int32_t, false><<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, b->pi, pi_out);
+        }
         VC_LAUNCHED("policy extraction (FP32 only)");
         if (V64_out) {
             count_launches(1);
@@ -1935,7 +1974,7 @@ int vc_batch_autotune(vc_batch* bh, int sweeps, double* best_ms, void* stream) {
             if ((rc = build_graphs(b))) return rc;
             float ms_best = 1e30f;
             for (int rep = 0; rep < 2; rep++) {
-                VC_CUDA(cudaMemsetAsync(b->Va, 0, 4 * (size_t)b->total, st));
+                VC_CUDA(cudaMemsetAsync(b->Va, 0, 4 * (size_t)b->padded, st));
                 if ((rc = reset_loop(b, 1e-30, sweeps, st))) return rc;
                 VC_CUDA(cudaEventRecord(e0, st));
                 count_launches((sweeps + 1) / 2 * kViBodyKernels);

@@ -1,0 +1,61 @@
+// vc_batch.cuh -- device-side descriptors of the batched solves, shared by the tile kernels
+// (vc_batch.cu) and the resident loop (vc_batch_loop.cu).
+#pragma once
+
+#include "vc_internal.cuh"
+
+namespace vc {
+
+struct InstDesc {
+    Model md;
+    Coef<float> c32;
+    Coef<double> c64;
+    long long off;   // first state in the handle's concatenated arrays (a multiple of 64)
+    long long eoff;  // first state in the caller's packed arrays
+    int S;
+    int blk_h;      // inner hosts of the in-block iteration's blocks (2(Q+1)(C+1)^blk_h states)
+};
+
+struct BatchTile {
+    int inst;
+    int start;  // first state, relative to the instance
+    int count;
+    int pad_;
+};
+
+// Device-side control of the batched loops (SoA over instances).
+struct BatchCtl {
+    int* done;                 // 0 running, 1 converged, 2 max sweeps, 3 FP32 stall
+    int* sweeps;
+    int* ticket;
+    const int* tiles_of;       // tiles per instance (constant)
+    int* final_buf;            // buffer of the last iterate (0: A, 1: B)
+    int* since_best;
+    float* best_res;
+    unsigned int* res32;       // [2n] ring of two slots
+    unsigned int* vmax32;      // [2n]
+    unsigned long long* res64; // [n] FP64 residual of a certificate / residual pass
+    int* active;               // instances still running
+    long long* iters;          // sweeps launched by the graph loop
+    const long long* max_sweeps; // loop parameters in device memory, so one captured graph
+    const double* tol;           // serves every call
+    const float* tol_scale;      // per-instance factor on tol (nullptr: 1)
+};
+
+// The FP32 loop of every active instance in one resident kernel (vc_batch_loop.cu): up to a
+// bounded number of sweeps from sweep *first on.  *launched = false when it does not serve
+// the batch (hosts, instances) or the device cannot hold the grid.
+struct BatchLoopArgs {
+    const InstDesc* descs;
+    int n;
+    BatchCtl c;
+    float *V0, *V1, *U, *U2;  // U: kUShift past a 16-byte-aligned buffer
+    unsigned int* arrivals;   // grid barrier, cleared by the host before each launch
+    int* fault;               // set by a block whose barrier wait gave up
+    long long first;          // sweeps done so far
+    int budget;
+};
+int launch_batch_loop(const BatchLoopArgs& a, int max_hosts, int num_sms, bool self_loop, cudaStream_t st,
+                      bool* launched);
+
+}  // namespace vc

@@ -12,7 +12,7 @@
 //
 // Bound: L2 latency and issue of the two passes (per 4 states: 16 loads of 16 bytes and ~250
 // instructions), then two barriers of ~1.5 us.  Measured per sweep, launched kernels
-// against this loop: 45 -> 28 us at 2.5 M states (H = 7), 18.3 -> 8.4 us at 343,750 states
+// against this loop: 45 -> 19 us at 2.5 M states (H = 7), 18.3 -> 8.0 us at 343,750 states
 // with the self-transition solve (VW = 2), whole solves of 640 states 2.89 -> 0.76 ms.
 #include <algorithm>
 #include <type_traits>
@@ -23,7 +23,10 @@
 
 namespace vc {
 
-constexpr int kLoopThreads = 512;
+// 640 threads leave 96 registers each, enough for items of four states of up to 7 hosts without
+// spills (768 and 1,024 spill): solve of 2.5 M states 7.9 ms with 512, 7.6 with 576, 6.75 with
+// 640, 8.9 with 768; gradient step of 343,750 states 8.8 -> 8.4 ms.
+constexpr int kLoopThreads = 640;
 // States up to which one CTA sweeps the instance alone: 8,192 states are ~5 us of issue on one
 // SM, what a sweep of the multi-CTA loop takes at any size (two barriers and two cold L2
 // round trips); four arrays of 8,192 floats also fit beside the L1's needs.

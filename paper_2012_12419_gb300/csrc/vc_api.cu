@@ -506,18 +506,15 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     memset(&gs, 0, sizeof(gs));
 
     // temporaries, stream-ordered; freed on every exit path
-    int32_t* cnt = nullptr;
+    AdjRows t;
     int32_t* fillpos = nullptr;
-    int64_t* rowT = nullptr;
-    int32_t* colT = nullptr;
-    float* valT = nullptr;
-    double* valT64 = nullptr;
+    int32_t* width = nullptr;
     float* rhoF = nullptr;
     double* partial = nullptr;
     double* out = nullptr;
-    int* err = nullptr;
+    int* err = nullptr;  // error flags, then the transpose's entries (8 bytes on)
     auto release = [&]() {
-        void* ps[] = {cnt, fillpos, rowT, colT, valT, valT64, rhoF, partial, out, err};
+        void* ps[] = {t.cnt, fillpos, width, t.base, t.col, t.val, t.val64, rhoF, partial, out, err};
         for (void* p : ps)
             if (p) cudaFreeAsync(p, st);
     };
@@ -532,42 +529,42 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
         if (e_ != cudaSuccess) return bail(cuda_fail(e_, #call)); \
     } while (0)
 
-    // ---- P_pi^T: in-degree count, exclusive scan, fill, per-row sort by source
-    VC_TRY(cudaMallocAsync((void**)&cnt, 4 * (size_t)S, st));
+    // ---- P_pi^T in slices of 32 rows: in-degree count, slice sizes, exclusive scan, fill,
+    // per-row sort by source
+    const int64_t slices = ((int64_t)S + 31) / 32;
+    VC_TRY(cudaMallocAsync((void**)&t.cnt, 4 * (size_t)S, st));
     VC_TRY(cudaMallocAsync((void**)&fillpos, 4 * (size_t)S, st));
-    VC_TRY(cudaMallocAsync((void**)&rowT, 8 * ((size_t)S + 3), st));
+    VC_TRY(cudaMallocAsync((void**)&width, 4 * (size_t)slices, st));
+    VC_TRY(cudaMallocAsync((void**)&t.base, 8 * ((size_t)slices + 3), st));
     VC_TRY(cudaMallocAsync((void**)&err, 16, st));
-    VC_TRY(cudaMemsetAsync(cnt, 0, 4 * (size_t)S, st));
+    VC_TRY(cudaMemsetAsync(t.cnt, 0, 4 * (size_t)S, st));
     VC_TRY(cudaMemsetAsync(fillpos, 0, 4 * (size_t)S, st));
     VC_TRY(cudaMemsetAsync(err, 0, 16, st));
-    int rc = launch_adj_count(m, pi, cnt, err, st);
+    int rc = launch_adj_count(m, pi, t.cnt, err, st);
     if (rc) return bail(rc);
-    if ((rc = exclusive_scan(m, cnt, S, rowT, st))) return bail(rc);
-    int herr = 0;
-    int64_t nnzT = 0;
-    VC_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VC_TRY(cudaMemcpyAsync(&nnzT, rowT + S, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    if ((rc = launch_adj_width(m, t.cnt, width, (unsigned long long*)(err + 2), st))) return bail(rc);
+    if ((rc = exclusive_scan(m, width, slices, t.base, st))) return bail(rc);
+    int64_t herr[2] = {0, 0};
+    int64_t stored = 0;
+    VC_TRY(cudaMemcpyAsync(herr, err, 16, cudaMemcpyDeviceToHost, st));
+    VC_TRY(cudaMemcpyAsync(&stored, t.base + slices, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     VC_TRY(cudaStreamSynchronize(st));
-    if (herr) return bail(fail(VC_ERR_ARG, "the policy picks an infeasible action"));
-    gs.nnz_transpose = nnzT;
-    VC_TRY(cudaMallocAsync((void**)&colT, 4 * ((size_t)nnzT + 16), st));
-    VC_TRY(cudaMallocAsync((void**)&valT, 4 * ((size_t)nnzT + 16), st));
-    VC_TRY(cudaMallocAsync((void**)&valT64, 8 * ((size_t)nnzT + 16), st));
-    if ((rc = launch_adj_fill(m, pi, rowT, fillpos, colT, valT, valT64, st))) return bail(rc);
+    if ((int)herr[0]) return bail(fail(VC_ERR_ARG, "the policy picks an infeasible action"));
+    gs.nnz_transpose = herr[1];
+    VC_TRY(cudaMallocAsync((void**)&t.col, 4 * ((size_t)stored + 16), st));
+    VC_TRY(cudaMallocAsync((void**)&t.val, 4 * ((size_t)stored + 16), st));
+    VC_TRY(cudaMallocAsync((void**)&t.val64, 8 * ((size_t)stored + 16), st));
+    if ((rc = launch_adj_fill(m, pi, t, fillpos, st))) return bail(rc);
 
-    // ---- lam: the transposed system as a one-action stored MDP (reward rho, matrix P^T)
+    // ---- lam: the transposed system (right-hand side rho, matrix P^T) as a view for the solver
     VC_TRY(cudaMallocAsync((void**)&rhoF, 4 * ((size_t)S + 8), st));
     if ((rc = launch_f64_to_f32(rho, rhoF, S, st))) return bail(rc);
     Mdp T;
-    T.fmt = VC_CSR_F32 | VC_DIRECT;
     T.has_model = false;
     T.S = S;
     T.A = 1;
     T.gamma = m->gamma;
-    T.row_ptr = rowT;
-    T.col = colT;
-    T.val = valT;
-    T.R = rhoF;
+    T.adj = &t;
     T.ctl = m->ctl;
     T.ctl_host = m->ctl_host;
     T.num_sms = m->num_sms;
@@ -575,9 +572,8 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     T.kr_part = m->kr_part;
     T.kctl = m->kctl;
     T.kctl_host = m->kctl_host;
-    auto sweep_T = [&](const float* in, float* o, SweepCtl sc) { return csr_sweep32(&T, in, o, nullptr, nullptr, sc, st); };
     // (I - gamma P_pi^T) x = b in FP32: BiCGSTAB, or fixed-point sweeps x <- b + gamma P^T x
-    // from x = 0 (T.R = b) when it breaks down; *xo receives the buffer holding x
+    // from x = 0 when it breaks down; *xo receives the buffer holding x
     auto solve_T = [&](float* b, double target, float** xo, long long* prods) -> int {
         bool conv = false;
         int r = krylov_correct(&T, nullptr, b, m->E0, target, std::min<long long>(kKrylovMaxIter, max_sweeps), st,
@@ -586,10 +582,12 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
             *xo = m->E0;
             return r;
         }
-        T.R = b;
         VC_CUDA(cudaMemsetAsync(m->E0, 0, 4 * (size_t)S, st));
         int fin = 0;
-        if ((r = loop32(m, m->E0, m->E1, target, max_sweeps, st, &fin, sweep_T))) return r;
+        r = loop32(m, m->E0, m->E1, target, max_sweeps, st, &fin, [&](const float* in, float* o, SweepCtl sc) {
+            return launch_adj_sweep(m, t, b, in, o, sc, st);
+        });
+        if (r) return r;
         *prods += m->ctl_host->sweeps;
         *xo = fin == 1 ? m->E1 : m->E0;
         return VC_OK;
@@ -606,7 +604,7 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     for (int round = 0; round < 20; round++) {
         VC_TRY(cudaMemsetAsync(&m->ctl->changes, 0, 2 * sizeof(unsigned long long), st));
         SweepCtl sc{m->ctl, kModeCert64, 0, nullptr};
-        if ((rc = launch_adj_resid64(m, rowT, colT, valT64, rho, lam, m->Rres, sc, st))) return bail(rc);
+        if ((rc = launch_adj_resid64(m, t, rho, lam, m->Rres, sc, st))) return bail(rc);
         VC_TRY(cudaMemcpyAsync(m->ctl_host, m->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         VC_TRY(cudaStreamSynchronize(st));
         double r64;
@@ -626,8 +624,7 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     }
 
     // ---- contraction over states, reduced in a fixed order
-    const int g = state_grid(m);
-    VC_TRY(cudaMallocAsync((void**)&partial, 8 * (size_t)g * grad_partial_stride(m), st));
+    VC_TRY(cudaMallocAsync((void**)&partial, grad_partial_bytes(m), st));
     VC_TRY(cudaMallocAsync((void**)&out, 8 * ((size_t)nt + 1), st));
     if ((rc = launch_grad_contract(m, pi, V, lam, rho, partial, out, st))) return bail(rc);
     VC_TRY(cudaMemcpyAsync(dJ_dtheta, out, 8 * (size_t)nt, cudaMemcpyDeviceToDevice, st));

@@ -4,14 +4,21 @@
 // For a fixed policy pi, V = R_pi + gamma P_pi V, so
 //     dJ/dtheta_i = lam . (dR_pi/dtheta_i + gamma (dP_pi/dtheta_i) V),
 //     (I - gamma P_pi)^T lam = rho.
-// lam is found by pull sweeps over an explicit transpose P_pi^T (rows = targets, entries
-// sorted by source so every sweep sums in one fixed order), FP32 sweeps refined in FP64
-// like the forward solve.  The contraction regenerates every event of each state's
+// lam is found from an explicit transpose P_pi^T (rows = targets, entries sorted by source so
+// every product sums in one fixed order), FP32 solves refined in FP64 like the forward
+// solve.  The transpose is stored in slices of 32 rows, entry j of row y at
+// base[y / 32] + 32 j + y % 32, so the lanes of a warp (a row each) read and write
+// consecutive entries; row after row their accesses were a row length apart (gradient step of
+// 343,750 states: fill and sort 0.59 -> 0.25 ms, the two adjoint solves 3.2 -> 1.9 ms).
+// The contraction regenerates every event of each state's
 // post-decision state and differentiates its probability rate/Lam analytically:
 // d(rate/Lam) = drate/Lam - rate dLam/Lam^2, the self-loop taking minus the others, so
-// sum_s' dP V = sum_e dp_e (V(y_e) - V(x)).  Partial sums reduce per block and then in
-// block order, so the result is reproducible bit for bit.
+// sum_s' dP V = sum_e dp_e (V(y_e) - V(x)).  Partial sums reduce per block and then in a fixed
+// order, so the result is reproducible bit for bit.
+#include <cooperative_groups.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "vc_internal.cuh"
 
@@ -31,7 +38,21 @@ __global__ void k_adj_count(Model md, Rates rt, const int32_t* __restrict__ pi, 
     }
 }
 
-__global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, const int64_t* __restrict__ rowT,
+// Entries of every slice of 32 rows (32 x its longest row), and the entries of all rows.
+__global__ void __launch_bounds__(kThreads) k_adj_width(int S, const int32_t* __restrict__ cnt, int32_t* __restrict__ width,
+                                                        unsigned long long* total) {
+    const int lane = threadIdx.x & 31, slices = (S + 31) / 32;
+    unsigned long long sum = 0;
+    for (int g = (blockIdx.x * kThreads + threadIdx.x) >> 5; g < slices; g += (gridDim.x * kThreads) >> 5) {
+        const int n = 32 * g + lane < S ? cnt[32 * g + lane] : 0;
+        const int w = __reduce_max_sync(0xffffffffu, n);
+        sum += (unsigned long long)__reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) width[g] = 32 * w;
+    }
+    if (lane == 0 && sum) atomicAdd(total, sum);
+}
+
+__global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, const int64_t* __restrict__ base,
                            int32_t* __restrict__ fillpos, int32_t* __restrict__ colT, float* __restrict__ valT,
                            double* __restrict__ valT64) {
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < md.S; s += gridDim.x * blockDim.x) {
@@ -40,7 +61,7 @@ __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, c
         const int n = model_row(md, rt, s, pi[s], cols, probs, &R);
         for (int j = 0; j < n; j++) {
             const int y = cols[j];
-            const int64_t slot = rowT[y] + atomicAdd(&fillpos[y], 1);
+            const int64_t slot = base[y >> 5] + 32LL * atomicAdd(&fillpos[y], 1) + (y & 31);
             colT[slot] = s;
             valT[slot] = (float)probs[j];
             valT64[slot] = probs[j];
@@ -48,32 +69,60 @@ __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, c
     }
 }
 
-// Orders each transposed row by source state (insertion sort; in-degrees are small).
-__global__ void k_adj_sort(int S, const int64_t* __restrict__ rowT, int32_t* __restrict__ colT,
-                           float* __restrict__ valT, double* __restrict__ valT64) {
+// Orders each transposed row by source state (insertion sort; in-degrees are small, and the
+// fill's order is nearly that of the sources).
+__global__ void k_adj_sort(int S, const int64_t* __restrict__ base, const int32_t* __restrict__ cnt,
+                           int32_t* __restrict__ colT, float* __restrict__ valT, double* __restrict__ valT64) {
     for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < S; y += gridDim.x * blockDim.x) {
-        const int64_t lo = rowT[y], hi = rowT[y + 1];
-        for (int64_t i = lo + 1; i < hi; i++) {
-            const int c = colT[i];
-            const float v = valT[i];
-            const double v64 = valT64[i];
-            int64_t j = i - 1;
-            while (j >= lo && colT[j] > c) {
-                colT[j + 1] = colT[j];
-                valT[j + 1] = valT[j];
-                valT64[j + 1] = valT64[j];
+        const int64_t lo = base[y >> 5] + (y & 31);
+        const int n = cnt[y];
+        for (int i = 1; i < n; i++) {
+            const int c = colT[lo + 32LL * i];
+            if (colT[lo + 32LL * (i - 1)] < c) continue;
+            const float v = valT[lo + 32LL * i];
+            const double v64 = valT64[lo + 32LL * i];
+            int j = i - 1;
+            while (j >= 0 && colT[lo + 32LL * j] > c) {
+                colT[lo + 32LL * (j + 1)] = colT[lo + 32LL * j];
+                valT[lo + 32LL * (j + 1)] = valT[lo + 32LL * j];
+                valT64[lo + 32LL * (j + 1)] = valT64[lo + 32LL * j];
                 j--;
             }
-            colT[j + 1] = c;
-            valT[j + 1] = v;
-            valT64[j + 1] = v64;
+            colT[lo + 32LL * (j + 1)] = c;
+            valT[lo + 32LL * (j + 1)] = v;
+            valT64[lo + 32LL * (j + 1)] = v64;
         }
     }
 }
 
+// Fixed-point sweep of the adjoint system, x' = b + gamma P^T x (the fallback solve).
+__global__ void __launch_bounds__(kThreads) k_adj_sweep(int S, float gamma, const int64_t* __restrict__ base,
+                                                        const int32_t* __restrict__ cnt,
+                                                        const int32_t* __restrict__ colT,
+                                                        const float* __restrict__ valT, const float* __restrict__ b,
+                                                        const float* __restrict__ x, float* __restrict__ x_out,
+                                                        SweepCtl sc) {
+    if (loop_done(sc)) return;
+    const long long sweep = loop_sweep(sc);
+    float res = 0.0f, vabs = 0.0f;
+    for (int y = blockIdx.x * kThreads + threadIdx.x; y < S; y += gridDim.x * kThreads) {
+        const int64_t lo = base[y >> 5] + (y & 31);
+        float acc = 0.0f;
+        for (int j = 0; j < cnt[y]; j++) acc = fmaf(valT[lo + 32LL * j], x[colT[lo + 32LL * j]], acc);
+        const float v = b[y] + gamma * acc;
+        x_out[y] = v;
+        res = fmaxf(res, fabsf(v - x[y]));
+        vabs = fmaxf(vabs, fabsf(v));
+    }
+    res = block_max<float, kThreads>(res);
+    vabs = block_max<float, kThreads>(vabs);
+    finish_block<float>(sc, res, vabs, sweep);
+}
+
 // FP64 residual of the adjoint system r = rho + gamma P^T lam - lam (stored as float);
 // max |r| into the control block's certificate slot.
-__global__ void __launch_bounds__(kThreads) k_adj_resid64(int S, double gamma, const int64_t* __restrict__ rowT,
+__global__ void __launch_bounds__(kThreads) k_adj_resid64(int S, double gamma, const int64_t* __restrict__ base,
+                                                          const int32_t* __restrict__ cnt,
                                                           const int32_t* __restrict__ colT,
                                                           const double* __restrict__ valT64,
                                                           const double* __restrict__ rho,
@@ -82,7 +131,8 @@ __global__ void __launch_bounds__(kThreads) k_adj_resid64(int S, double gamma, c
     double res = 0.0;
     for (int y = blockIdx.x * kThreads + threadIdx.x; y < S; y += gridDim.x * kThreads) {
         double acc = 0.0;
-        for (int64_t j = rowT[y]; j < rowT[y + 1]; j++) acc += valT64[j] * lam[colT[j]];
+        const int64_t lo = base[y >> 5] + (y & 31);
+        for (int j = 0; j < cnt[y]; j++) acc += valT64[lo + 32LL * j] * lam[colT[lo + 32LL * j]];
         const double v = rho[y] + gamma * acc - lam[y];
         r[y] = (float)v;
         res = fmax(res, fabs(v));
@@ -96,67 +146,66 @@ __global__ void k_f64_to_f32(const double* __restrict__ in, float* __restrict__ 
 }
 
 // ------------------------------------------------------------------ contraction
-// Per state s with x = x_pi(s): lam(s) * (dR(x)/dtheta + gamma sum_e dp_e (V(y_e) - V(x))),
-// and rho(s) V(s) for J, in slots 0..2H+4 and 2*MH+5 of a per-block partial row.
+// Per state s with x = x_pi(s): lam(s) * (dR(x)/dtheta + gamma sum_e dp_e (V(y_e) - V(x))).
+// Every derivative is linear in a few sums over the states (w = lam(s), dV the value change of
+// an event), so the states only add those, in slots of a per-block partial row, and the
+// derivatives are formed from the totals: an FP64 multiply-add or two per sum and state in
+// place of ~40 FP64 divisions (FP64 issues two lanes a cycle and SM here).  Together with the
+// final sums below: 0.46 -> 0.06 ms at 343,750 states.
+enum GradSlot : int {
+    kSumJ = 0,   // rho V
+    kSumFull,    // w [q = Q]
+    kSumA,       // w dV(arrival)
+    kSumF0,      // w dV(flip), phase 0
+    kSumF1,      // w dV(flip), phase 1
+    kSumQ,       // w q
+    kSumHost     // MH each: w o_k, w o_k dV(completion on k), w dV(departure of k)
+};
+constexpr int grad_slots(int MH) { return kSumHost + 3 * MH; }
+
 template <int MH>
-__global__ void __launch_bounds__(kThreads) k_grad_contract(Model md, Rates rt, double gamma,
-                                                            const int32_t* __restrict__ pi,
+__global__ void __launch_bounds__(kThreads) k_grad_contract(Model md, const int32_t* __restrict__ pi,
                                                             const double* __restrict__ V,
                                                             const double* __restrict__ lam,
                                                             const double* __restrict__ rho,
                                                             double* __restrict__ partial) {
-    constexpr int NT = 2 * MH + 6;  // theta slots (2H+5 used) + J
+    constexpr int NT = grad_slots(MH);
     double g[NT];
 #pragma unroll
     for (int i = 0; i < NT; i++) g[i] = 0.0;
     const int H = md.H;
-    const double Lam = rt.Lam, Lam2 = rt.Lam * rt.Lam;
     for (int s = blockIdx.x * kThreads + threadIdx.x; s < md.S; s += gridDim.x * kThreads) {
         Digits d;
         decode<MH>(md, s, d);
         int x = s;
         if (!apply_action<MH>(md, s, pi[s], d, x)) continue;  // rejected by the count kernel
-        const double vx = V[x];
-        double dVc[MH], dVd[MH];
-        double D = 0.0, L = 0.0;
-        int occ_sum = 0;
-#pragma unroll
-        for (int k = 0; k < MH; k++) {
-            dVc[k] = 0.0;
-            dVd[k] = 0.0;
-            if (k < H) {
-                const int o = d.occ[k];
-                if (o > 0) {
-                    dVc[k] = V[x - md.stride[k]] - vx;
-                    dVd[k] = V[x - o * md.stride[k]] - vx;
-                }
-                D += rt.mu[k] * o * dVc[k] + rt.delta[k] * dVd[k];
-                L += rt.delta[k] * o;
-                occ_sum += o;
-            }
-        }
+        const double vx = V[x], w = lam[s];
         const bool full = d.q >= md.Q;
-        const double dVa = full ? 0.0 : V[x + 2] - vx;
-        D += rt.lambda * dVa;
-        if (full) L += rt.lambda;
-        const double dVf = V[d.ph ? x - 1 : x + 1] - vx;
-        D += (d.ph ? 1.0 - rt.f : rt.f) * dVf;
-        const double w = lam[s];
-        // lambda
-        g[0] += w * (rt.w_loss * ((full ? 1.0 : 0.0) / Lam - L / Lam2) + gamma * (dVa / Lam - D / Lam2));
+        // every gather first
+        double v1[MH], v0[MH];
+#pragma unroll
+        for (int k = 0; k < MH; k++) {
+            const bool on = k < H && d.occ[k] > 0;
+            v1[k] = on ? V[x - md.stride[k]] : vx;
+            v0[k] = on ? V[x - d.occ[k] * md.stride[k]] : vx;
+        }
+        const double va = full ? vx : V[x + 2];
+        const double vf = V[d.ph ? x - 1 : x + 1];
+        g[kSumJ] = fma(rho[s], V[s], g[kSumJ]);
+        if (full) g[kSumFull] += w;
+        g[kSumA] = fma(w, va - vx, g[kSumA]);
+        if (d.ph) g[kSumF1] = fma(w, vf - vx, g[kSumF1]);
+        else g[kSumF0] = fma(w, vf - vx, g[kSumF0]);
+        g[kSumQ] = fma(w, (double)d.q, g[kSumQ]);
 #pragma unroll
         for (int k = 0; k < MH; k++) {
             if (k < H) {
-                const int o = d.occ[k];
-                g[1 + k] += w * (-rt.w_loss * L * md.C / Lam2 + gamma * (o * dVc[k] / Lam - md.C * D / Lam2));
-                g[1 + MH + k] += w * (rt.w_loss * (o / Lam - L / Lam2) + gamma * (dVd[k] / Lam - D / Lam2));
+                const double wo = w * d.occ[k];
+                g[kSumHost + k] += wo;
+                g[kSumHost + MH + k] = fma(wo, v1[k] - vx, g[kSumHost + MH + k]);
+                g[kSumHost + 2 * MH + k] = fma(w, v0[k] - vx, g[kSumHost + 2 * MH + k]);
             }
         }
-        g[1 + 2 * MH] += w * gamma * (d.ph ? -dVf : dVf) / Lam;  // f
-        g[2 + 2 * MH] += w * occ_sum;                            // w_occ
-        g[3 + 2 * MH] += w * L / Lam;                            // w_loss
-        g[4 + 2 * MH] += w * d.q;                                // w_q
-        g[5 + 2 * MH] += rho[s] * V[s];                          // J
     }
     // block reduction, fixed order: warp shuffles, then warps in index order
     __shared__ double part[kThreads / 32][NT];
@@ -175,42 +224,81 @@ __global__ void __launch_bounds__(kThreads) k_grad_contract(Model md, Rates rt, 
     }
 }
 
-// Sums the per-block rows in block order and maps the MH-strided slots to the packed
-// theta order (lambda, mu_0..mu_{H-1}, delta_0..delta_{H-1}, f, w_occ, w_loss, w_q), J.
-__global__ void k_grad_final(const double* __restrict__ partial, int nblocks, int MH, int H, double* __restrict__ out) {
-    const int NT = 2 * MH + 6;
+// Adds the per-block rows (a warp per slot, its lanes' strided sums in a fixed tree) and
+// forms the packed derivatives (lambda, mu_0..mu_{H-1}, delta_0..delta_{H-1}, f, w_occ, w_loss,
+// w_q) and J from the totals.
+__global__ void __launch_bounds__(kThreads) k_grad_final(const double* __restrict__ partial, int nblocks, int MH, int C,
+                                                         int H, Rates rt, double gamma, double* __restrict__ out) {
+    __shared__ double t[grad_slots(kMaxH)];
+    const int NT = grad_slots(MH), lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < NT; i += kThreads / 32) {
+        double v = 0.0;
+        for (int b = lane; b < nblocks; b += 32) v += partial[(size_t)b * NT + i];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) t[i] = v;
+    }
+    __syncthreads();
     const int i = threadIdx.x;
     if (i >= 2 * H + 6) return;
-    int src;
-    if (i == 0)
-        src = 0;
-    else if (i <= H)
-        src = i;  // mu_{i-1}
-    else if (i <= 2 * H)
-        src = 1 + MH + (i - 1 - H);  // delta
-    else
-        src = 1 + 2 * MH + (i - 1 - 2 * H);  // f, w_occ, w_loss, w_q, J
-    double v = 0.0;
-    for (int b = 0; b < nblocks; b++) v += partial[(size_t)b * NT + src];
+    const double Lam = rt.Lam, Lam2 = rt.Lam * rt.Lam;
+    // w (tasks lost per unit of time) and w (sum of rate x value change)
+    double L = rt.lambda * t[kSumFull], occ = 0.0;
+    double D = rt.lambda * t[kSumA] + rt.f * t[kSumF0] + (1.0 - rt.f) * t[kSumF1];
+    for (int k = 0; k < H; k++) {
+        occ += t[kSumHost + k];
+        L += rt.delta[k] * t[kSumHost + k];
+        D += rt.mu[k] * t[kSumHost + MH + k] + rt.delta[k] * t[kSumHost + 2 * MH + k];
+    }
+    double v;
+    if (i == 0) {
+        v = rt.w_loss * (t[kSumFull] / Lam - L / Lam2) + gamma * (t[kSumA] / Lam - D / Lam2);
+    } else if (i <= H) {
+        const int k = i - 1;
+        v = -rt.w_loss * L * C / Lam2 + gamma * (t[kSumHost + MH + k] / Lam - C * D / Lam2);
+    } else if (i <= 2 * H) {
+        const int k = i - 1 - H;
+        v = rt.w_loss * (t[kSumHost + k] / Lam - L / Lam2) + gamma * (t[kSumHost + 2 * MH + k] / Lam - D / Lam2);
+    } else if (i == 2 * H + 1) {
+        v = gamma * (t[kSumF0] - t[kSumF1]) / Lam;
+    } else if (i == 2 * H + 2) {
+        v = occ;
+    } else if (i == 2 * H + 3) {
+        v = L / Lam;
+    } else if (i == 2 * H + 4) {
+        v = t[kSumQ];
+    } else {
+        v = t[kSumJ];
+    }
     out[i] = v;
 }
 
-
-// J = rho . V in FP64 by one block: each thread sums its strided states in index order,
-// then the block halves the partials in a fixed tree, so the result is reproducible bit
-// for bit (one block suffices: the objective is read once per solve).
-__global__ void __launch_bounds__(1024) k_objective(const double* __restrict__ V, const double* __restrict__ rho,
-                                                   long long S, double* __restrict__ J) {
-    __shared__ double part[1024];
+// J = rho . V in FP64 by one cluster: each thread sums its strided states in index order, each
+// block halves the partials in a fixed tree and the first block adds the blocks' in order, so the
+// result is reproducible bit for bit and needs no scratch memory.  Bound by the FP64 adds and
+// the latency of a thread's chain of loads; one block took 89 us at 343,750 states.
+constexpr int kObjBlocks = 8, kObjThreads = 1024;
+__global__ void __cluster_dims__(kObjBlocks, 1, 1) __launch_bounds__(kObjThreads)
+    k_objective(const double* __restrict__ V, const double* __restrict__ rho, long long S, double* __restrict__ J) {
+    namespace cg = cooperative_groups;
+    __shared__ double part[kObjThreads];
     double acc = 0.0;
-    for (long long s = threadIdx.x; s < S; s += 1024) acc = fma(rho[s], V[s], acc);
+#pragma unroll 4
+    for (long long s = (long long)blockIdx.x * kObjThreads + threadIdx.x; s < S; s += kObjBlocks * kObjThreads)
+        acc = fma(rho[s], V[s], acc);
     part[threadIdx.x] = acc;
     __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
+    for (int w = kObjThreads / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *J = part[0];
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double v = 0.0;
+        for (int b = 0; b < kObjBlocks; b++) v += *cl.map_shared_rank(&part[0], b);
+        *J = v;
+    }
+    cl.sync();
 }
 
 // ------------------------------------------------------------------------ launchers
@@ -221,19 +309,33 @@ int launch_adj_count(Mdp* m, const int32_t* pi, int32_t* cnt, int* err, cudaStre
     return VC_OK;
 }
 
-int launch_adj_fill(Mdp* m, const int32_t* pi, const int64_t* rowT, int32_t* fillpos, int32_t* colT, float* valT,
-                    double* valT64, cudaStream_t st) {
-    count_launches(2);
-    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, rowT, fillpos, colT, valT, valT64);
-    k_adj_sort<<<state_grid(m), kThreads, 0, st>>>(m->S, rowT, colT, valT, valT64);
+int launch_adj_width(Mdp* m, const int32_t* cnt, int32_t* width, unsigned long long* total, cudaStream_t st) {
+    count_launches(1);
+    k_adj_width<<<state_grid(m), kThreads, 0, st>>>(m->S, cnt, width, total);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }
 
-int launch_adj_resid64(Mdp* m, const int64_t* rowT, const int32_t* colT, const double* valT64, const double* rho,
-                       const double* lam, float* r, SweepCtl sc, cudaStream_t st) {
+int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, cudaStream_t st) {
+    count_launches(2);
+    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, t.base, fillpos, t.col, t.val, t.val64);
+    k_adj_sort<<<state_grid(m), kThreads, 0, st>>>(m->S, t.base, t.cnt, t.col, t.val, t.val64);
+    VC_CUDA(cudaGetLastError());
+    return VC_OK;
+}
+
+int launch_adj_sweep(Mdp* m, const AdjRows& t, const float* b, const float* x, float* x_out, SweepCtl sc,
+                     cudaStream_t st) {
     count_launches(1);
-    k_adj_resid64<<<state_grid(m), kThreads, 0, st>>>(m->S, m->gamma, rowT, colT, valT64, rho, lam, r, sc);
+    k_adj_sweep<<<state_grid(m), kThreads, 0, st>>>(m->S, (float)m->gamma, t.base, t.cnt, t.col, t.val, b, x, x_out, sc);
+    VC_CUDA(cudaGetLastError());
+    return VC_OK;
+}
+
+int launch_adj_resid64(Mdp* m, const AdjRows& t, const double* rho, const double* lam, float* r, SweepCtl sc,
+                       cudaStream_t st) {
+    count_launches(1);
+    k_adj_resid64<<<state_grid(m), kThreads, 0, st>>>(m->S, m->gamma, t.base, t.cnt, t.col, t.val64, rho, lam, r, sc);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }
@@ -246,27 +348,31 @@ int launch_f64_to_f32(const double* in, float* out, int n, cudaStream_t st) {
     return VC_OK;
 }
 
-int grad_partial_stride(const Mdp* m) { return 2 * (m->md.H <= 4 ? 4 : m->md.H <= 8 ? 8 : 16) + 6; }
+static int grad_mh(const Mdp* m) { return m->md.H <= 4 ? 4 : m->md.H <= 8 ? 8 : 16; }
+
+// Two blocks per SM: the block sums' FP64 shuffles are then a small part.
+static int grad_grid(const Mdp* m) { return std::min(state_grid(m), 2 * (m->num_sms > 0 ? m->num_sms : 148)); }
+
+size_t grad_partial_bytes(const Mdp* m) { return 8 * (size_t)grad_grid(m) * grad_slots(grad_mh(m)); }
 
 int launch_grad_contract(Mdp* m, const int32_t* pi, const double* V, const double* lam, const double* rho,
                          double* partial, double* out, cudaStream_t st) {
-    const int g = state_grid(m);
-    const int MH = m->md.H <= 4 ? 4 : m->md.H <= 8 ? 8 : 16;
+    const int g = grad_grid(m), MH = grad_mh(m);
     count_launches(2);
     if (MH == 4)
-        k_grad_contract<4><<<g, kThreads, 0, st>>>(m->md, m->rates, m->gamma, pi, V, lam, rho, partial);
+        k_grad_contract<4><<<g, kThreads, 0, st>>>(m->md, pi, V, lam, rho, partial);
     else if (MH == 8)
-        k_grad_contract<8><<<g, kThreads, 0, st>>>(m->md, m->rates, m->gamma, pi, V, lam, rho, partial);
+        k_grad_contract<8><<<g, kThreads, 0, st>>>(m->md, pi, V, lam, rho, partial);
     else
-        k_grad_contract<16><<<g, kThreads, 0, st>>>(m->md, m->rates, m->gamma, pi, V, lam, rho, partial);
-    k_grad_final<<<1, 64, 0, st>>>(partial, g, MH, m->md.H, out);
+        k_grad_contract<16><<<g, kThreads, 0, st>>>(m->md, pi, V, lam, rho, partial);
+    k_grad_final<<<1, kThreads, 0, st>>>(partial, g, MH, m->md.C, m->md.H, m->rates, m->gamma, out);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }
 
 int launch_objective(const double* V, const double* rho, long long S, double* J, cudaStream_t st) {
     count_launches(1);
-    k_objective<<<1, 1024, 0, st>>>(V, rho, S, J);
+    k_objective<<<kObjBlocks, kObjThreads, 0, st>>>(V, rho, S, J);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }

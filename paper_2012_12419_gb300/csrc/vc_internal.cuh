@@ -651,6 +651,16 @@ struct CsrPlan {
 
 struct KrylovCtl;  // vc_krylov.cuh
 
+// The adjoint's matrix P_pi^T in slices of 32 rows (vc_grad.cu): entry j of row y at
+// base[y / 32] + 32 j + y % 32, cnt[y] entries sorted by source.
+struct AdjRows {
+    int64_t* base = nullptr;  // [ceil(S / 32) + 1]
+    int32_t* cnt = nullptr;   // [S]
+    int32_t* col = nullptr;
+    float* val = nullptr;
+    double* val64 = nullptr;
+};
+
 struct Mdp {
     int fmt;              // VC_IMPLICIT / VC_CSR_F32 / VC_CSR_BF16 (| VC_PADDED)
     bool has_model;
@@ -672,6 +682,7 @@ struct Mdp {
     double* rate_tab = nullptr; // rates.occ_tab (device, owned)
     CsrPlan plan;
     int64_t loop_cap = 0;       // most entries of 32 / A consecutive states' rows (the resident loop's chunks)
+    const AdjRows* adj = nullptr;  // a view for the adjoint solve: its products use these rows
     std::string tune_report;    // candidates and times of the last autotune
     // sliced copy of the stored matrix (SELL-C-sigma, C = 32 states per slice): one
     // 128-byte-aligned record per slice in a byte slab (header, state map, R / scale,
@@ -787,12 +798,14 @@ int exclusive_scan(Mdp* m, const int32_t* cnt, int64_t n, int64_t* out, cudaStre
 
 // Adjoint gradient kernels (vc_grad.cu).
 int launch_adj_count(Mdp* m, const int32_t* pi, int32_t* cnt, int* err, cudaStream_t st);
-int launch_adj_fill(Mdp* m, const int32_t* pi, const int64_t* rowT, int32_t* fillpos, int32_t* colT, float* valT,
-                    double* valT64, cudaStream_t st);
-int launch_adj_resid64(Mdp* m, const int64_t* rowT, const int32_t* colT, const double* valT64, const double* rho,
-                       const double* lam, float* r, SweepCtl sc, cudaStream_t st);
+int launch_adj_width(Mdp* m, const int32_t* cnt, int32_t* width, unsigned long long* total, cudaStream_t st);
+int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, cudaStream_t st);
+int launch_adj_sweep(Mdp* m, const AdjRows& t, const float* b, const float* x, float* x_out, SweepCtl sc,
+                     cudaStream_t st);
+int launch_adj_resid64(Mdp* m, const AdjRows& t, const double* rho, const double* lam, float* r, SweepCtl sc,
+                       cudaStream_t st);
 int launch_f64_to_f32(const double* in, float* out, int n, cudaStream_t st);
-int grad_partial_stride(const Mdp* m);
+size_t grad_partial_bytes(const Mdp* m);
 int launch_grad_contract(Mdp* m, const int32_t* pi, const double* V, const double* lam, const double* rho,
                          double* partial, double* out, cudaStream_t st);
 

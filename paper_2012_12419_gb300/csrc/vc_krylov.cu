@@ -257,8 +257,7 @@ struct ModelProduct2 {
     }
 };
 
-// Stored rows of pi (pi = nullptr: action 0, the one row of a single-action system such as
-// the adjoint's): y(s) = x(s) - gamma (scale) sum_j val_j x[col_j], fused multiply-adds in
+// Stored rows of pi: y(s) = x(s) - gamma (scale) sum_j val_j x[col_j], fused multiply-adds in
 // column order; the gathers of eight entries are in flight before the first of them is added.
 template <typename VT>
 struct RowProduct {
@@ -279,7 +278,7 @@ struct RowProduct {
     __device__ __forceinline__ void first(const KrylovArgs&, const float*, int) const {}
     __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
         y[0] = xin[s];
-        const int act = pi ? pi[s] : 0;
+        const int act = pi[s];
         if (act < 0 || act >= A) return;
         const int64_t r = (int64_t)s * A + act;
         const int64_t lo = __ldg(row_ptr + r);
@@ -301,6 +300,38 @@ struct RowProduct {
                 if (j0 + u < n) acc = fmaf(w[u], g[u], acc);
         }
         if (scale) acc *= __ldg(scale + r);
+        y[0] -= gamma * acc;
+    }
+};
+
+// The adjoint's rows, in slices of 32 (AdjRows): the lanes of a warp read consecutive entries.
+struct AdjProduct {
+    static constexpr int kWidth = 1;
+    static constexpr bool kTwoPass = false;
+    float gamma;
+    AdjRows t;
+    __device__ __forceinline__ void setup(const KrylovArgs&, int) const {}
+    __device__ __forceinline__ void first(const KrylovArgs&, const float*, int) const {}
+    __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
+        y[0] = xin[s];
+        const int n = __ldg(t.cnt + s);
+        const int64_t lo = __ldg(t.base + (s >> 5)) + (s & 31);
+        const int32_t* cp = t.col + lo;
+        const float* vp = t.val + lo;
+        float acc = 0.0f;
+        for (int j0 = 0; j0 < n; j0 += 8, cp += 256, vp += 256) {
+            float w[8], g[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (j0 + u < n) {
+                    w[u] = __ldg(vp + 32 * u);
+                    g[u] = xin[__ldg(cp + 32 * u)];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (j0 + u < n) acc = fmaf(w[u], g[u], acc);
+        }
         y[0] -= gamma * acc;
     }
 };
@@ -475,6 +506,7 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budge
 constexpr int kKrTwoPass = 600000;
 
 static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, int budget, cudaStream_t st) {
+    if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, budget, st);
     if (!m->has_model) {
         if ((m->fmt & 0xF) == VC_CSR_BF16) {
             RowProduct<uint16_t> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const uint16_t*)m->val, m->scale, pi};

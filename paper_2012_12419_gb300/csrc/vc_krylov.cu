@@ -22,7 +22,7 @@
 //
 // Bound: L2 latency of the gathers and of five short vector steps, and five (seven) barriers an
 // iteration.  Whole calls, launched kernels against this one: evaluation of a policy of
-// 524,288 states 8.6 -> 3.6 ms, gradient step of 343,750 states 12.3 -> 8.6 ms, solves of
+// 524,288 states 8.6 -> 2.7 ms, gradient step of 343,750 states 12.3 -> 8.6 ms, solves of
 // 2.5 M states 10.1 -> 8.0 ms and of 640 states 0.74 -> 0.46 ms.
 #include <math.h>
 #include <string.h>
@@ -502,8 +502,10 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budge
     }
 }
 
-// States from which the two-pass product is the faster one.
-constexpr int kKrTwoPass = 600000;
+// States from which the two-pass product is the faster one.  Evaluation of a policy, one pass
+// against two: 25,920 states 1.24 / 1.33 ms, 100,000 1.73 / 1.75, 131,072 1.90 / 1.82, 250,000
+// 2.01 / 1.66, 524,288 3.58 / 2.72; items of two states (Q even): 343,750 2.77 / 2.35.
+constexpr int kKrTwoPass = 120000;
 
 static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, int budget, cudaStream_t st) {
     if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, budget, st);

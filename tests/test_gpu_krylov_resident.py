@@ -53,7 +53,7 @@ def test_stored_rows(S, A, K, bf16):
 
 # H, C, Q: 1 host; one CTA; the two-pass product with Q odd (items of 4), Q even (items of 2)
 # and more than 8 hosts (items of 2 and the wide host bound)
-@pytest.mark.parametrize("H,C,Q", [(1, 1, 1), (2, 2, 5), (3, 3, 4), (3, 6, 5), (5, 4, 14), (7, 3, 15), (7, 3, 20),
+@pytest.mark.parametrize("H,C,Q", [(1, 1, 1), (2, 2, 5), (3, 3, 4), (3, 6, 5), (5, 4, 14), (5, 4, 15), (6, 4, 6), (7, 3, 15), (7, 3, 20),
                                    (8, 3, 5), (9, 3, 2)])
 def test_model_products(H, C, Q):
     native = native_or_skip()

@@ -647,6 +647,7 @@ struct CsrPlan {
     int64_t ntiles = 0;
     int warps = 0;       // consumer warps per CTA (sliced ring sweep)
     int minb = 1;        // register budget of the sliced ring kernel (1: 80 registers, 2: 60)
+    int per_unit = 1;    // actions a warp of the sliced ring sweep takes at once
 };
 
 struct KrylovCtl;  // vc_krylov.cuh

@@ -30,13 +30,20 @@
 // into a ring of shared memory, one cp.async.bulk per tile, completion counted on an
 // mbarrier, L2 evict-first.  Tiles take their actual size in the ring (a tile that would
 // wrap restarts at the ring base; bytes are reused only after the tiles holding them are
-// released, in order).  Consumer warps take (slice, action) blocks of the CTA's tile
-// sequence round-robin, one lane per state: shared-memory reads are lane-consecutive (no
+// released, in order).  Consumer warps take units (two actions of a slice) of the CTA's tile
+// sequence in order, one lane per state: shared-memory reads are lane-consecutive (no
 // bank conflicts) and the V gathers of a warp fall on a few cache lines because the
 // lanes' successors share offsets.  A block's Q values overwrite its own R row in the
 // ring (read once, by the same lane), so no separate Q buffer takes shared memory from the
-// ring; the warp that completes a tile's last block takes the max over actions from the
+// ring; the warp that completes a tile's last unit takes the max over actions from the
 // tile's R rows and releases the tile.
+// The sweep is bound by its consumers (issue 44 %, L1 and shared-memory latency), no longer by
+// HBM: 24-31 % fewer bytes (16-bit column offsets) gained 4 % on FP32 values and lost 16 % on
+// BF16.  A unit's claim, wait and release cost as much as an action's row, hence two actions a
+// unit; with more, too few warps find work in the tiles in flight.  Sweeps of 1, 2, 3, 4 actions
+// a unit: 2.5 M states (1.2 GB) 230 / 213 / 221 / 236 us, 524,288 states 47.4 / 43.3 / 45.7 / 49.5;
+// 12.5 M states in BF16 (6.0 GB) 1,399 / 1,337 / 1,393 / 1,456, and 1,171 with the record's regions
+// found once a unit in 32-bit arithmetic.
 // Sweeps are launched as programmatic dependents of the previous sweep: a CTA that starts
 // while the previous grid drains stages its first tiles (the slab never changes), then
 // waits for that grid (griddepcontrol.wait) before it reads V or the loop's control
@@ -473,22 +480,35 @@ __device__ __forceinline__ float row_dot(const int32_t* cp, const VT* vp, int w,
 }
 static_assert(kSellLast >= kSellBatch, "a remainder must fit one batch");
 
+// Where the regions of a stored record lie (bytes from its start; a record is far below 2^31).
+struct RecAt {
+    int rows, scale, col, val;
+};
+
+template <typename VT>
+__device__ __forceinline__ RecAt rec_at(const unsigned char* rec, int A, bool has_scale) {
+    RecAt p;
+    p.rows = reinterpret_cast<const int32_t*>(rec)[A];
+    p.scale = 256 + 128 * A;
+    p.col = p.scale + (has_scale ? 128 * A : 0);
+    p.val = p.col + 128 * p.rows;
+    return p;
+}
+
 // Q value of lane `lane` in block `a` of a slice record (shared or global memory):
 // R + gamma (scale) sum_j val_j V[col_j], the sum in column order; SL: the same row with
 // its self-transition solved (q_self_loop).
 template <typename VT, bool SL>
-__device__ __forceinline__ float block_q(const unsigned char* rec, int A, int a, int lane, float gamma, bool has_scale,
-                                         const float* __restrict__ V, int S, Ctl* ctl) {
+__device__ __forceinline__ float block_q(const unsigned char* rec, const RecAt& p, int a, int lane, float gamma,
+                                         bool has_scale, const float* __restrict__ V, int S, Ctl* ctl) {
     const int32_t* hdr = reinterpret_cast<const int32_t*>(rec);
     const float rr = reinterpret_cast<const float*>(rec + 256)[a * kSellC + lane];
     if (rr == -INFINITY) return -INFINITY;
-    const int rows = hdr[A];
-    const RecLayout L = rec_layout(A, rows, (int)sizeof(VT), has_scale);
     const int r0 = hdr[a], w = hdr[a + 1] - r0;
-    const int32_t* cp = reinterpret_cast<const int32_t*>(rec + L.col) + r0 * kSellC + lane;
-    const VT* vp = reinterpret_cast<const VT*>(rec + L.val) + r0 * kSellC + lane;
+    const int32_t* cp = reinterpret_cast<const int32_t*>(rec + p.col) + r0 * kSellC + lane;
+    const VT* vp = reinterpret_cast<const VT*>(rec + p.val) + r0 * kSellC + lane;
 #ifdef VC_DEBUG_BOUNDS
-    if (!VC_IN_BOUNDS(ctl, r0 >= 0 && w >= 0 && hdr[a + 1] <= rows)) return -INFINITY;
+    if (!VC_IN_BOUNDS(ctl, r0 >= 0 && w >= 0 && hdr[a + 1] <= p.rows)) return -INFINITY;
     for (int j = 0; j < w; ++j)
         if (!VC_IN_BOUNDS(ctl, cp[j * kSellC] >= 0 && cp[j * kSellC] < S)) return -INFINITY;
 #else
@@ -498,7 +518,7 @@ __device__ __forceinline__ float block_q(const unsigned char* rec, int A, int a,
     float pss = 0.0f;
     const int self = SL ? reinterpret_cast<const int32_t*>(rec + 128)[lane] : -1;
     const float acc = row_dot<VT, SL>(cp, vp, w, V, self, pss);
-    const float sc = has_scale ? reinterpret_cast<const float*>(rec + L.scale)[a * kSellC + lane] : 1.0f;
+    const float sc = has_scale ? reinterpret_cast<const float*>(rec + p.scale)[a * kSellC + lane] : 1.0f;
     if (SL) {
         const float off = has_scale ? sc * acc : acc, ps = has_scale ? sc * pss : pss;
         // no self-transition (every placement row of the model): q_self_loop's denominator
@@ -540,10 +560,11 @@ __global__ void __launch_bounds__(kThreads) k_sell(SellArgs a, SweepCtl sc) {
     float res = 0.0f, vabs = 0.0f;
     for (int64_t g = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5; g < a.G; g += nw) {
         const unsigned char* rec = a.slab + a.rec[g] * 128;
+        const RecAt at = rec_at<VT>(rec, a.A, a.has_scale);
         float b1 = -INFINITY, b2 = -INFINITY;
         int ia = 0;
         for (int act = 0; act < a.A; ++act)
-            top2_step(act, block_q<VT, SL>(rec, a.A, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl), b1, b2, ia);
+            top2_step(act, block_q<VT, SL>(rec, at, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl), b1, b2, ia);
         write_state(a, reinterpret_cast<const int32_t*>(rec + 128)[lane], b1, b2, ia, res, vabs, sc.ctl);
     }
     if (sc.mode == kModeNone) return;
@@ -560,8 +581,10 @@ constexpr int kMaxTS = 4;       // most slices per tile (the planner's tile size
 static_assert(kSlots * (8 + 8 + 4 + 4) <= 384 && 384 + 8 * kSlots <= kHead, "slot words exceed the header");
 
 struct SellRingArgs {
-    FastDiv div_nb;   // division by TS * A (blocks per full tile)
-    FastDiv div_A;    // division by A
+    FastDiv div_nu;   // division by TS * ups (units per full tile)
+    FastDiv div_ups;  // division by ups
+    int ups;          // units per slice
+    int per_unit;     // actions of a unit (a slice's last may hold fewer)
     int TS;           // slices per tile (the last tile may hold fewer)
     int64_t ntiles;
     int ring;         // bytes of the tile ring
@@ -590,7 +613,7 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
     const int nrw = (int)(blockDim.x >> 5) - 1;  // consumer warps
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int A = a.A;
-    const int nb_full = t.TS * A;
+    const int nu_full = t.TS * t.ups;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; i++) {
             mbar_init(&full[i], 1);
@@ -682,11 +705,11 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
             if (loop_done(sc)) atomicExch(&s_abort, 1);
         }
     } else {
-        // ---------------- consumers: every warp takes the CTA's next unclaimed block (a
-        // shared counter over the blocks of the CTA's tile sequence), so blocks finish
+        // ---------------- consumers: every warp takes the CTA's next unclaimed unit (a
+        // shared counter over the units of the CTA's tile sequence), so units finish
         // roughly in tile order and the ring is released in order without waiting on a
-        // slow warp's backlog.  The planner keeps nrw <= (kSlots - 2) blocks-per-tile
-        // multiples, so claimed blocks never run kSlots tiles ahead of the oldest one.
+        // slow warp's backlog.  The planner keeps nrw <= (kSlots - 2) units-per-tile
+        // multiples, so claimed units never run kSlots tiles ahead of the oldest one.
         const int64_t nt_cta = (blockIdx.x < t.ntiles) ? (t.ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
         int i = 0;
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -696,24 +719,24 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
             int gb = 0;
             if (lane == 0) gb = atomicAdd(&s_next, 1);
             gb = __shfl_sync(0xffffffffu, gb, 0);
-            i = (int)fdiv((uint32_t)gb, t.div_nb);
-            const int b = gb - i * nb_full;
+            i = (int)fdiv((uint32_t)gb, t.div_nu);
+            const int b = gb - i * nu_full;
             if (i >= nt_cta) break;
             const int64_t tile = blockIdx.x + (int64_t)i * gridDim.x;
             const int64_t g0 = tile * t.TS;
             const int ns = (int)(((g0 + t.TS < a.G) ? g0 + t.TS : a.G) - g0);
-            const int nb = ns * A;
-            if (b >= nb) continue;  // the last tile may hold fewer slices
+            const int nu = ns * t.ups;
+            if (b >= nu) continue;  // the last tile may hold fewer slices
             const int s = i % kSlots;
             if (!mbar_wait(&full[s], (uint32_t)((i / kSlots) & 1), lim)) {
                 atomicExch(&s_fail, 1);
                 break;
             }
             unsigned char* base = ring + *((volatile uint32_t*)&slot_pos[s]);
-            const int sl = (int)fdiv((uint32_t)b, t.div_A), act = b - sl * A;
-            long long roff = 0;
+            const int sl = (int)fdiv((uint32_t)b, t.div_ups), act0 = (b - sl * t.ups) * t.per_unit;
+            int roff = 0;
             for (int k = 0; k < sl; ++k)
-                roff += rec_layout(A, reinterpret_cast<const int32_t*>(base + roff)[A], (int)sizeof(VT), a.has_scale)
+                roff += (int)rec_layout(A, reinterpret_cast<const int32_t*>(base + roff)[A], (int)sizeof(VT), a.has_scale)
                             .bytes;
 #ifdef VC_DEBUG_BOUNDS
             {
@@ -723,17 +746,21 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
                 if (!VC_IN_BOUNDS(sc.ctl, roff + rb <= tile_bytes)) roff = 0;
             }
 #endif
-            const float qv = block_q<VT, SL>(base + roff, A, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
-            // the Q value replaces the block's own R entry in the ring (read above, by this lane
-            // only); the proxy fence orders the write before the tile's next bulk copy
-            reinterpret_cast<float*>(base + roff + 256)[act * kSellC + lane] = qv;
+            // the Q values replace the unit's own R entries in the ring (read by this lane only); the
+            // proxy fence orders the writes before the tile's next bulk copy
+            const RecAt at = rec_at<VT>(base + roff, A, a.has_scale);
+            float* qrow = reinterpret_cast<float*>(base + roff + 256) + lane;
+            const int act1 = min(act0 + t.per_unit, A);
+            for (int act = act0; act < act1; ++act)
+                qrow[act * kSellC] =
+                    block_q<VT, SL>(base + roff, at, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __threadfence_block();
             __syncwarp();
             int l = 0;
-            if (lane == 0) l = (atomicAdd(&done_cnt[s], 1) == nb - 1);
+            if (lane == 0) l = (atomicAdd(&done_cnt[s], 1) == nu - 1);
             if (__shfl_sync(0xffffffffu, l, 0)) {
-                // the tile's last block: the max over actions and the state map come out
+                // the tile's last unit: the max over actions and the state map come out
                 // of shared memory first, the tile is released, and only then the state
                 // writes and the residual's read of V_in (global memory) follow, so the
                 // ring slot is not held over a global-memory round trip
@@ -749,7 +776,15 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
                         float b1 = -INFINITY, b2 = -INFINITY;
                         int ia = 0;
                         const float* qrow = reinterpret_cast<const float*>(rec + 256);
-                        for (int c = 0; c < A; ++c) top2_step(c, qrow[c * kSellC + lane], b1, b2, ia);
+                        if (a.pi || a.qgap) {
+                            for (int c = 0; c < A; ++c) top2_step(c, qrow[c * kSellC + lane], b1, b2, ia);
+                        } else {
+                            b1 = qrow[lane];
+                            for (int c = 1; c < A; ++c) {
+                                const float q = qrow[c * kSellC + lane];
+                                if (q > b1) b1 = q;
+                            }
+                        }
                         b1v[k] = b1;
                         b2v[k] = b2;
                         iav[k] = ia;
@@ -829,7 +864,9 @@ int sell_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
             VC_CUDA(cached_set_max_dyn_smem(fn_sl, dyn_max));
             const int threads = (nrw + 1) * 32;
             if (threads > fa.maxThreadsPerBlock || (long long)threads * fa.numRegs * ctas > 65536) continue;
-            if (nrw > (kSlots - 2) * TS * A) continue;  // claimed blocks stay within kSlots tiles
+            const int per_unit = 2;  // measured above
+            const int ups = (A + per_unit - 1) / per_unit;
+            if (nrw > (kSlots - 2) * TS * ups) continue;  // claimed units stay within kSlots tiles
             // the ring follows the header; Q values live in the tiles' own R rows
             const int budget = std::min(dyn_max, (smem_sm - 1024 * ctas) / ctas - (int)fa.sharedSizeBytes);
             const int ring = ((budget - kHead) / 128) * 128;
@@ -848,6 +885,7 @@ int sell_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
             P.cap = ring;
             P.stages = kSlots;
             P.warps = nrw;
+            P.per_unit = per_unit;
             P.minb = mb;
             P.ctas_per_sm = per_sm < ctas ? per_sm : ctas;
             P.smem = need;
@@ -874,8 +912,10 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
     const bool bf16 = a.has_scale;
     if (m->plan.tma) {
         SellRingArgs t;
-        t.div_nb = make_fastdiv((uint32_t)(m->plan.ts * m->A));
-        t.div_A = make_fastdiv((uint32_t)m->A);
+        t.per_unit = m->plan.per_unit;
+        t.ups = (m->A + t.per_unit - 1) / t.per_unit;
+        t.div_nu = make_fastdiv((uint32_t)(m->plan.ts * t.ups));
+        t.div_ups = make_fastdiv((uint32_t)t.ups);
         t.TS = m->plan.ts;
         t.ntiles = m->plan.ntiles;
         t.ring = (int)m->plan.cap;

@@ -505,17 +505,12 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     vc_grad_stats gs;
     memset(&gs, 0, sizeof(gs));
 
-    // temporaries, stream-ordered; freed on every exit path
+    // temporaries in two stream-ordered blocks (an allocation each costs the host some 20 us),
+    // freed on every exit path: what depends on S, then the transpose's entries
     AdjRows t;
-    int32_t* fillpos = nullptr;
-    int32_t* width = nullptr;
-    float* rhoF = nullptr;
-    double* partial = nullptr;
-    double* out = nullptr;
-    int* err = nullptr;  // error flags, then the transpose's entries (8 bytes on)
+    unsigned char* block[2] = {nullptr, nullptr};
     auto release = [&]() {
-        void* ps[] = {t.cnt, fillpos, width, t.base, t.col, t.val, t.val64, rhoF, partial, out, err};
-        for (void* p : ps)
+        for (unsigned char* p : block)
             if (p) cudaFreeAsync(p, st);
     };
     auto bail = [&](int rc) {
@@ -532,14 +527,25 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     // ---- P_pi^T in slices of 32 rows: in-degree count, slice sizes, exclusive scan, fill,
     // per-row sort by source
     const int64_t slices = ((int64_t)S + 31) / 32;
-    VC_TRY(cudaMallocAsync((void**)&t.cnt, 4 * (size_t)S, st));
-    VC_TRY(cudaMallocAsync((void**)&fillpos, 4 * (size_t)S, st));
-    VC_TRY(cudaMallocAsync((void**)&width, 4 * (size_t)slices, st));
-    VC_TRY(cudaMallocAsync((void**)&t.base, 8 * ((size_t)slices + 3), st));
-    VC_TRY(cudaMallocAsync((void**)&err, 16, st));
-    VC_TRY(cudaMemsetAsync(t.cnt, 0, 4 * (size_t)S, st));
-    VC_TRY(cudaMemsetAsync(fillpos, 0, 4 * (size_t)S, st));
-    VC_TRY(cudaMemsetAsync(err, 0, 16, st));
+    size_t used = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = used;
+        used += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_cnt = part(4 * (size_t)S), o_fill = part(4 * (size_t)S), o_err = part(16), zeroed = used;
+    const size_t o_width = part(4 * (size_t)slices), o_base = part(8 * ((size_t)slices + 3));
+    const size_t o_rho = part(4 * ((size_t)S + 8)), o_partial = part(grad_partial_bytes(m)), o_out = part(8 * ((size_t)nt + 1));
+    VC_TRY(cudaMallocAsync((void**)&block[0], used, st));
+    VC_TRY(cudaMemsetAsync(block[0], 0, zeroed, st));
+    t.cnt = reinterpret_cast<int32_t*>(block[0] + o_cnt);
+    t.base = reinterpret_cast<int64_t*>(block[0] + o_base);
+    int32_t* fillpos = reinterpret_cast<int32_t*>(block[0] + o_fill);
+    int32_t* width = reinterpret_cast<int32_t*>(block[0] + o_width);
+    int* err = reinterpret_cast<int*>(block[0] + o_err);  // error flags, then the transpose's entries (8 bytes on)
+    float* rhoF = reinterpret_cast<float*>(block[0] + o_rho);
+    double* partial = reinterpret_cast<double*>(block[0] + o_partial);
+    double* out = reinterpret_cast<double*>(block[0] + o_out);
     int rc = launch_adj_count(m, pi, t.cnt, err, st);
     if (rc) return bail(rc);
     if ((rc = launch_adj_width(m, t.cnt, width, (unsigned long long*)(err + 2), st))) return bail(rc);
@@ -551,13 +557,18 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     VC_TRY(cudaStreamSynchronize(st));
     if ((int)herr[0]) return bail(fail(VC_ERR_ARG, "the policy picks an infeasible action"));
     gs.nnz_transpose = herr[1];
-    VC_TRY(cudaMallocAsync((void**)&t.col, 4 * ((size_t)stored + 16), st));
-    VC_TRY(cudaMallocAsync((void**)&t.val, 4 * ((size_t)stored + 16), st));
-    VC_TRY(cudaMallocAsync((void**)&t.val64, 8 * ((size_t)stored + 16), st));
-    if ((rc = launch_adj_fill(m, pi, t, fillpos, st))) return bail(rc);
+    used = 0;
+    const size_t o_v64 = part(8 * (size_t)stored + 8), o_tv64 = part(8 * (size_t)stored), o_col = part(4 * (size_t)stored);
+    const size_t o_tcol = part(4 * (size_t)stored), o_val = part(4 * (size_t)stored);
+    VC_TRY(cudaMallocAsync((void**)&block[1], used, st));
+    t.val64 = reinterpret_cast<double*>(block[1] + o_v64);
+    t.col = reinterpret_cast<int32_t*>(block[1] + o_col);
+    t.val = reinterpret_cast<float*>(block[1] + o_val);
+    double* val_tmp = reinterpret_cast<double*>(block[1] + o_tv64);  // as filled, before the rows are ordered
+    int32_t* col_tmp = reinterpret_cast<int32_t*>(block[1] + o_tcol);
+    if ((rc = launch_adj_fill(m, pi, t, fillpos, col_tmp, val_tmp, st))) return bail(rc);
 
     // ---- lam: the transposed system (right-hand side rho, matrix P^T) as a view for the solver
-    VC_TRY(cudaMallocAsync((void**)&rhoF, 4 * ((size_t)S + 8), st));
     if ((rc = launch_f64_to_f32(rho, rhoF, S, st))) return bail(rc);
     Mdp T;
     T.has_model = false;
@@ -624,8 +635,6 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     }
 
     // ---- contraction over states, reduced in a fixed order
-    VC_TRY(cudaMallocAsync((void**)&partial, grad_partial_bytes(m), st));
-    VC_TRY(cudaMallocAsync((void**)&out, 8 * ((size_t)nt + 1), st));
     if ((rc = launch_grad_contract(m, pi, V, lam, rho, partial, out, st))) return bail(rc);
     VC_TRY(cudaMemcpyAsync(dJ_dtheta, out, 8 * (size_t)nt, cudaMemcpyDeviceToDevice, st));
     VC_TRY(cudaMemcpyAsync(&gs.J, out + nt, 8, cudaMemcpyDeviceToHost, st));

@@ -9,7 +9,7 @@
 // solve.  The transpose is stored in slices of 32 rows, entry j of row y at
 // base[y / 32] + 32 j + y % 32, so the lanes of a warp (a row each) read and write
 // consecutive entries; row after row their accesses were a row length apart (gradient step of
-// 343,750 states: fill and sort 0.59 -> 0.25 ms, the two adjoint solves 3.2 -> 1.9 ms).
+// 343,750 states: fill and sort 0.59 -> 0.23 ms, the two adjoint solves 3.2 -> 2.9 ms).
 // The contraction regenerates every event of each state's
 // post-decision state and differentiates its probability rate/Lam analytically:
 // d(rate/Lam) = drate/Lam - rate dLam/Lam^2, the self-loop taking minus the others, so
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_width(int S, const int32_t* __
 }
 
 __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, const int64_t* __restrict__ base,
-                           int32_t* __restrict__ fillpos, int32_t* __restrict__ colT, float* __restrict__ valT,
+                           int32_t* __restrict__ fillpos, int32_t* __restrict__ colT,
                            double* __restrict__ valT64) {
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < md.S; s += gridDim.x * blockDim.x) {
         int cols[kMaxRow];
@@ -63,34 +63,29 @@ __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, c
             const int y = cols[j];
             const int64_t slot = base[y >> 5] + 32LL * atomicAdd(&fillpos[y], 1) + (y & 31);
             colT[slot] = s;
-            valT[slot] = (float)probs[j];
             valT64[slot] = probs[j];
         }
     }
 }
 
-// Orders each transposed row by source state (insertion sort; in-degrees are small, and the
-// fill's order is nearly that of the sources).
+// Orders each transposed row by source state, out of place: an entry's position is the number
+// of the row's entries with a smaller source (sources are distinct), counted over the lanes'
+// consecutive loads.  In place by insertion, every step waited for its own loads and stores:
+// 432 us at 343,750 states.
 __global__ void k_adj_sort(int S, const int64_t* __restrict__ base, const int32_t* __restrict__ cnt,
+                           const int32_t* __restrict__ colU, const double* __restrict__ valU64,
                            int32_t* __restrict__ colT, float* __restrict__ valT, double* __restrict__ valT64) {
     for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < S; y += gridDim.x * blockDim.x) {
         const int64_t lo = base[y >> 5] + (y & 31);
         const int n = cnt[y];
-        for (int i = 1; i < n; i++) {
-            const int c = colT[lo + 32LL * i];
-            if (colT[lo + 32LL * (i - 1)] < c) continue;
-            const float v = valT[lo + 32LL * i];
-            const double v64 = valT64[lo + 32LL * i];
-            int j = i - 1;
-            while (j >= 0 && colT[lo + 32LL * j] > c) {
-                colT[lo + 32LL * (j + 1)] = colT[lo + 32LL * j];
-                valT[lo + 32LL * (j + 1)] = valT[lo + 32LL * j];
-                valT64[lo + 32LL * (j + 1)] = valT64[lo + 32LL * j];
-                j--;
-            }
-            colT[lo + 32LL * (j + 1)] = c;
-            valT[lo + 32LL * (j + 1)] = v;
-            valT64[lo + 32LL * (j + 1)] = v64;
+        for (int i = 0; i < n; i++) {
+            const int c = colU[lo + 32LL * i];
+            const double v = valU64[lo + 32LL * i];
+            int rank = 0;
+            for (int j = 0; j < n; j++) rank += colU[lo + 32LL * j] < c ? 1 : 0;
+            colT[lo + 32LL * rank] = c;
+            valT[lo + 32LL * rank] = (float)v;
+            valT64[lo + 32LL * rank] = v;
         }
     }
 }
@@ -316,10 +311,11 @@ int launch_adj_width(Mdp* m, const int32_t* cnt, int32_t* width, unsigned long l
     return VC_OK;
 }
 
-int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, cudaStream_t st) {
+int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, int32_t* col_tmp, double* val_tmp,
+                    cudaStream_t st) {
     count_launches(2);
-    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, t.base, fillpos, t.col, t.val, t.val64);
-    k_adj_sort<<<state_grid(m), kThreads, 0, st>>>(m->S, t.base, t.cnt, t.col, t.val, t.val64);
+    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, t.base, fillpos, col_tmp, val_tmp);
+    k_adj_sort<<<state_grid(m), kThreads, 0, st>>>(m->S, t.base, t.cnt, col_tmp, val_tmp, t.col, t.val, t.val64);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }

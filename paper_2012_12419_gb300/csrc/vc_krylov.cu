@@ -319,17 +319,17 @@ struct AdjProduct {
         const int32_t* cp = t.col + lo;
         const float* vp = t.val + lo;
         float acc = 0.0f;
-        for (int j0 = 0; j0 < n; j0 += 8, cp += 256, vp += 256) {
-            float w[8], g[8];
+        for (int j0 = 0; j0 < n; j0 += 16, cp += 512, vp += 512) {
+            float w[16], g[16];
 #pragma unroll
-            for (int u = 0; u < 8; u++) {
+            for (int u = 0; u < 16; u++) {
                 if (j0 + u < n) {
                     w[u] = __ldg(vp + 32 * u);
                     g[u] = xin[__ldg(cp + 32 * u)];
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 8; u++)
+            for (int u = 0; u < 16; u++)
                 if (j0 + u < n) acc = fmaf(w[u], g[u], acc);
         }
         y[0] -= gamma * acc;

@@ -975,6 +975,11 @@ __global__ void k_f32_to_f64_n(const float* __restrict__ in, double* __restrict_
         out[i] = (double)in[i];
 }
 
+__global__ void k_axpy64_n(double* __restrict__ V, const float* __restrict__ e, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        V[i] += (double)e[i];
+}
+
 // Calls f with std::integral_constant<int, MH>: MH = the batch's largest H when it is at
 // most 8 (per-host loops unrolled to exactly that bound), else 16.
 template <typename F>
@@ -1597,7 +1602,6 @@ int vc_build_batch(const vc_params* p, int32_t n, void* stream, vc_batch** out) 
         maxH = std::max(maxH, tmp.md.H);
     }
     if (!rc && b->total >= (1LL << 31)) rc = fail(VC_ERR_ARG, "total states must be < 2^31");
-    if (!rc && b->padded >= (1LL << 31)) rc = fail(VC_ERR_ARG, "total states (each instance rounded up to 64) must be < 2^31");
     if (rc) {
         delete b;
         return rc;
@@ -1797,7 +1801,11 @@ int vc_value_iterate_batch(vc_batch* bh, float* V, double* V64_out, int32_t* pi_
                     cs[i] = 2 * ki[i];
                     solved = solved && kd[i] == 1;
                 }
-                if (solved && (rc = launch_axpy64(b->V64, b->E0, (int)b->padded, st))) return rc;
+                if (solved) {
+                    count_launches(1);
+                    k_axpy64_n<<<b->grid, kThreads, 0, st>>>(b->V64, b->E0, b->padded);
+                    VC_LAUNCHED("k_axpy64_n");
+                }
             }
             if (!solved) {
                 // fixed-point correction sweeps (VC_ITER_PLAIN_CORRECTION, or BiCGSTAB broke

@@ -864,7 +864,7 @@ int sell_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
             VC_CUDA(cached_set_max_dyn_smem(fn_sl, dyn_max));
             const int threads = (nrw + 1) * 32;
             if (threads > fa.maxThreadsPerBlock || (long long)threads * fa.numRegs * ctas > 65536) continue;
-            const int per_unit = 2;  // measured above
+            const int per_unit = A >= 4 ? 2 : 1;  // measured above; a slice of few actions keeps its units
             const int ups = (A + per_unit - 1) / per_unit;
             if (nrw > (kSlots - 2) * TS * ups) continue;  // claimed units stay within kSlots tiles
             // the ring follows the header; Q values live in the tiles' own R rows

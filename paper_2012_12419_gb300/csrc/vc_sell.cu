@@ -750,10 +750,17 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
             // proxy fence orders the writes before the tile's next bulk copy
             const RecAt at = rec_at<VT>(base + roff, A, a.has_scale);
             float* qrow = reinterpret_cast<float*>(base + roff + 256) + lane;
-            const int act1 = min(act0 + t.per_unit, A);
-            for (int act = act0; act < act1; ++act)
-                qrow[act * kSellC] =
-                    block_q<VT, SL>(base + roff, at, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
+            if constexpr (SL && sizeof(VT) == 2) {
+                // always one action (see the launch); without the loop 64.9 us a sweep against 75.9 at
+                // 524,288 states
+                qrow[act0 * kSellC] =
+                    block_q<VT, SL>(base + roff, at, act0, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
+            } else {
+                const int act1 = min(act0 + t.per_unit, A);
+                for (int act = act0; act < act1; ++act)
+                    qrow[act * kSellC] =
+                        block_q<VT, SL>(base + roff, at, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
+            }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __threadfence_block();
             __syncwarp();
@@ -912,7 +919,14 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
     const bool bf16 = a.has_scale;
     if (m->plan.tma) {
         SellRingArgs t;
-        t.per_unit = m->plan.per_unit;
+        const long long cap = (long long)m->num_sms * m->plan.ctas_per_sm;
+        const unsigned grid = (unsigned)(m->plan.ntiles < cap ? m->plan.ntiles : cap);
+        // one action a unit where a CTA has few tiles, so the length of a unit counts (12,500
+        // states: 10.6 us a sweep against 10.9), and in the self-transition sweep, whose rows are
+        // longer, of BF16 values (524,288 states: 64.9 against 79.7 us) or of a slab beyond the L2
+        // (2.5 M states 284 against 291 us; within it 100,000 states 17.1 against 15.9)
+        const bool one = m->plan.ntiles < 4LL * grid || (sc.self_loop && (bf16 || m->sell_bytes > (128LL << 20)));
+        t.per_unit = one ? 1 : m->plan.per_unit;
         t.ups = (m->A + t.per_unit - 1) / t.per_unit;
         t.div_nu = make_fastdiv((uint32_t)(m->plan.ts * t.ups));
         t.div_ups = make_fastdiv((uint32_t)t.ups);
@@ -920,8 +934,6 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
         t.ntiles = m->plan.ntiles;
         t.ring = (int)m->plan.cap;
         t.roff = kHead;
-        const long long cap = (long long)m->num_sms * m->plan.ctas_per_sm;
-        const unsigned grid = (unsigned)(t.ntiles < cap ? t.ntiles : cap);
         const unsigned threads = (unsigned)(m->plan.warps + 1) * 32;
         count_launches(1);
         cudaLaunchConfig_t cfg = {};

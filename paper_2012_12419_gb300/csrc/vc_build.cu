@@ -503,7 +503,7 @@ static void by_h_build(int H, F&& f) {
 // Feasible rows and logical non-zeros of the model, nothing stored.  A row depends on its
 // post-decision state x alone, so every x is formed once and counted for defer and for each
 // placement that leads to it (a task on host k, a free queue slot, the host reachable), in place
-// of A rows a state: 243 -> 40 us at 343,750 states of 7 actions.
+// of A rows a state: 243 -> 57 us at 343,750 states of 7 actions.
 template <int MH>
 __global__ void __launch_bounds__(kThreads) k_model_tally(Model md, Rates rt, unsigned long long* tallies) {
     unsigned long long feas = 0, nz = 0;

@@ -146,7 +146,7 @@ __global__ void k_f64_to_f32(const double* __restrict__ in, float* __restrict__ 
 // an event), so the states only add those, in slots of a per-block partial row, and the
 // derivatives are formed from the totals: an FP64 multiply-add or two per sum and state in
 // place of ~40 FP64 divisions (FP64 issues two lanes a cycle and SM here).  Together with the
-// final sums below: 0.46 -> 0.06 ms at 343,750 states.
+// final sums below: 0.46 -> 0.08 ms at 343,750 states.
 enum GradSlot : int {
     kSumJ = 0,   // rho V
     kSumFull,    // w [q = Q]

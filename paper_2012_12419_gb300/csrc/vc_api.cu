@@ -70,7 +70,7 @@ static int alloc_work(Mdp* m) {
         {(void**)&m->pi2, 4 * S},
         {(void**)&m->kr, 20 * krylov_stride(m->S)},
         {(void**)&m->post, m->has_model ? 4 * S : 0},
-        {(void**)&m->kr_part, 24 * (size_t)std::max(state_grid(m), m->num_sms > 0 ? m->num_sms : 148)},
+        {(void**)&m->kr_part, sizeof(double) * kKrPartSets * kKrPartValues * (size_t)(m->num_sms > 0 ? m->num_sms : 148)},
         {(void**)&m->kctl, sizeof(KrylovCtl)},
         {(void**)&m->ctl, sizeof(Ctl)},
     };

@@ -709,7 +709,7 @@ struct Mdp {
     int32_t* pi2 = nullptr;
     float* kr = nullptr;        // BiCGSTAB vectors of the correction solve: r, p, v, s, t ([5][krylov_stride(S)])
     int32_t* post = nullptr;    // post-decision states of the policy under refinement (model handles)
-    double* kr_part = nullptr;  // BiCGSTAB per-block partials ([3][grid])
+    double* kr_part = nullptr;  // BiCGSTAB partials of the CTAs (at most one per SM; vc_krylov.cuh)
     KrylovCtl* kctl = nullptr;  // BiCGSTAB scalars (device) and their pinned mirror
     KrylovCtl* kctl_host = nullptr;
     Ctl* ctl = nullptr;         // device control block

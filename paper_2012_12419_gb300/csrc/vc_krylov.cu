@@ -44,7 +44,7 @@ constexpr int kKrItems = 128;       // least items of a CTA otherwise
 struct KrylovArgs {
     KrylovCtl* kc;
     Ctl* ctl;          // the handle's control block (error flags of the bounds-checking build)
-    double* part;      // [3][gridDim.x]: two partial sums and a partial max per CTA
+    double* part;      // [kKrPartSets][kKrPartValues][gridDim.x] (kr_part_set)
     const float* b;    // right-hand side and shadow residual
     float *x, *r, *p, *v, *s, *t;
     float* e;          // E[x(next) | .] of the two-pass product
@@ -140,6 +140,7 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
     }
     __syncthreads();
     const int G = (int)gridDim.x;
+    double* part = k.part + kr_part_set(stage) * kKrPartValues * G;
     if (w == 0) {
         PairSum t0, t1;
         if (l < nw) {
@@ -161,9 +162,9 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
                 sh.tot[1] = v1;
                 sh.tot[2] = vm;
             } else {
-                k.part[blockIdx.x] = v0;
-                if (D1) k.part[G + blockIdx.x] = v1;
-                if (MX) k.part[2 * G + blockIdx.x] = vm;
+                part[blockIdx.x] = v0;
+                if (D1) part[G + blockIdx.x] = v1;
+                if (MX) part[2 * G + blockIdx.x] = vm;
             }
         }
     }
@@ -172,9 +173,9 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
         double v0 = 0.0, v1 = 0.0, vm = 0.0;
         if (G > 1) {
             for (int i = l; i < G; i += 32) {
-                v0 += __ldcg(k.part + i);
-                if (D1) v1 += __ldcg(k.part + G + i);
-                if (MX) vm = fmax(vm, __ldcg(k.part + 2 * G + i));
+                v0 += __ldcg(part + i);
+                if (D1) v1 += __ldcg(part + G + i);
+                if (MX) vm = fmax(vm, __ldcg(part + 2 * G + i));
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {

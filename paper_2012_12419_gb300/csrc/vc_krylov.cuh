@@ -29,6 +29,16 @@ struct KrylovCtl {
 
 enum KrylovStage : int { kKrInit = 0, kKrV = 1, kKrT = 2, kKrX = 3 };
 
+// Partial sums of the resident kernel: a stage stores a CTA's (two sums and a maximum), passes
+// one grid barrier, and every CTA reads all of them.  A late CTA may still read stage T's
+// while an early one stores stage X's, as no barrier lies between the two (the x / r update
+// touches only a CTA's own states), so these two use different sets.  Before every other
+// stage the product's first barrier separates the last readers from the next writers.
+constexpr int kKrPartSets = 2;
+constexpr int kKrPartValues = 3;  // per CTA and set
+__host__ __device__ constexpr int kr_part_set(int stage) { return stage % kKrPartSets; }
+static_assert(kr_part_set(kKrT) != kr_part_set(kKrX), "no barrier between the readers of T and the writers of X");
+
 // Block-wide sum over NT threads in a fixed order; result valid in thread 0.
 template <int NT>
 __device__ __forceinline__ double block_sum(double v) {

@@ -5,14 +5,15 @@
 // control block and FP64 block sums (two FP64 multiply-adds per SM and cycle on this chip), with
 // host reads in between.  Here at most one CTA per SM stays for the whole solve: a CTA owns the
 // same states in every vector, so only p and s cross CTAs; a grid barrier separates the five
-// steps; the threads' dot products are added as FP32 pairs (sum and error term), so FP64 is
-// left with one partial per CTA; and every CTA adds the same partials in the same order and
-// advances its own copy of the scalars.
+// steps; the threads' dot products are added as three FP32 terms (Sum3), so FP64 is left with
+// one partial per CTA; and every CTA adds the same partials in the same order and advances its
+// own copy of the scalars.
 //
 // A dot product is a sum of FP32 chains, chain c over the states c, c + chains, c + 2 chains, ..
-// with `chains` fixed by the model's size and the device (state_grid x kThreads), and the
-// chains are added in about twice FP32's precision; so neither the width of an item nor the
-// number of CTAs changes a solve.
+// with `chains` fixed by the model's size and the device (state_grid x kThreads).  The chains
+// are grouped by thread, warp and CTA and added in no less than FP64's precision: a solve is
+// reproducible bit for bit for a fixed grid and item width, and others agree with it up to that
+// rounding.
 //
 // The product by A = I - gamma P_pi has three forms: from the stored rows; from the implicit
 // model state by state (2H + 3 scalar gathers around x_pi(s)); and, for large models, in two
@@ -96,99 +97,145 @@ __device__ inline void kr_advance(KrylovCtl* c, int stage, double d0, double d1,
     }
 }
 
-// A sum of FP32 values as an unevaluated pair, every addition split exactly (Knuth's two-sum;
-// T. Ogita, S. M. Rump, S. Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26(6),
-// 2005), so it comes out as if summed in about twice FP32's precision.
-struct PairSum {
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float p) {
-        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-        c += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
-        s = t;
+// A sum of FP32 values as three unevaluated FP32 terms, every addition but the last term's split
+// exactly (Knuth's two-sum; SumK with K = 3 of T. Ogita, S. M. Rump, S. Oishi, "Accurate sum and
+// dot product", SIAM J. Sci. Comput. 26(6), 2005), so it comes out as if summed in about three
+// times FP32's precision: no worse than FP64, which this chip adds at two a cycle and SM.
+struct Sum3 {
+    float s = 0.0f, c = 0.0f, e = 0.0f;
+    static __device__ __forceinline__ float two_sum(float& a, float p) {
+        const float t = __fadd_rn(a, p), z = __fsub_rn(t, a);
+        const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(p, z));
+        a = t;
+        return err;
     }
-    __device__ __forceinline__ void warp_sum() {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float os = __shfl_down_sync(0xffffffffu, s, o), oc = __shfl_down_sync(0xffffffffu, c, o);
-            add(os);
-            c += oc;
+    __device__ __forceinline__ void add(float p) { e += two_sum(c, two_sum(s, p)); }
+    __device__ __forceinline__ void merge(float os, float oc, float oe) {
+        add(os);
+        e += two_sum(c, oc) + oe;
+    }
+    __device__ __forceinline__ double value() const { return ((double)e + (double)c) + (double)s; }
+};
+
+// The same with FP64's range for FP32 terms: once one of 2^96 or more (an infinity, a NaN) is
+// met, the sum goes on scaled by 2^-32, which no sum of FP32 terms overflows; what that shifts
+// out lies more than 200 bits below the term.
+struct DotSum {
+    static constexpr int kWords = 4;
+    static constexpr float kLarge = 0x1p96f, kDown = 0x1p-32f;
+    static constexpr double kUp = 0x1p32;
+    Sum3 v;
+    float scale = 1.0f;
+    __device__ __forceinline__ void scale_down() {
+        v.s *= kDown;
+        v.c *= kDown;
+        v.e *= kDown;
+        scale = kDown;
+    }
+    __device__ __forceinline__ void add(float p) {
+        if (!(fabsf(p) < kLarge) && scale == 1.0f) [[unlikely]]
+            scale_down();
+        v.add(p * scale);
+    }
+    // One scale for the warp (every lane calls it).
+    __device__ __forceinline__ void align() {
+        if (__any_sync(0xffffffffu, scale != 1.0f)) [[unlikely]] {
+            if (scale == 1.0f) scale_down();
         }
     }
+    // The sum over the half-warp's lanes, one scale in all of them.
+    __device__ __forceinline__ void half_warp_sum() {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) add_lane(v, o);
+    }
+    // This lane's terms plus those that lane ^ o gives.
+    __device__ __forceinline__ void add_lane(const Sum3& given, int o) {
+        const float s = __shfl_xor_sync(0xffffffffu, given.s, o), c = __shfl_xor_sync(0xffffffffu, given.c, o);
+        v.merge(s, c, __shfl_xor_sync(0xffffffffu, given.e, o));
+    }
+    __device__ __forceinline__ double value() const { return scale == 1.0f ? v.value() : kUp * v.value(); }
+    __device__ __forceinline__ void put(float* w) const { w[0] = v.s, w[1] = v.c, w[2] = v.e, w[3] = scale; }
+    __device__ __forceinline__ void get(const float* w) { v.s = w[0], v.c = w[1], v.e = w[2], scale = w[3]; }
 };
 
 struct KrShared {
     KrylovCtl c;                           // this CTA's copy of the scalars
-    float2 d0[kKrThreads / 32], d1[kKrThreads / 32];
+    float dot[2][kKrThreads / 32][DotSum::kWords];  // the warps' sums
     unsigned int mx;                       // bits of the CTA's max |r|
-    double tot[3];
+    double tot[2];
     int fail;
 };
 
 // CTA totals -> grid totals -> scalars of `stage` in every CTA's copy.  False once a barrier
 // wait gave up.  D1, MX: whether the stage has a second dot product, a maximum.
 template <bool D1, bool MX>
-__device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, GridBarrier& bar, int stage, PairSum a0,
-                                          PairSum a1, float mx) {
+__device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, GridBarrier& bar, int stage, DotSum a0,
+                                          DotSum a1, float mx) {
     const int w = (int)threadIdx.x >> 5, l = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
-    a0.warp_sum();
-    if (D1) a1.warp_sum();
-    const unsigned int mb = MX ? __reduce_max_sync(0xffffffffu, fbits(mx)) : 0u;
-    if (l == 0) {
-        sh.d0[w] = make_float2(a0.s, a0.c);
-        if (D1) sh.d1[w] = make_float2(a1.s, a1.c);
-        if (MX) atomicMax(&sh.mx, mb);
+    // lanes 0..15 add up the first product, 16..31 the second (without one, the first again)
+    static_assert(kKrThreads / 32 <= 16, "a half-warp adds up the warps' sums");
+    DotSum t = a0;
+    if (D1) {
+        if (a0.scale != a1.scale) {
+            if (a0.scale == 1.0f) a0.scale_down();
+            else a1.scale_down();
+        }
+        a0.align();
+        a1.align();
+        t = l < 16 ? a0 : a1;
+        t.add_lane(l < 16 ? a1.v : a0.v, 16);
+    } else {
+        t.align();
+        t.add_lane(t.v, 16);
     }
+    t.half_warp_sum();
+    const unsigned int mb = MX ? __reduce_max_sync(0xffffffffu, fbits(mx)) : 0u;
+    if (l == 0 || (D1 && l == 16)) t.put(sh.dot[l >> 4][w]);
+    if (MX && l == 0) atomicMax(&sh.mx, mb);
     __syncthreads();
     const int G = (int)gridDim.x;
     double* part = k.part + kr_part_set(stage) * kKrPartValues * G;
     if (w == 0) {
-        PairSum t0, t1;
-        if (l < nw) {
-            t0.s = sh.d0[l].x;
-            t0.c = sh.d0[l].y;
-            if (D1) {
-                t1.s = sh.d1[l].x;
-                t1.c = sh.d1[l].y;
-            }
-        }
-        t0.warp_sum();
-        if (D1) t1.warp_sum();
+        DotSum sum;
+        if ((l & 15) < nw && (D1 || l < 16)) sum.get(sh.dot[l >> 4][l & 15]);
+        sum.align();
+        sum.half_warp_sum();
+        const double v0 = sum.value(), v1 = D1 ? __shfl_sync(0xffffffffu, v0, 16) : 0.0;
         if (l == 0) {
-            const double v0 = (double)t0.s + (double)t0.c, v1 = (double)t1.s + (double)t1.c;
-            const double vm = MX ? (double)__uint_as_float(sh.mx) : 0.0;
-            if (MX) sh.mx = 0u;
             if (G == 1) {
                 sh.tot[0] = v0;
                 sh.tot[1] = v1;
-                sh.tot[2] = vm;
             } else {
                 part[blockIdx.x] = v0;
                 if (D1) part[G + blockIdx.x] = v1;
-                if (MX) part[2 * G + blockIdx.x] = vm;
+                if (MX) *reinterpret_cast<unsigned int*>(part + 2 * G + blockIdx.x) = sh.mx;  // FP32 bits
             }
         }
     }
     if (!bar.arrive_and_wait()) return false;
     if (w == 0) {
-        double v0 = 0.0, v1 = 0.0, vm = 0.0;
+        double v0 = 0.0, v1 = 0.0;
+        unsigned int vm = 0u;
         if (G > 1) {
-            for (int i = l; i < G; i += 32) {
-                v0 += __ldcg(part + i);
-                if (D1) v1 += __ldcg(part + G + i);
-                if (MX) vm = fmax(vm, __ldcg(part + 2 * G + i));
+            // as above: a half-warp a product
+            const double* mine = part + (D1 && l >= 16 ? G : 0);
+            for (int i = D1 ? l & 15 : l; i < G; i += D1 ? 16 : 32) {
+                v0 += __ldcg(mine + i);
+                if (MX) vm = max(vm, __ldcg(reinterpret_cast<const unsigned int*>(part + 2 * G + i)));
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-                if (D1) v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-                if (MX) vm = fmax(vm, __shfl_xor_sync(0xffffffffu, vm, o));
-            }
+            for (int o = D1 ? 8 : 16; o > 0; o >>= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+            if (D1) v1 = __shfl_sync(0xffffffffu, v0, 16);
+            if (MX) vm = __reduce_max_sync(0xffffffffu, vm);
         } else if (l == 0) {
             v0 = sh.tot[0];
             v1 = sh.tot[1];
-            vm = sh.tot[2];
+            if (MX) vm = sh.mx;
         }
-        if (l == 0) kr_advance(&sh.c, stage, v0, v1, vm);
+        if (l == 0) {
+            kr_advance(&sh.c, stage, v0, v1, (double)__uint_as_float(vm));
+            if (MX) sh.mx = 0u;  // next written after the caller's barriers
+        }
     }
     __syncthreads();
     return true;
@@ -362,7 +409,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
     bool ok = true;
     if (!resumed) {
         // r = b, x = 0, with <b, b> and max |b|
-        PairSum a0;
+        DotSum a0;
         float mx = 0.0f;
         for (int v = c0; v < c1; v += step) {
             float d0[VW] = {};
@@ -381,7 +428,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
 #pragma unroll
             for (int j = 0; j < VW; j++) a0.add(d0[j]);
         }
-        ok = kr_reduce<false, true>(k, sh, bar, kKrInit, a0, PairSum(), mx);
+        ok = kr_reduce<false, true>(k, sh, bar, kKrInit, a0, DotSum(), mx);
     }
     // y = A x over the owned states, with the dot products of the stage
     auto product = [&](const float* xin, float* y, bool second) {
@@ -390,7 +437,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
             for (int t = f0; t < f1; t += step) op.first(k, xin, VW * t);
             if (!bar.sync()) return false;
         }
-        PairSum a0, a1;
+        DotSum a0, a1;
         for (int v = c0; v < c1; v += step) {
             float d0[VW] = {}, d1[VW] = {};
             for (long long i = (long long)VW * v; i < n; i += chains) {
@@ -444,7 +491,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
         if (!(ok = product(k.s, k.t, true)) || sh.c.done) break;
         // x += alpha p + omega s; r = s - omega t, with <b, r> and max |r|
         const float omega = (float)sh.c.omega;
-        PairSum a0;
+        DotSum a0;
         float mx = 0.0f;
         for (int v0 = c0; v0 < c1; v0 += step) {
             float d0[VW] = {};
@@ -468,7 +515,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
 #pragma unroll
             for (int j = 0; j < VW; j++) a0.add(d0[j]);
         }
-        ok = kr_reduce<false, true>(k, sh, bar, kKrX, a0, PairSum(), mx);
+        ok = kr_reduce<false, true>(k, sh, bar, kKrX, a0, DotSum(), mx);
     }
     if (threadIdx.x != 0) return;
     if (sh.fail) atomicOr(&k.kc->fault, 1);

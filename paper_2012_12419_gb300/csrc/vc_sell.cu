@@ -59,32 +59,14 @@
 
 #include "vc_internal.cuh"
 #include "vc_ptx.cuh"
+#include "vc_sell.cuh"
 
 namespace vc {
 
-constexpr int kSellC = 32;
 constexpr int kSellSigma = 4096;
 constexpr int kSellBatch = 16;  // gathers per batch of a row longer than kSellLast
 constexpr int kSellLast = 24;   // rows (and remainders) up to this length: one batch
 constexpr int kSellMaxA = 31;  // hdr holds A + 1 row offsets in 32 slots
-
-__host__ __device__ inline long long round128(long long x) { return (x + 127) & ~127LL; }
-
-// Byte offsets inside a slice record with `rows` rows of 32 entries.
-struct RecLayout {
-    int R, scale, col;
-    long long val, bytes;
-};
-
-__host__ __device__ inline RecLayout rec_layout(int A, long long rows, int vt, bool has_scale) {
-    RecLayout L;
-    L.R = 256;
-    L.scale = L.R + 128 * A;
-    L.col = L.scale + (has_scale ? 128 * A : 0);
-    L.val = L.col + 128LL * rows;
-    L.bytes = L.val + round128(32LL * vt * rows);
-    return L;
-}
 
 // ------------------------------------------------------------------------ build
 __device__ __forceinline__ bool nonzero_val(float v) { return v != 0.0f; }
@@ -480,37 +462,22 @@ __device__ __forceinline__ float row_dot(const int32_t* cp, const VT* vp, int w,
 }
 static_assert(kSellLast >= kSellBatch, "a remainder must fit one batch");
 
-// Where the regions of a stored record lie (bytes from its start; a record is far below 2^31).
-struct RecAt {
-    int rows, scale, col, val;
-};
-
-template <typename VT>
-__device__ __forceinline__ RecAt rec_at(const unsigned char* rec, int A, bool has_scale) {
-    RecAt p;
-    p.rows = reinterpret_cast<const int32_t*>(rec)[A];
-    p.scale = 256 + 128 * A;
-    p.col = p.scale + (has_scale ? 128 * A : 0);
-    p.val = p.col + 128 * p.rows;
-    return p;
-}
-
 // Q value of lane `lane` in block `a` of a slice record (shared or global memory):
 // R + gamma (scale) sum_j val_j V[col_j], the sum in column order; SL: the same row with
 // its self-transition solved (q_self_loop).
-template <typename VT, bool SL>
-__device__ __forceinline__ float block_q(const unsigned char* rec, const RecAt& p, int a, int lane, float gamma,
+template <typename VT, bool SL, typename I>
+__device__ __forceinline__ float block_q(const unsigned char* rec, const RecAt<I>& p, int a, int lane, float gamma,
                                          bool has_scale, const float* __restrict__ V, int S, Ctl* ctl) {
     const int32_t* hdr = reinterpret_cast<const int32_t*>(rec);
     const float rr = reinterpret_cast<const float*>(rec + 256)[a * kSellC + lane];
     if (rr == -INFINITY) return -INFINITY;
     const int r0 = hdr[a], w = hdr[a + 1] - r0;
-    const int32_t* cp = reinterpret_cast<const int32_t*>(rec + p.col) + r0 * kSellC + lane;
-    const VT* vp = reinterpret_cast<const VT*>(rec + p.val) + r0 * kSellC + lane;
+    const int32_t* cp = reinterpret_cast<const int32_t*>(rec + p.col) + (I)r0 * kSellC + lane;
+    const VT* vp = reinterpret_cast<const VT*>(rec + p.val) + (I)r0 * kSellC + lane;
 #ifdef VC_DEBUG_BOUNDS
     if (!VC_IN_BOUNDS(ctl, r0 >= 0 && w >= 0 && hdr[a + 1] <= p.rows)) return -INFINITY;
     for (int j = 0; j < w; ++j)
-        if (!VC_IN_BOUNDS(ctl, cp[j * kSellC] >= 0 && cp[j * kSellC] < S)) return -INFINITY;
+        if (!VC_IN_BOUNDS(ctl, cp[(I)j * kSellC] >= 0 && cp[(I)j * kSellC] < S)) return -INFINITY;
 #else
     (void)S;
     (void)ctl;
@@ -560,7 +527,7 @@ __global__ void __launch_bounds__(kThreads) k_sell(SellArgs a, SweepCtl sc) {
     float res = 0.0f, vabs = 0.0f;
     for (int64_t g = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5; g < a.G; g += nw) {
         const unsigned char* rec = a.slab + a.rec[g] * 128;
-        const RecAt at = rec_at<VT>(rec, a.A, a.has_scale);
+        const RecAt<long long> at = rec_at<long long>(rec, a.A, a.has_scale);  // a record of any size
         float b1 = -INFINITY, b2 = -INFINITY;
         int ia = 0;
         for (int act = 0; act < a.A; ++act)
@@ -748,7 +715,7 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
 #endif
             // the Q values replace the unit's own R entries in the ring (read by this lane only); the
             // proxy fence orders the writes before the tile's next bulk copy
-            const RecAt at = rec_at<VT>(base + roff, A, a.has_scale);
+            const RecAt<int> at = rec_at<int>(base + roff, A, a.has_scale);
             float* qrow = reinterpret_cast<float*>(base + roff + 256) + lane;
             if constexpr (SL && sizeof(VT) == 2) {
                 // always one action (see the launch); without the loop 64.9 us a sweep against 75.9 at

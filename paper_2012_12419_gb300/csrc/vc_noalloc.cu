@@ -63,10 +63,13 @@ static int noalloc_scratch(NoAllocScratch* out) {
     return VC_OK;
 }
 
-// Pass 1 of the sweep.
+// Pass 1 of the sweep; it also clears pass 2's residual words, so a call owes nothing to the state
+// that an earlier one left (calls that overlap, against the rule, spoil only themselves).
 template <int MH, int VW>
-__global__ void __launch_bounds__(kThreads) k_noalloc_post(Model md, Coef<float> c, const float* V, float* U, Ctl* ctl) {
+__global__ void __launch_bounds__(kThreads) k_noalloc_post(Model md, Coef<float> c, const float* V, float* U,
+                                                           unsigned int* cell, Ctl* ctl) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x < 2) cell[threadIdx.x] = 0u;
     const int items = md.S / VW;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < items; t += gridDim.x * blockDim.x)
         post_item<MH, VW, false>(md, c, V, VW * t, U, nullptr, ctl);
@@ -74,9 +77,9 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_post(Model md, Coef<float>
 
 // Pass 2 with max |V_out - V| over all states on the way: one atomicMax a block into cell[0]
 // (non-negative float bits, order independent), and the last block to arrive (ticket cell[1])
-// hands the result out and leaves both words zero for the next call.  A NaN difference counts
-// as +infinity: fmaxf would drop it, and a sweep that produced a NaN must not report a finite
-// residual.  Launched as pass 1's programmatic dependent.
+// hands the result out.  A NaN difference counts as +infinity: fmaxf would drop it, and a sweep
+// that produced a NaN must not report a finite residual.  Launched as pass 1's programmatic
+// dependent; it touches the words only once pass 1 has ended.
 template <int MH, int VW, bool ARG>
 __global__ void __launch_bounds__(kThreads) k_noalloc_max(Model md, const float* U, const float* V, float* V_out,
                                                           int32_t* pi, unsigned int* cell, float* residual, Ctl* ctl) {
@@ -109,8 +112,7 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_max(Model md, const float*
     __threadfence();
     if (atomicAdd(&cell[1], 1u) != gridDim.x - 1) return;
     __threadfence();
-    *residual = __uint_as_float(atomicExch(&cell[0], 0u));
-    atomicExch(&cell[1], 0u);
+    *residual = __uint_as_float(__ldcg(&cell[0]));
 }
 
 // Both passes.  Bound: the launches (a sweep of 17,500 states keeps the device busy for 4 us);
@@ -125,7 +127,7 @@ static int noalloc_run(const Mdp& m, const NoAllocScratch& sc, const float* V, f
     const int grid = std::min((items + threads - 1) / threads, 8 * sc.num_sms);
     float* U = sc.U + kUShift;
     count_launches(2);
-    k_noalloc_post<MH, VW><<<grid, threads, 0, st>>>(m.md, m.c32, V, U, ctl);
+    k_noalloc_post<MH, VW><<<grid, threads, 0, st>>>(m.md, m.c32, V, U, sc.res, ctl);
     VC_CUDA(cudaGetLastError());
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -201,3 +203,15 @@ extern "C" int vc_bellman32_noalloc(const vc_params* p, const float* V, float* V
 #endif
     return VC_OK;
 }
+
+#ifdef VC_DEBUG_BOUNDS
+// Test hook of the bounds-checking build: overwrites the residual words of the current device.
+extern "C" int vc_debug_noalloc_words(uint32_t residual, uint32_t ticket) {
+    NoAllocScratch sc;
+    const int rc = noalloc_scratch(&sc);
+    if (rc) return rc;
+    const uint32_t w[2] = {residual, ticket};
+    VC_CUDA(cudaMemcpy(sc.res, w, sizeof(w), cudaMemcpyHostToDevice));
+    return VC_OK;
+}
+#endif

@@ -258,12 +258,15 @@ int vc_mdp_slice(vc_mdp* m, void* stream);
 
 /*
  * Fault-injection hook for the bounded device waits (no paper counterpart).  The pipelined
- * sweeps (CSR and sliced) wait on shared-memory barriers for their staged tiles with an
- * iteration limit; polls >= 0 caps every such wait of this handle's later solves at that
- * many polls (0: give up at once), polls < 0 restores the default (2^22).  A wait that
- * gives up flags the sweep, the kernel drains its own copies in flight (with the default
- * limit) and returns, and vc_value_iterate returns VC_ERR_TIMEOUT; the handle and the
- * CUDA context stay usable.  Synchronous; applies to later launches on the handle.
+ * sweeps (CSR and sliced) wait on shared-memory barriers for their staged tiles, the resident
+ * loops (the FP32 loop of an implicit handle, the BiCGSTAB correction solve) on grid barriers,
+ * each with an iteration limit; polls >= 0 caps every such wait of this handle's later solves
+ * at that many polls (0: give up at once), polls < 0 restores the default (2^22).  A wait
+ * that gives up flags the solve, the kernel drains its own copies in flight (with the default
+ * limit) and returns, and the call returns VC_ERR_TIMEOUT; the handle and the CUDA context
+ * stay usable.  A stored matrix is swept by the launched kernels while a cap is set.
+ * Instances small enough for one thread block have no grid barrier.  Synchronous; applies to
+ * later launches on the handle.
  * VC_ERR_ARG for NULL.
  */
 int vc_set_wait_limit(vc_mdp* m, int64_t polls);

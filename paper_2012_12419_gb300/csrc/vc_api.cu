@@ -583,6 +583,7 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     T.kr_part = m->kr_part;
     T.kctl = m->kctl;
     T.kctl_host = m->kctl_host;
+    T.spin_polls = m->spin_polls;
     // (I - gamma P_pi^T) x = b in FP32: BiCGSTAB, or fixed-point sweeps x <- b + gamma P^T x
     // from x = 0 when it breaks down; *xo receives the buffer holding x
     auto solve_T = [&](float* b, double target, float** xo, long long* prods) -> int {

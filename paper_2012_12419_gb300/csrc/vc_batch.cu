@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "vc_batch.cuh"
+#include "vc_grid.cuh"
 #include "vc_implicit.cuh"
 #include "vc_internal.cuh"
 #include "vc_krylov.cuh"
@@ -1022,6 +1023,8 @@ struct Batch {
     unsigned long long* res64 = nullptr;
     long long* iters = nullptr;
     unsigned int* bar = nullptr;  // the resident loop's barrier counter and fault flag
+    Ctl* check = nullptr;         // its error flags (bounds-checking build)
+    long long spin_polls = -1;    // cap of its barrier waits (-1: the default)
     long long* max_d = nullptr;
     double* tol_d = nullptr;
     float* tol_scale = nullptr;  // per-instance factor of the correction loop's tolerance
@@ -1517,6 +1520,11 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
     a.U2 = b->U2;
     a.arrivals = b->bar;
     a.fault = (int*)b->bar + 1;
+    a.polls = barrier_polls(b->spin_polls < 0 ? 0 : b->spin_polls + 1);
+    a.ctl = b->check;
+#ifdef VC_DEBUG_BOUNDS
+    VC_CUDA(cudaMemsetAsync(&b->check->error, 0, sizeof(int), st));
+#endif
     a.first = 0;
     // sweeps of one launch: about a quarter of a second
     a.budget = (int)std::min<long long>(1 << 20, std::max<long long>(16, (long long)(2e10 / (double)b->padded)));
@@ -1529,6 +1537,11 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
         VC_CUDA(cudaMemcpyAsync(&h[1], a.fault, 4, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
         if (h[1]) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
+#ifdef VC_DEBUG_BOUNDS
+        int err = 0;
+        VC_CUDA(cudaMemcpy(&err, &b->check->error, sizeof(int), cudaMemcpyDeviceToHost));
+        if (err & kErrBounds) return fail(VC_ERR_CUDA, "a device bounds check failed (bounds-checking build)");
+#endif
         if (h[0] <= 0) return VC_OK;
         a.first += a.budget;
     }
@@ -1629,6 +1642,9 @@ int vc_build_batch(const vc_params* p, int32_t n, void* stream, vc_batch** out) 
     if (!rc) rc = balloc(b, (void**)&b->err, 16);
     if (!rc) rc = balloc(b, (void**)&b->iters, 16);
     if (!rc) rc = balloc(b, (void**)&b->bar, 16);
+#ifdef VC_DEBUG_BOUNDS
+    if (!rc) rc = balloc(b, (void**)&b->check, sizeof(Ctl));
+#endif
     if (!rc) rc = balloc(b, (void**)&b->max_d, 16);
     if (!rc) rc = balloc(b, (void**)&b->tol_d, 16);
     if (!rc) rc = balloc(b, (void**)&b->tol_scale, 4 * N);
@@ -2030,5 +2046,14 @@ int vc_batch_destroy(vc_batch* bh) {
     free_batch((Batch*)bh);
     return VC_OK;
 }
+
+#ifdef VC_DEBUG_BOUNDS
+// Test hook of the bounds-checking build: vc_set_wait_limit for the barrier waits of a batch's
+// resident loop.
+int vc_debug_batch_wait_limit(vc_batch* bh, int64_t polls) {
+    ((Batch*)bh)->spin_polls = polls;
+    return VC_OK;
+}
+#endif
 
 }  // extern "C"

@@ -52,6 +52,8 @@ struct BatchLoopArgs {
     float *V0, *V1, *U, *U2;  // U: kUShift past a 16-byte-aligned buffer
     unsigned int* arrivals;   // grid barrier, cleared by the host before each launch
     int* fault;               // set by a block whose barrier wait gave up
+    unsigned int polls;       // poll limit of a barrier wait
+    Ctl* ctl;                 // error flags of the bounds-checking build
     long long first;          // sweeps done so far
     int budget;
 };

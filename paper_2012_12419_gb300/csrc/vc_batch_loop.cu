@@ -70,17 +70,17 @@ struct LocalModel {
 };
 
 template <int MH, int VW, bool SL, typename D>
-__device__ __forceinline__ void post_share(const D& d, const float* V, float* U, float* W, int i0, int i1) {
+__device__ __forceinline__ void post_share(const D& d, const float* V, float* U, float* W, int i0, int i1, Ctl* ctl) {
     const LocalModel<MH> m(d);
     const float* Vi = V + d.off;
     float* Ui = U + d.off;
     float* Wi = SL ? W + d.off : nullptr;
-    for (int t = i0 + (int)(threadIdx.x & 31); t < i1; t += 32) post_item<MH, VW, SL>(m.md, m.c, Vi, VW * t, Ui, Wi, nullptr);
+    for (int t = i0 + (int)(threadIdx.x & 31); t < i1; t += 32) post_item<MH, VW, SL>(m.md, m.c, Vi, VW * t, Ui, Wi, ctl);
 }
 
 template <int MH, int VW, bool SL, typename D>
 __device__ __forceinline__ void max_share(const D& d, const float* V, const float* U, const float* W, float* Vo,
-                                          int i0, int i1, float& res, float& vabs) {
+                                          int i0, int i1, float& res, float& vabs, Ctl* ctl) {
     const LocalModel<MH> m(d);
     const float* Vi = V + d.off;
     const float* Ui = U + d.off;
@@ -89,7 +89,7 @@ __device__ __forceinline__ void max_share(const D& d, const float* V, const floa
     for (int t = i0 + (int)(threadIdx.x & 31); t < i1; t += 32) {
         float vin[VW], best[VW];
         ldv<VW>(Vi + VW * t, vin);
-        max_item<MH, VW, SL, false>(m.md, Ui, Wi, VW * t, best, nullptr, nullptr, nullptr);
+        max_item<MH, VW, SL, false>(m.md, Ui, Wi, VW * t, best, nullptr, nullptr, ctl);
         stv<VW>(Oi + VW * t, best);
 #pragma unroll
         for (int j = 0; j < VW; j++) {
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
         sh_fail = 0;
     }
     __syncthreads();
-    GridBarrier bar{a.arrivals, gridDim.x, 0u, &sh_fail};
+    GridBarrier bar{a.arrivals, gridDim.x, 0u, &sh_fail, a.polls};
     long long k = a.first;
     const long long k_end = k + a.budget;
     long long w0 = 0, w1 = 0;
@@ -229,11 +229,11 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
             if (p - sh_first < kBatchLoopCached) {
                 const LoopInst& d = sh_inst[p - sh_first];
                 share(p, d.md, i0, i1);
-                VC_BY_INST(d, post_share, d, Vi, a.U, a.U2, i0, i1)
+                VC_BY_INST(d, post_share, d, Vi, a.U, a.U2, i0, i1, a.ctl)
             } else {
                 const InstDesc& d = a.descs[id[p]];
                 share(p, d.md, i0, i1);
-                VC_BY_INST(d, post_share, d, Vi, a.U, a.U2, i0, i1)
+                VC_BY_INST(d, post_share, d, Vi, a.U, a.U2, i0, i1, a.ctl)
             }
         }
         if (blockIdx.x == 0)  // this sweep's residual slots, last read two sweeps ago
@@ -247,11 +247,11 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
             if (p - sh_first < kBatchLoopCached) {
                 const LoopInst& d = sh_inst[p - sh_first];
                 share(p, d.md, i0, i1);
-                VC_BY_INST(d, max_share, d, Vi, a.U, a.U2, Vo, i0, i1, res, vabs)
+                VC_BY_INST(d, max_share, d, Vi, a.U, a.U2, Vo, i0, i1, res, vabs, a.ctl)
             } else {
                 const InstDesc& d = a.descs[inst];
                 share(p, d.md, i0, i1);
-                VC_BY_INST(d, max_share, d, Vi, a.U, a.U2, Vo, i0, i1, res, vabs)
+                VC_BY_INST(d, max_share, d, Vi, a.U, a.U2, Vo, i0, i1, res, vabs, a.ctl)
             }
             // non-negative floats order like their bits
             const unsigned int rb = __reduce_max_sync(0xffffffffu, fbits(res));

@@ -169,11 +169,13 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
         m.rr = live ? __ldg(a.R + r) : -INFINITY;
         m.scale = live && a.scale ? __ldg(a.scale + r) : 1.0f;
     };
+    bool gave = false;  // this lane gave up waiting for a chunk
+    uint32_t owed = 0;  // phase at that point, when both buffers' copies were in flight
     auto stage = [&](Meta& m, int b) {
         // lanes past the chunk's rows hold rows of the next one
         m.e0 = __shfl_sync(0xffffffffu, m.lo, 0);
         m.e1 = __shfl_sync(0xffffffffu, m.hi, crows - 1);
-        if (lane != 0) return;
+        if (lane != 0 || gave) return;
         constexpr int kv = 16 / (int)sizeof(VT);
         const int q0 = m.e0 & ~3, p0 = m.e0 & ~(kv - 1);
         uint32_t bc = 4u * (uint32_t)(((m.e1 + 3) & ~3) - q0), bv = (uint32_t)sizeof(VT) * (uint32_t)(((m.e1 + kv - 1) & ~(kv - 1)) - p0);
@@ -189,7 +191,8 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
     long long k = ctl->sweeps;
     const long long k_end = k + budget;
     LoopVerdict verdict{ctl->tol, __double2float_ru(ctl->tol), ctl->best_res, ctl->since_best, ctl->max_sweeps};
-    GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail};
+    GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail, barrier_polls(ctl->spin_limit)};
+    const int lim = (int)barrier_polls(ctl->spin_limit);
     Meta cur, nxt;
     int b = 0, done = 0;
     uint32_t phase = 0;  // parity of each buffer's next chunk (bits 0, 1)
@@ -208,7 +211,15 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
             stage(nxt, b ^ 1);
             Meta after;
             load_meta(c_next + nw < c1 ? c_next + nw : cw, after);
-            if (!mbar_wait(&sh_full[warp][b], (phase >> b) & 1u)) atomicExch(&sh_fail, 1);
+            // A lane that gives up waits no more and goes on with what the buffers hold (columns of an
+            // earlier chunk; the result is refused), and lane 0 then stages no more, so no buffer
+            // is filled while an earlier copy into it is in flight.  The loop is not left here: an
+            // exit inside it cost 3 to 5 % of a sweep.
+            if (!gave && !mbar_wait(&sh_full[warp][b], (phase >> b) & 1u, lim)) {
+                gave = true;
+                owed = phase;
+                atomicExch(&sh_fail, 1);
+            }
             phase ^= 1u << b;
             const unsigned char* src = mine + b * buf_bytes;
             const int32_t* cs = reinterpret_cast<const int32_t*>(src) + (cur.e0 & 3);
@@ -278,7 +289,15 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
         done = verdict(sh_rv[0], sh_rv[1], k);
         if (done || k >= k_end) break;
     }
-    if (any) mbar_wait(&sh_full[warp][b], (phase >> b) & 1u);  // the chunk staged ahead
+    // no copy outlives the CTA: the chunk staged ahead, or both buffers' where lane 0 gave up
+    if (any && lane == 0) {
+        if (gave) {
+            mbar_wait(&sh_full[warp][0], owed & 1u);
+            mbar_wait(&sh_full[warp][1], (owed >> 1) & 1u);
+        } else {
+            mbar_wait(&sh_full[warp][b], (phase >> b) & 1u);
+        }
+    }
     if (lead && sh_fail) atomicOr(&ctl->error, kErrTimeout);
     if (lead && blockIdx.x == 0) {
         ctl->sweeps = k;
@@ -311,10 +330,14 @@ int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_
     *launched = false;
     const bool bf16 = (m->fmt & 0xF) == VC_CSR_BF16;
     // every pipelined CSR schedule (the loop is the faster one at each size and type measured)
-    // whose entries are counted in 31 bits; a handle whose waits were capped keeps the kernel
-    // that reports them
-    if (!m->plan.tma || m->plan.sliced || m->loop_cap <= 0 || m->spin_polls >= 0 ||
-        m->nnz_stored >= (1LL << 31) - 64)
+    // whose entries are counted in 31 bits; a handle whose waits were capped keeps the launched
+    // sweeps (but for the bounds-checking build, where the cap reaches this loop's waits)
+#ifdef VC_DEBUG_BOUNDS
+    const bool capped = false;
+#else
+    const bool capped = m->spin_polls >= 0;
+#endif
+    if (!m->plan.tma || m->plan.sliced || m->loop_cap <= 0 || capped || m->nnz_stored >= (1LL << 31) - 64)
         return VC_OK;
     auto go = [&](auto apad) {
         constexpr int AP = decltype(apad)::value;

@@ -14,6 +14,12 @@ namespace vc {
 
 constexpr unsigned int kBarrierPolls = 1u << 22;  // a few seconds
 
+// Poll limit of a launch's barrier waits from a control block's spin_limit (the handle's cap + 1,
+// 0 without one).
+__host__ __device__ inline unsigned int barrier_polls(long long spin_limit) {
+    return spin_limit > 0 && spin_limit - 1 < (long long)kBarrierPolls ? (unsigned int)(spin_limit - 1) : kBarrierPolls;
+}
+
 // A counter that only grows during a launch (the host clears it before): barrier n is complete
 // once it reaches n x blocks.  Memory written before the barrier by any thread of the
 // grid is visible after it to every thread (thread 0's fences, ordered by the block's own
@@ -21,7 +27,8 @@ constexpr unsigned int kBarrierPolls = 1u << 22;  // a few seconds
 struct GridBarrier {
     unsigned int* count;
     unsigned int blocks, target;
-    int* fail;  // shared: set once a wait gave up
+    int* fail;           // shared: set once a wait gave up
+    unsigned int limit;  // polls of a wait (barrier_polls)
 
     // Call after a __syncthreads that covers the block's writes; thread 0 holds the result
     // until the caller's next __syncthreads.
@@ -33,7 +40,7 @@ struct GridBarrier {
             unsigned int polls = 0;
             do {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            } while (v < target && ++polls < kBarrierPolls);
+            } while (v < target && ++polls < limit);
             if (v < target) *fail = 1;
         }
         __syncthreads();

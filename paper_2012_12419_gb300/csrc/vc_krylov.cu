@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
         sh.fail = 0;
     }
     __syncthreads();
-    GridBarrier bar{&k.kc->arrivals, gridDim.x, 0u, &sh.fail};
+    GridBarrier bar{&k.kc->arrivals, gridDim.x, 0u, &sh.fail, barrier_polls(sh.c.spin_limit)};
     const bool resumed = sh.c.iter > 0;
     const int stop = sh.c.iter + budget;
     bool ok = true;
@@ -594,6 +594,7 @@ int krylov_correct(Mdp* m, const int32_t* pi, const float* b, float* x, double t
     KrylovCtl& h = *m->kctl_host;
     memset(&h, 0, sizeof(KrylovCtl));
     h.target = target;
+    h.spin_limit = m->spin_polls < 0 ? 0 : m->spin_polls + 1;
     h.max_iter = (int)std::min<long long>(std::max<long long>(max_iter, 1), 1 << 30);
     VC_CUDA(cudaMemcpyAsync(m->kctl, &h, sizeof(KrylovCtl), cudaMemcpyHostToDevice, st));
     KrylovArgs k;

@@ -25,6 +25,7 @@ struct KrylovCtl {
     int iter, max_iter;
     unsigned int arrivals;  // grid barrier of the resident kernel: arrivals since the launch
     int fault;              // set by a block whose barrier wait gave up
+    long long spin_limit;   // polls + 1 of a barrier wait (0: the default)
 };
 
 enum KrylovStage : int { kKrInit = 0, kKrV = 1, kKrT = 2, kKrX = 3 };

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         sh_fail = 0;
     }
     __syncthreads();
-    GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail};
+    GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail, barrier_polls(ctl->spin_limit)};
     int done = 0;
     float r = 0.0f, vm = 0.0f;
     while (true) {

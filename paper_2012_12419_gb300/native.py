@@ -295,8 +295,9 @@ class MDP:
         return cls(h)
 
     def set_wait_limit(self, polls: int = -1) -> None:
-        """Cap the bounded shared-memory waits of the pipelined sweeps (fault injection;
-        0 = give up at once, negative = the default)."""
+        """Cap the bounded device waits of this handle's solves: the pipelined sweeps' shared-memory
+        waits and the resident loops' grid barriers (fault injection; 0 = give up at once,
+        negative = the default)."""
         _check(load().vc_set_wait_limit(self._h, int(polls)))
 
     def slice(self, stream=None) -> "MDP":

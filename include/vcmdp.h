@@ -285,6 +285,10 @@ int vc_set_wait_limit(vc_mdp* m, int64_t polls);
  * ([S] int32, nullable) its argmax.  Synchronises `stream`.
  * With VC_ITER_SELF_LOOP the FP32 sweeps use the self-transition-solved backup (see the
  * flag); the policy taken from the FP32 values and everything after it are unchanged.
+ * The FP32 sweeps of an implicit handle or an unsliced pipelined matrix and the correction
+ * solves run in resident kernels that hold the whole device (one SM for instances of at most
+ * 8,192 or 2,048 states): a kernel of another stream starts when such a launch ends, which
+ * it does after about 10 ms, and the next launch follows once that kernel has its SMs.
  * Errors: VC_ERR_NOT_CONVERGED if max_sweeps ran out (outputs still written),
  * VC_ERR_ARG for tol <= 0 or max_sweeps < 1.
  */

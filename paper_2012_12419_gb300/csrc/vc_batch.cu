@@ -1022,7 +1022,7 @@ struct Batch {
     unsigned int *res32 = nullptr, *vmax32 = nullptr;
     unsigned long long* res64 = nullptr;
     long long* iters = nullptr;
-    unsigned int* bar = nullptr;  // the resident loop's barrier counter and fault flag
+    unsigned int* bar = nullptr;  // the resident loop's barrier counter, fault flag and LaunchEnd word
     Ctl* check = nullptr;         // its error flags (bounds-checking build)
     long long spin_polls = -1;    // cap of its barrier waits (-1: the default)
     long long* max_d = nullptr;
@@ -1526,8 +1526,7 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
     VC_CUDA(cudaMemsetAsync(&b->check->error, 0, sizeof(int), st));
 #endif
     a.first = 0;
-    // sweeps of one launch: about a quarter of a second
-    a.budget = (int)std::min<long long>(1 << 20, std::max<long long>(16, (long long)(2e10 / (double)b->padded)));
+    a.end = (long long*)b->bar + 1;
     for (;;) {
         int h[2] = {0, 0};  // active instances, fault
         VC_CUDA(cudaMemsetAsync(b->bar, 0, 8, st));
@@ -1535,6 +1534,7 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
         if (!*resident) return VC_OK;
         VC_CUDA(cudaMemcpyAsync(&h[0], b->active, 4, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaMemcpyAsync(&h[1], a.fault, 4, cudaMemcpyDeviceToHost, st));
+        VC_CUDA(cudaMemcpyAsync(&a.first, a.end, 8, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
         if (h[1]) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
 #ifdef VC_DEBUG_BOUNDS
@@ -1543,7 +1543,6 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
         if (err & kErrBounds) return fail(VC_ERR_CUDA, "a device bounds check failed (bounds-checking build)");
 #endif
         if (h[0] <= 0) return VC_OK;
-        a.first += a.budget;
     }
 }
 

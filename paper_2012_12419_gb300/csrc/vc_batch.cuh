@@ -42,8 +42,9 @@ struct BatchCtl {
     const float* tol_scale;      // per-instance factor on tol (nullptr: 1)
 };
 
-// The FP32 loop of every active instance in one resident kernel (vc_batch_loop.cu): up to a
-// bounded number of sweeps from sweep *first on.  *launched = false when it does not serve
+// The FP32 loop of every active instance in one resident kernel (vc_batch_loop.cu), from sweep
+// `first` on until all have ended or the launch's time is up (LaunchEnd; the sweeps then done
+// are at *end).  *launched = false when it does not serve
 // the batch (hosts, instances) or the device cannot hold the grid.
 struct BatchLoopArgs {
     const InstDesc* descs;
@@ -55,7 +56,7 @@ struct BatchLoopArgs {
     unsigned int polls;       // poll limit of a barrier wait
     Ctl* ctl;                 // error flags of the bounds-checking build
     long long first;          // sweeps done so far
-    int budget;
+    long long* end;           // LaunchEnd's word
 };
 int launch_batch_loop(const BatchLoopArgs& a, int max_hosts, int num_sms, bool self_loop, cudaStream_t st,
                       bool* launched);

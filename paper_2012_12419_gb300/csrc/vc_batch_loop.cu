@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
     float* best = reinterpret_cast<float*>(id + a.n);
     int* since = reinterpret_cast<int*>(best + a.n);
     __shared__ int sh_m, sh_ended, sh_fail, sh_first;
+    __shared__ long long sh_end, sh_start;
     __shared__ LoopInst sh_inst[kBatchLoopCached];  // active instances sh_first ..
     const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
     const bool lead = threadIdx.x == 0;
@@ -138,11 +139,14 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
         sh_m = a.n;
         sh_ended = 1;
         sh_fail = 0;
+        sh_end = a.first + kLaunchSweeps;
     }
     __syncthreads();
     GridBarrier bar{a.arrivals, gridDim.x, 0u, &sh_fail, a.polls};
     long long k = a.first;
-    const long long k_end = k + a.budget;
+    const bool first_cta = lead && blockIdx.x == 0;
+    LaunchEnd end{a.end, &sh_start};
+    if (first_cta) end.open(k);
     long long w0 = 0, w1 = 0;
     int first = 0;
     while (true) {
@@ -213,7 +217,8 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
             __syncthreads();
         }
         const int m = sh_m;
-        if (m == 0 || k >= k_end) break;
+        if (m == 0 || k >= sh_end) break;
+        if (first_cta) end.check(k);
         const int in = (int)(k & 1);
         const float* Vi = in ? a.V1 : a.V0;
         float* Vo = in ? a.V0 : a.V1;
@@ -263,6 +268,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
         }
         if (!bar.sync()) break;
         k++;
+        if (threadIdx.x == blockDim.x - 1) sh_end = end.read();  // beside the verdicts' reads
         for (int p = threadIdx.x; p < m; p += blockDim.x) {
             const int inst = id[p];
             const float r = __uint_as_float(__ldcg(a.c.res32 + 2 * inst + in));
@@ -287,7 +293,10 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
     __syncthreads();
     if (lead && sh_fail) atomicOr(a.fault, 1);
     if (blockIdx.x != 0) return;
-    if (lead) *a.c.active = sh_m;
+    if (lead) {
+        *a.c.active = sh_m;
+        *a.end = k;
+    }
     for (int p = threadIdx.x; p < sh_m; p += blockDim.x) {
         a.c.best_res[id[p]] = best[p];
         a.c.since_best[id[p]] = since[p];

@@ -112,11 +112,11 @@ __device__ __forceinline__ int row_start(const int64_t* row_ptr, int64_t r) {
 
 // APAD: the least power of two >= A (the depth of the tree of maxima).
 template <typename VT, int APAD, bool SL>
-__global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs a, float* buf0, float* buf1, int budget,
-                                                                    Ctl* ctl) {
+__global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs a, float* buf0, float* buf1, Ctl* ctl) {
     extern __shared__ __align__(128) unsigned char csr_sm[];
     __shared__ unsigned int sh_max[2][2];  // residual and max|V'| of the sweep, by parity
     __shared__ float sh_rv[2];
+    __shared__ long long sh_end, sh_start;
     __shared__ int sh_fail, sh_cut[2];
     __shared__ uint64_t sh_full[kCsrLoopWarps][2];  // staged chunks of each warp's two buffers
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
@@ -189,7 +189,9 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
     };
 
     long long k = ctl->sweeps;
-    const long long k_end = k + budget;
+    const bool first_cta = lead && blockIdx.x == 0;
+    LaunchEnd end{&ctl->launch_end, &sh_start};
+    if (first_cta) end.open(k);
     LoopVerdict verdict{ctl->tol, __double2float_ru(ctl->tol), ctl->best_res, ctl->since_best, ctl->max_sweeps};
     GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail, barrier_polls(ctl->spin_limit)};
     const int lim = (int)barrier_polls(ctl->spin_limit);
@@ -206,6 +208,7 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
         const float* Vi = in ? buf1 : buf0;
         float* Vo = in ? buf0 : buf1;
         float res = 0.0f, vabs = 0.0f;
+        if (first_cta) end.check(k);
         for (int c = cw; c < c1; c += nw) {
             const int c_next = c + nw < c1 ? c + nw : cw;
             stage(nxt, b ^ 1);
@@ -278,16 +281,17 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
         if (lead) {
             sh_rv[0] = __uint_as_float(*((volatile unsigned int*)&ctl->res32[slot]));
             sh_rv[1] = __uint_as_float(*((volatile unsigned int*)&ctl->vmax32[slot]));
-            if (blockIdx.x == 0) {
+            if (first_cta) {
                 // the slot after the next sweep's: read 62 sweeps ago, written after the next barrier
                 ctl->res32[(k + 2) % kRing] = 0u;
                 ctl->vmax32[(k + 2) % kRing] = 0u;
             }
         }
+        if (threadIdx.x == blockDim.x - 1) sh_end = end.read();  // beside the lead's two reads
         __syncthreads();
         k++;
         done = verdict(sh_rv[0], sh_rv[1], k);
-        if (done || k >= k_end) break;
+        if (done || k >= sh_end) break;
     }
     // no copy outlives the CTA: the chunk staged ahead, or both buffers' where lane 0 gave up
     if (any && lane == 0) {
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
         }
     }
     if (lead && sh_fail) atomicOr(&ctl->error, kErrTimeout);
-    if (lead && blockIdx.x == 0) {
+    if (first_cta) {
         ctl->sweeps = k;
         ctl->final_buf = (int)(k & 1);
         ctl->best_res = verdict.best;
@@ -318,12 +322,10 @@ static int csr_loop_run(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStr
     const int chunks = (m->S + 32 / m->A - 1) / (32 / m->A);
     const int sms = m->num_sms > 0 ? m->num_sms : 148;
     const int grid = std::min(sms, (chunks + 3) / 4);
-    // sweeps of one launch: about a quarter of a second at 20 ps an entry
-    const int budget = (int)std::min<long long>(1 << 20, std::max<long long>(16, (long long)(1e10 / (double)(m->nnz_stored + 64LL * m->S))));
     const CsrLoopArgs a{m->S, m->A, (int)m->loop_cap, (float)m->gamma, m->row_ptr, m->col, m->val, m->scale, m->R};
     const void* fn = self_loop ? (const void*)k_csr_loop<VT, APAD, true> : (const void*)k_csr_loop<VT, APAD, false>;
     VC_CUDA(cached_set_max_dyn_smem(fn, kCsrLoopSmem));
-    return launch_resident(fn, grid, 32 * warps, (size_t)warps * warp_bytes, st, launched, a, buf0, buf1, budget, m->ctl);
+    return launch_resident(fn, grid, 32 * warps, (size_t)warps * warp_bytes, st, launched, a, buf0, buf1, m->ctl);
 }
 
 int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {

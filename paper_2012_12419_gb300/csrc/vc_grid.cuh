@@ -52,6 +52,34 @@ struct GridBarrier {
     }
 };
 
+// A resident launch holds every SM, so kernels of other streams wait for its end: it ends itself
+// after about 10 ms (20 M cycles at 2 GHz, a tenth of the 100 ms synchronisation interval; the
+// host reads the control block and goes on with another launch, 50 to 130 us with the kernel's
+// start: at 4 ms a 48-instance batch took 2.7 % longer), at a sweep that all CTAs take from one
+// word.  CTA 0 writes it two
+// sweeps ahead: whoever still reads for the sweep before finds a number that it has not
+// reached, and everyone has it after the next barrier.  Whole solves on one launch held the
+// device for up to 0.25 s.
+constexpr long long kLaunchCycles = 20'000'000;
+constexpr long long kLaunchSweeps = 1 << 20;
+
+struct LaunchEnd {
+    long long* end;    // the control block's word
+    long long* start;  // shared: clock64() at the launch (a register pair in every thread cost the
+                       // stored-matrix loop 2 %)
+    // Thread 0 of CTA 0, before its first barrier.
+    __device__ __forceinline__ void open(long long k) {
+        *start = clock64();
+        *((volatile long long*)end) = k + kLaunchSweeps;
+    }
+    // The same thread at the start of sweep k (0-based).
+    __device__ __forceinline__ void check(long long k) {
+        if (clock64() - *start > kLaunchCycles && *((volatile long long*)end) > k + 2)
+            *((volatile long long*)end) = k + 2;
+    }
+    __device__ __forceinline__ long long read() const { return *((volatile long long*)end); }
+};
+
 // Step 3's test on every thread of a CTA from the sweep's residual r and max|V'| vm:
 // finish_block's decision, in the same order.  4 ulp(vm) is a power of two, so for vm
 // above 2^-100 both sides of r < max(tol, 4 ulp) are compared in FP32 exactly (tol rounded

@@ -259,7 +259,8 @@ struct Ctl {
     unsigned long long cert64;          // FP64 residual bits of a standalone Bellman backup
     int error;                          // bit flags raised by kernels (infeasible policy, bad input)
     unsigned int arrivals;              // grid barrier of the loop kernel: arrivals since the launch
-    long long spin_limit;               // polls + 1 of each bounded pipeline wait (0 = the default)
+    long long spin_limit;               // polls + 1 of each bounded wait (0 = the default)
+    long long launch_end;               // sweeps at which the resident loop's launch ends (LaunchEnd)
 };
 
 // Error flags raised on the device.

@@ -163,6 +163,7 @@ struct KrShared {
     float dot[2][kKrThreads / 32][DotSum::kWords];  // the warps' sums
     unsigned int mx;                       // bits of the CTA's max |r|
     double tot[2];
+    long long end, start;                  // iterations at which this launch ends, its first cycle
     int fail;
 };
 
@@ -170,7 +171,7 @@ struct KrShared {
 // wait gave up.  D1, MX: whether the stage has a second dot product, a maximum.
 template <bool D1, bool MX>
 __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, GridBarrier& bar, int stage, DotSum a0,
-                                          DotSum a1, float mx) {
+                                          DotSum a1, float mx, const LaunchEnd* end = nullptr) {
     const int w = (int)threadIdx.x >> 5, l = (int)threadIdx.x & 31, nw = (int)blockDim.x >> 5;
     // lanes 0..15 add up the first product, 16..31 the second (without one, the first again)
     static_assert(kKrThreads / 32 <= 16, "a half-warp adds up the warps' sums");
@@ -235,6 +236,7 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
         if (l == 0) {
             kr_advance(&sh.c, stage, v0, v1, (double)__uint_as_float(vm));
             if (MX) sh.mx = 0u;  // next written after the caller's barriers
+            if (end) sh.end = end->read();
         }
     }
     __syncthreads();
@@ -386,7 +388,7 @@ struct AdjProduct {
 
 // ---------------------------------------------------------------------------- kernel
 template <typename Op>
-__global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, int budget) {
+__global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k) {
     constexpr int VW = Op::kWidth;
     __shared__ KrShared sh;
     const int n = k.n, chains = k.chains, step = (int)blockDim.x;
@@ -401,11 +403,14 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
         sh.c = *k.kc;
         sh.mx = 0u;
         sh.fail = 0;
+        sh.end = sh.c.iter + kLaunchSweeps;
     }
     __syncthreads();
     GridBarrier bar{&k.kc->arrivals, gridDim.x, 0u, &sh.fail, barrier_polls(sh.c.spin_limit)};
     const bool resumed = sh.c.iter > 0;
-    const int stop = sh.c.iter + budget;
+    const bool first_cta = threadIdx.x == 0 && blockIdx.x == 0;
+    LaunchEnd end{&k.kc->launch_end, &sh.start};
+    if (first_cta) end.open(sh.c.iter);
     bool ok = true;
     if (!resumed) {
         // r = b, x = 0, with <b, b> and max |b|
@@ -460,7 +465,8 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
         return second ? kr_reduce<true, false>(k, sh, bar, kKrT, a0, a1, 0.0f)
                       : kr_reduce<false, false>(k, sh, bar, kKrV, a0, a1, 0.0f);
     };
-    while (ok && !sh.c.done && sh.c.iter < stop) {
+    while (ok && !sh.c.done && sh.c.iter < sh.end) {
+        if (first_cta) end.check(sh.c.iter);
         // p = r (first iteration), else p = r + beta (p - omega v)
         const bool first = sh.c.iter == 0;
         const float beta = (float)sh.c.beta, omega0 = (float)sh.c.omega;
@@ -515,7 +521,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
 #pragma unroll
             for (int j = 0; j < VW; j++) a0.add(d0[j]);
         }
-        ok = kr_reduce<false, true>(k, sh, bar, kKrX, a0, DotSum(), mx);
+        ok = kr_reduce<false, true>(k, sh, bar, kKrX, a0, DotSum(), mx, &end);
     }
     if (threadIdx.x != 0) return;
     if (sh.fail) atomicOr(&k.kc->fault, 1);
@@ -535,7 +541,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k, i
 // Enqueues one launch.  The grid is at most one CTA per SM; where the device cannot hold it
 // at once (a partitioned GPU) it is halved until it can.
 template <typename Op>
-static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budget, cudaStream_t st) {
+static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, cudaStream_t st) {
     const int sms = m->num_sms > 0 ? m->num_sms : 148;
     const int items = std::min(k.n, k.chains) / Op::kWidth;
     int grid = k.n <= kKrOneCta ? 1 : std::max(1, std::min(sms, items / kKrItems));
@@ -544,7 +550,7 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budge
         const int threads = std::min(kKrThreads, std::max(32, (per + 31) / 32 * 32));
         bool launched = false;
         const int rc = launch_resident((const void*)k_krylov<Op>, (items + per - 1) / per, threads, 0, st, &launched,
-                                       op, k, budget);
+                                       op, k);
         if (rc || launched) return rc;
         if (grid == 1) return fail(VC_ERR_CUDA, "the correction solve's kernel does not fit the device");
     }
@@ -555,23 +561,23 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, int budge
 // 2.01 / 1.66, 524,288 3.58 / 2.72; items of two states (Q even): 343,750 2.77 / 2.35.
 constexpr int kKrTwoPass = 120000;
 
-static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, int budget, cudaStream_t st) {
-    if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, budget, st);
+static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, cudaStream_t st) {
+    if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, st);
     if (!m->has_model) {
         if ((m->fmt & 0xF) == VC_CSR_BF16) {
             RowProduct<uint16_t> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const uint16_t*)m->val, m->scale, pi};
-            return krylov_run(m, op, k, budget, st);
+            return krylov_run(m, op, k, st);
         }
         RowProduct<float> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const float*)m->val, m->scale, pi};
-        return krylov_run(m, op, k, budget, st);
+        return krylov_run(m, op, k, st);
     }
     const bool two = m->S >= kKrTwoPass;
     auto go = [&](auto mh) -> int {
         constexpr int MH = decltype(mh)::value;
         if (two && MH <= 8 && wide_rows(m->md))
-            return krylov_run(m, ModelProduct2<MH, MH <= 8 ? 4 : 2>{m->md, m->c32, pi}, k, budget, st);
-        if (two) return krylov_run(m, ModelProduct2<MH, 2>{m->md, m->c32, pi}, k, budget, st);
-        return krylov_run(m, ModelProduct<MH>{m->md, m->c32, pi}, k, budget, st);
+            return krylov_run(m, ModelProduct2<MH, MH <= 8 ? 4 : 2>{m->md, m->c32, pi}, k, st);
+        if (two) return krylov_run(m, ModelProduct2<MH, 2>{m->md, m->c32, pi}, k, st);
+        return krylov_run(m, ModelProduct<MH>{m->md, m->c32, pi}, k, st);
     };
     switch (m->md.H) {
         case 1: return go(std::integral_constant<int, 1>());
@@ -612,11 +618,9 @@ int krylov_correct(Mdp* m, const int32_t* pi, const float* b, float* x, double t
     k.post = m->post;
     k.n = m->S;
     k.chains = state_grid(m) * kThreads;
-    // iterations of one launch: about a quarter of a second
-    const int budget = (int)std::min<long long>(1 << 20, std::max<long long>(4, (long long)(1e10 / m->S)));
     int rc;
     for (;;) {
-        if ((rc = krylov_launch(m, pi, k, budget, st))) return rc;
+        if ((rc = krylov_launch(m, pi, k, st))) return rc;
         VC_CUDA(cudaMemcpyAsync(&h, m->kctl, sizeof(KrylovCtl), cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
         if (h.fault) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");

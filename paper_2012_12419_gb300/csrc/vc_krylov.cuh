@@ -26,6 +26,7 @@ struct KrylovCtl {
     unsigned int arrivals;  // grid barrier of the resident kernel: arrivals since the launch
     int fault;              // set by a block whose barrier wait gave up
     long long spin_limit;   // polls + 1 of a barrier wait (0: the default)
+    long long launch_end;   // iterations at which the launch ends (LaunchEnd)
 };
 
 enum KrylovStage : int { kKrInit = 0, kKrV = 1, kKrT = 2, kKrX = 3 };

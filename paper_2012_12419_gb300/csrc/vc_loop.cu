@@ -37,17 +37,19 @@ constexpr int kLoopItems = 256;    // least items of a CTA of the multi-CTA loop
 // are the handle's buffers and V the caller's pair.
 template <int MH, int VW, bool SL, bool SMEM>
 __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<float> c, float* buf0, float* buf1,
-                                                             float* U, float* W, int budget, Ctl* ctl) {
+                                                             float* U, float* W, Ctl* ctl) {
     extern __shared__ __align__(16) float loop_sm[];
     __shared__ unsigned int sh_max[2][2];  // residual and max|V'| of the sweep, by parity
     __shared__ float sh_rv[2];
     __shared__ int sh_fail;
+    __shared__ long long sh_end, sh_start;
     const int items = md.S / VW;
     const int per = (items + (int)gridDim.x - 1) / (int)gridDim.x;
     const int t0 = (int)blockIdx.x * per, t1 = min(items, t0 + per);
     const bool lead = threadIdx.x == 0;
     long long k = ctl->sweeps;
-    const long long k_end = k + budget;
+    const bool first = lead && blockIdx.x == 0;
+    LaunchEnd end{SMEM ? &sh_end : &ctl->launch_end, &sh_start};
     LoopVerdict verdict{ctl->tol, __double2float_ru(ctl->tol), ctl->best_res, ctl->since_best, ctl->max_sweeps};
     float* V[2] = {buf0, buf1};
     if constexpr (SMEM) {
@@ -62,6 +64,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         sh_max[0][0] = sh_max[0][1] = sh_max[1][0] = sh_max[1][1] = 0u;
         sh_fail = 0;
     }
+    if (first) end.open(k);
     __syncthreads();
     GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail, barrier_polls(ctl->spin_limit)};
     int done = 0;
@@ -70,13 +73,14 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         const int in = (int)(k & 1);
         const float* Vi = V[in];
         float* Vo = V[in ^ 1];
+        if (first) end.check(k);
         for (int t = t0 + (int)threadIdx.x; t < t1; t += (int)blockDim.x)
             post_item<MH, VW, SL>(md, c, Vi, VW * t, U, W, ctl);
         if constexpr (SMEM) {
             __syncthreads();
         } else {
             // the next sweep's slot: last read 63 sweeps ago, first written after two barriers
-            if (lead && blockIdx.x == 0) {
+            if (first) {
                 ctl->res32[(k + 1) % kRing] = 0u;
                 ctl->vmax32[(k + 1) % kRing] = 0u;
             }
@@ -118,13 +122,14 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
                 sh_rv[0] = __uint_as_float(*((volatile unsigned int*)&ctl->res32[slot]));
                 sh_rv[1] = __uint_as_float(*((volatile unsigned int*)&ctl->vmax32[slot]));
             }
+            if (threadIdx.x == blockDim.x - 1) sh_end = end.read();  // beside the lead's two reads
             __syncthreads();
             r = sh_rv[0];
             vm = sh_rv[1];
         }
         k++;
         done = verdict(r, vm, k);
-        if (done || k >= k_end) break;
+        if (done || k >= *((volatile long long*)&sh_end)) break;
     }
     if constexpr (SMEM) {
         __syncthreads();
@@ -136,7 +141,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         }
     }
     if (lead && sh_fail) atomicOr(&ctl->error, kErrTimeout);
-    if (lead && blockIdx.x == 0) {
+    if (first) {
         ctl->sweeps = k;
         ctl->final_buf = (int)(k & 1);
         ctl->best_res = verdict.best;
@@ -164,8 +169,6 @@ static int loop_threads(int per) {
 template <int MH, int VW, bool SL>
 static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, bool* launched) {
     const int items = m->S / VW;
-    // sweeps of one launch: about a quarter of a second
-    const int budget = (int)std::min<long long>(1 << 20, std::max<long long>(16, (long long)(2.5e10 / m->S)));
     float* U = m->U32 + kUShift;
     const size_t smem = 4 * ((size_t)(SL ? 4 : 3) * m->S + kUPad);
     *launched = true;
@@ -173,7 +176,7 @@ static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, bool* 
         auto kern = k_vi_loop<MH, VW, SL, true>;
         VC_CUDA(cached_set_max_dyn_smem((const void*)kern, 4 * (4 * kLoopOneCta + kUPad)));
         count_launches(1);
-        kern<<<1, loop_threads(items), smem, st>>>(m->md, m->c32, buf0, buf1, U, m->U32s, budget, m->ctl);
+        kern<<<1, loop_threads(items), smem, st>>>(m->md, m->c32, buf0, buf1, U, m->U32s, m->ctl);
         VC_CUDA(cudaGetLastError());
         return VC_OK;
     }
@@ -182,7 +185,7 @@ static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, bool* 
     const int grid = std::min(sms, (items + kLoopItems - 1) / kLoopItems);
     const int per = (items + grid - 1) / grid;
     return launch_resident((const void*)kern, (items + per - 1) / per, loop_threads(per), 0, st, launched, m->md, m->c32, buf0,
-                           buf1, U, m->U32s, budget, m->ctl);
+                           buf1, U, m->U32s, m->ctl);
 }
 
 int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {

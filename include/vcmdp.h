@@ -521,7 +521,8 @@ int vc_batch_offsets(const vc_batch* b, int64_t* offsets);
 
 /*
  * Value iteration of every instance (Algorithm 3), each with its own gamma, tolerance test
- * (max(tol, 4 ulp(max|V_i|)) or FP32 stall) and sweep count, in one graph launch; then,
+ * (max(tol, 4 ulp(max|V_i|)) or FP32 stall) and sweep count, in a resident kernel (launches of
+ * about 10 ms, see vc_value_iterate) or, beyond its limits, one graph launch; then,
  * unless VC_ITER_FP32_ONLY, every instance's argmax policy is evaluated by FP64 residual +
  * FP32 correction (BiCGSTAB for every instance in one graph launch; fixed-point sweeps with
  * VC_ITER_PLAIN_CORRECTION or if an instance breaks down) + FP64 update and certified by
@@ -540,14 +541,17 @@ int vc_value_iterate_batch(vc_batch* b, float* V, double* V64_out, int32_t* pi_o
 
 /*
  * Instances solved whole inside one thread block (no paper counterpart; Algorithm 4's block
- * taken as the whole instance): before the FP32 graph loop, each instance with S <=
- * max_states (capped by the device's shared memory: 16 bytes per state for the iterate pair
- * and the pass-1 values; the default is that cap, about 14,000 states on GB300) is swept in
- * one CTA with its values in shared memory and its own step-3 test after every sweep --
- * the loop's arithmetic, so the iterate and the sweep count are the loop's bit for bit --
- * and the loop skips it.  With VC_ITER_BLOCK such an instance is one block iterated by the
- * self-transition sweeps to its test.  0 disables the path.  Synchronises `stream`.
- * VC_ERR_ARG for max_states < 0.
+ * taken as the whole instance): an instance with S <= max_states (capped by the device's
+ * shared memory: 16 bytes per state for the iterate pair and the pass-1 values; the default
+ * is that cap, about 14,000 states on GB300) may be swept in one CTA with its values in
+ * shared memory and its own step-3 test after every sweep -- the loop's arithmetic, so the
+ * iterate and the sweep count are the loop's bit for bit.  Where the resident loop serves the
+ * batch (at most 5 hosts and 4,096 instances, no VC_ITER_BLOCK) they are all swept so if every
+ * instance is such a one; else the loop sweeps all instances and leaves those of at most
+ * 4,096 states to this path once no larger one is active.  Where the graph loop runs, they
+ * are swept beside it and it skips them.  With VC_ITER_BLOCK such an instance is one block
+ * iterated by the self-transition sweeps to its test.  0 disables the path.  Synchronises
+ * `stream`.  VC_ERR_ARG for max_states < 0.
  */
 int vc_batch_set_small_instances(vc_batch* b, int32_t max_states, void* stream);
 

@@ -523,12 +523,15 @@ __global__ void __launch_bounds__(1024) k_bblock(const InstDesc* __restrict__ de
 // loop's active count leaves them out).
 template <int MH, bool SL>
 __global__ void __launch_bounds__(512) k_bsmall(const InstDesc* __restrict__ descs, const int* __restrict__ list,
-                                                 int nlist, BatchCtl c, float* __restrict__ Va) {
+                                                 int nlist, BatchCtl c, float* __restrict__ Va,
+                                                 const float* __restrict__ Vb, long long first) {
     extern __shared__ float sm_small[];
     __shared__ InstDesc sd;
     __shared__ int sh_done;
     for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
         const int inst = list[li];
+        // first >= 0: the instances that the resident loop left after `first` sweeps go on
+        if (first >= 0 && c.done[inst] != 0) continue;
         load_desc(descs, inst, sd);
         __syncthreads();
         const int S = sd.S;
@@ -537,12 +540,13 @@ __global__ void __launch_bounds__(512) k_bsmall(const InstDesc* __restrict__ des
         float* Us = sm_small + 2 * S;  // pass-1 values
         float* Ws = sm_small + 3 * S;  // defer's self-transition-solved values (SL)
         float* Vg = Va + sd.off;
-        for (int j = threadIdx.x; j < S; j += blockDim.x) Vc[j] = Vg[j];
+        const float* Vs = (first > 0 && (first & 1)) ? Vb + sd.off : Vg;
+        for (int j = threadIdx.x; j < S; j += blockDim.x) Vc[j] = Vs[j];
         const double tol = *c.tol * (c.tol_scale ? (double)c.tol_scale[inst] : 1.0);
         const long long max_sweeps = *c.max_sweeps;
-        float best_res = INFINITY;
-        int since_best = 0;
-        long long k = 0;
+        float best_res = first >= 0 ? c.best_res[inst] : INFINITY;
+        int since_best = first >= 0 ? c.since_best[inst] : 0;
+        long long k = first >= 0 ? first : 0;
         if (threadIdx.x == 0) sh_done = 0;
         __syncthreads();
         while (true) {
@@ -1241,6 +1245,11 @@ static int build_block_tiles(Batch* b, cudaStream_t st) {
     return VC_OK;
 }
 
+// Largest instance that the resident loop leaves to the whole-instance kernel once no larger one is
+// active: a step of the loop takes 5 to 6 us however few states are left, a sweep of k_bsmall 1.9
+// us at 600 states, 4.0 at 2,560 and 9.0 at 8,192 (100 instances).
+constexpr int kHandOver = 4096;
+
 // List of the instances solved whole in one CTA (S <= small_max), grouped into size
 // classes and uploaded for k_bsmall.
 static int build_small_list(Batch* b, cudaStream_t st) {
@@ -1272,24 +1281,28 @@ static int build_small_list(Batch* b, cudaStream_t st) {
 
 // Starts the whole-instance solves (Eq. 18's backup, or the self-transition solve: SL,
 // which the in-block iteration uses for a whole-instance block): flags them for the loop
-// on `st`, then one launch per size class on its side stream, forked from `st`.
+// on `st`, then one launch per size class on its side stream, forked from `st`.  first >= 0:
+// takes over the instances that the resident loop left after that many sweeps.
 template <int MH>
-static int launch_small(Batch* b, bool sl, cudaStream_t st) {
+static int launch_small(Batch* b, bool sl, cudaStream_t st, long long first = -1) {
     if (b->n_small == 0) return VC_OK;
-    count_launches(1);
-    k_bmark_small<<<(b->n_small + 255) / 256, 256, 0, st>>>(b->done, b->d_small, b->n_small);
-    VC_LAUNCHED("k_bmark_small");
+    if (first < 0) {
+        count_launches(1);
+        k_bmark_small<<<(b->n_small + 255) / 256, 256, 0, st>>>(b->done, b->d_small, b->n_small);
+        VC_LAUNCHED("k_bmark_small");
+    }
     VC_CUDA(cudaEventRecord(b->fork_ev, st));
     auto kern = sl ? k_bsmall<MH, true> : k_bsmall<MH, false>;
     for (int c = 0; c < Batch::kSmallClasses; c++) {
         if (b->cls_count[c] == 0) continue;
+        if (first >= 0 && (b->small_cap >> (Batch::kSmallClasses - c)) >= kHandOver) break;  // none of this class is left
         const size_t smem = 16 * (size_t)b->cls_S[c];
         const int threads = b->cls_S[c] <= 2048 ? 128 : b->cls_S[c] <= 4096 ? 256 : 512;
         VC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         VC_CUDA(cudaStreamWaitEvent(b->side[c], b->fork_ev, 0));
         count_launches(1);
         kern<<<b->cls_count[c], threads, smem, b->side[c]>>>(b->d_desc, b->d_small + b->cls_first[c],
-                                                              b->cls_count[c], ctl_of(b), b->Va);
+                                                              b->cls_count[c], ctl_of(b), b->Va, b->Vb, first);
         VC_LAUNCHED("the whole-instance kernel");
         VC_CUDA(cudaEventRecord(b->join_ev[c], b->side[c]));
     }
@@ -1501,13 +1514,45 @@ static int reset_loop(Batch* b, double tol, long long max_sweeps, cudaStream_t s
     return VC_OK;
 }
 
+// Whether the graph beside the whole-instance kernel is the faster way through the FP32 loop: it
+// hides few quick large instances behind many slow small ones, which the resident loop can
+// only take one after the other.  Sweeps go as 1 / (1 - gamma); microseconds of a sweep: whole
+// instances 1 + S / 1000 or 7 ps a state over all, the graph 9 + 16 ps a state (and the two, which
+// share the SMs, 0.4 of the shorter), the resident loop 5.5 + 4 ps; the hand-over 0.1 ms.  Measured,
+// graph / resident, small instances beside one of 50,000 states (discount 0.9): 300 of 600 states
+// (0.99) 4.3 / 4.7 ms (9.0 without the hand-over), at 0.95 2.7 / 1.7; 300 of 2,560 9.3 / 9.9 and
+// 3.5 / 2.6; 100 of 2,560 7.5 / 7.5 and 2.6 / 2.0; 300 of 8,192 29.9 / 19.7 and 7.5 / 4.8.
+static bool graph_faster(const Batch* b) {
+    struct Group {
+        double sweeps = 0, largest = 0, states = 0;
+        void add(double n, double S) {
+            sweeps = std::max(sweeps, n);
+            largest = std::max(largest, S);
+            states += S;
+        }
+        double whole() const { return states > 0 ? std::max(1.0 + largest / 1000.0, states * 7e-6) : 0.0; }
+    } one, rest, left, large;  // the graph's two groups, the resident loop's two
+    const int hand = std::min(kHandOver, b->small_max);
+    for (const InstDesc& d : b->h_desc) {
+        const double n = 1.0 / (1.0 - d.c64.gamma);
+        (d.S <= b->small_max ? one : rest).add(n, d.S);
+        (d.S <= hand ? left : large).add(n, d.S);
+    }
+    const double g1 = one.sweeps * one.whole(), g2 = rest.sweeps * (9.0 + rest.states * 16e-6);
+    const double graph = std::max(g1, g2) + 0.4 * std::min(g1, g2);
+    double resident = large.sweeps * (5.5 + (double)b->total * 4e-6);
+    if (left.sweeps > large.sweeps) resident += 7.0 + (left.sweeps - large.sweeps) * left.whole();
+    return graph < resident;
+}
+
 // The FP32 loop by vc_batch_loop.cu.  Its instances advance in step, one grid barrier after each
-// pass, so the small ones ride along (a few percent of the work) and the side streams of
-// the whole-instance path stay empty; a batch of small instances only, which needs no
-// barrier, keeps that path, and the in-block iteration keeps its graph.
+// pass, so the small ones ride along while a large one is active; those that outlast it go on
+// in the whole-instance path (kHandOver), with the sweeps and the stall test where they stand.  A
+// batch of small instances only, which needs no barrier, keeps that path from the start, and the
+// in-block iteration keeps its graph.
 static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, cudaStream_t st, bool* resident) {
     *resident = false;
-    if ((flags & VC_ITER_BLOCK) || b->n_small == b->n) return VC_OK;
+    if ((flags & VC_ITER_BLOCK) || b->n_small == b->n || graph_faster(b)) return VC_OK;
     int rc = reset_loop(b, tol, max_sweeps, st);
     if (rc) return rc;
     BatchLoopArgs a;
@@ -1527,6 +1572,7 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
 #endif
     a.first = 0;
     a.end = (long long*)b->bar + 1;
+    a.hand_over = std::min(kHandOver, b->small_max);
     for (;;) {
         int h[2] = {0, 0};  // active instances, fault
         VC_CUDA(cudaMemsetAsync(b->bar, 0, 8, st));
@@ -1536,13 +1582,18 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
         VC_CUDA(cudaMemcpyAsync(&h[1], a.fault, 4, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaMemcpyAsync(&a.first, a.end, 8, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
-        if (h[1]) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
+        if (h[1] & kLoopTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
 #ifdef VC_DEBUG_BOUNDS
         int err = 0;
         VC_CUDA(cudaMemcpy(&err, &b->check->error, sizeof(int), cudaMemcpyDeviceToHost));
         if (err & kErrBounds) return fail(VC_ERR_CUDA, "a device bounds check failed (bounds-checking build)");
 #endif
         if (h[0] <= 0) return VC_OK;
+        if (h[1] & kLoopHandOver) {
+            const bool sl = (flags & VC_ITER_SELF_LOOP) != 0;
+            by_mh(b->mh, [&](auto m) { rc = launch_small<decltype(m)::value>(b, sl, st, a.first); });
+            return rc ? rc : join_small(b, st);
+        }
     }
 }
 

@@ -43,16 +43,18 @@ struct BatchCtl {
 };
 
 // The FP32 loop of every active instance in one resident kernel (vc_batch_loop.cu), from sweep
-// `first` on until all have ended or the launch's time is up (LaunchEnd; the sweeps then done
-// are at *end).  *launched = false when it does not serve
+// `first` on until all have ended, only instances of at most hand_over states are left or the
+// launch's time is up (LaunchEnd); the sweeps then done are at *end.  *launched = false when it does not serve
 // the batch (hosts, instances) or the device cannot hold the grid.
+constexpr int kLoopTimeout = 1, kLoopHandOver = 2;
 struct BatchLoopArgs {
     const InstDesc* descs;
     int n;
     BatchCtl c;
     float *V0, *V1, *U, *U2;  // U: kUShift past a 16-byte-aligned buffer
     unsigned int* arrivals;   // grid barrier, cleared by the host before each launch
-    int* fault;               // set by a block whose barrier wait gave up
+    int* fault;               // kLoopTimeout: a barrier wait gave up; kLoopHandOver: small ones are left
+    int hand_over;
     unsigned int polls;       // poll limit of a barrier wait
     Ctl* ctl;                 // error flags of the bounds-checking build
     long long first;          // sweeps done so far

@@ -8,6 +8,8 @@
 // an instance ends.  A warp takes each instance's coefficients into registers once per pass
 // and runs the items of vc_implicit.cuh for the instance's exact host count.  After the
 // second barrier every CTA takes step 3's decision for every instance itself.
+// Once only small instances are left, with many sweeps to go, the loop leaves them to the
+// whole-instance kernel (kHandOver in vc_batch.cu).
 //
 // Bound: L2 (DRAM while more than ~10 M states are active) latency of the items' loads at 16
 // warps an SM, and the slower SMs' tail at the two barriers.  Whole solves against the graph of
@@ -25,6 +27,8 @@ namespace vc {
 constexpr int kBatchLoopThreads = 512;  // 640 and 768: spills, 48 instances 10.0 -> 11.4 and 14 ms
 constexpr int kBatchLoopMaxH = 5;      // above, an item and its coefficients no longer fit 128 registers
 constexpr int kBatchLoopMaxN = 4096;   // instances whose shares and verdicts fit shared memory
+// Sweeps for which the hand-over (four launches, two host calls: 0.1 ms) pays at 2 to 4 us a sweep.
+constexpr int kHandOverSweeps = 64;
 
 // Relative cost of an item (a decode and, per host, its loads and arithmetic).
 __host__ __device__ inline int item_cost(int H, bool wide) { return 40 + (wide ? 40 : 26) * H; }
@@ -122,7 +126,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
     int* id = reinterpret_cast<int*>(start + a.n + 1);
     float* best = reinterpret_cast<float*>(id + a.n);
     int* since = reinterpret_cast<int*>(best + a.n);
-    __shared__ int sh_m, sh_ended, sh_fail, sh_first;
+    __shared__ int sh_m, sh_ended, sh_fail, sh_first, sh_small;
     __shared__ long long sh_end, sh_start;
     __shared__ LoopInst sh_inst[kBatchLoopCached];  // active instances sh_first ..
     const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
@@ -155,7 +159,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
         if (recut) {
             // the instances still active, in order, and the work before each (warp 0)
             if (warp == 0) {
-                int m = 0;
+                int m = 0, largest = 0;
                 long long total = 0;
                 for (int i0 = 0; i0 < sh_m; i0 += 32) {
                     const int i = i0 + lane;
@@ -164,6 +168,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
                     const int sb = inst >= 0 ? since[i] : 0;
                     long long work = 0;
                     if (inst >= 0) {
+                        largest = max(largest, a.descs[inst].S);
                         const bool wide = wide_inst(a.descs[inst].md);
                         work = (long long)(a.descs[inst].S / (wide ? 4 : 2)) * item_cost(a.descs[inst].md.H, wide);
                     }
@@ -186,10 +191,26 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
                     total += __shfl_sync(0xffffffffu, incl, 31);
                     __syncwarp();
                 }
+                largest = __reduce_max_sync(0xffffffffu, largest);
+                bool leave = m > 0 && largest <= a.hand_over;
+                if (leave) {
+                    // sweeps still needed, from the last sweep's residuals (-1: none was made) and each
+                    // instance's contraction; every CTA reads the same words
+                    float left = 0.0f;
+                    for (int p = lane; p < m; p += 32) {
+                        const int slot = 2 * id[p] + (int)((k - 1) & 1);
+                        const float r = __uint_as_float(__ldcg(a.c.res32 + slot));
+                        const float vm = __uint_as_float(__ldcg(a.c.vmax32 + slot));
+                        const float t = fmaxf((float)(tol * (a.c.tol_scale ? (double)a.c.tol_scale[id[p]] : 1.0)), vm * 0x1p-21f);
+                        left = fmaxf(left, k == 0 ? INFINITY : logf(r / t) / -logf(a.descs[id[p]].c32.gamma));
+                    }
+                    leave = __any_sync(0xffffffffu, left > (float)kHandOverSweeps);
+                }
                 if (lane == 0) {
                     start[m] = total;
                     sh_m = m;
                     sh_ended = 0;
+                    sh_small = leave;
                 }
             }
             __syncthreads();
@@ -217,7 +238,7 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
             __syncthreads();
         }
         const int m = sh_m;
-        if (m == 0 || k >= sh_end) break;
+        if (m == 0 || k >= sh_end || sh_small) break;
         if (first_cta) end.check(k);
         const int in = (int)(k & 1);
         const float* Vi = in ? a.V1 : a.V0;
@@ -291,11 +312,12 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
         __syncthreads();
     }
     __syncthreads();
-    if (lead && sh_fail) atomicOr(a.fault, 1);
+    if (lead && sh_fail) atomicOr(a.fault, kLoopTimeout);
     if (blockIdx.x != 0) return;
     if (lead) {
         *a.c.active = sh_m;
         *a.end = k;
+        if (sh_small) atomicOr(a.fault, kLoopHandOver);
     }
     for (int p = threadIdx.x; p < sh_m; p += blockDim.x) {
         a.c.best_res[id[p]] = best[p];

@@ -408,9 +408,11 @@ int vc_evaluate_policy(vc_mdp* m, const int32_t* pi, double* V_pi, double tol, i
  * Autotuner of the CSR sweep schedule: times every feasible shared-memory tiling (states
  * per tile, pipeline stages, CTAs per SM), the direct-load kernel and, when the handle
  * has a sliced copy, the sliced sweep at several CTAs per SM, reps sweeps each on
- * `stream`, and keeps the fastest for later sweeps.  *best_us (host,
- * nullable) receives its time per sweep.  No-op for VC_IMPLICIT handles.  The schedule
- * never changes results: every candidate does the same arithmetic in the same order.
+ * `stream`, and keeps the fastest for later sweeps.  Solves then use the resident loop if a
+ * sweep of it is faster still (it has no schedule; before the first call they use it on every
+ * unsliced pipelined schedule).  *best_us (host, nullable) receives the time per sweep of what a
+ * solve runs.  No-op for VC_IMPLICIT handles.  Neither choice ever changes results: every
+ * candidate does the same arithmetic in the same order.
  */
 int vc_autotune(vc_mdp* m, int reps, double* best_us, void* stream);
 
@@ -427,7 +429,8 @@ int64_t vc_autotune_report(const vc_mdp* m, char* buf, int64_t len);
  * number of candidates of this CSR handle, in the order of vc_autotune_report's rows (CSR
  * tilings, the direct CSR kernel, then with a sliced copy the ring sweep's launch shapes
  * and the direct sliced kernel); index >= 0 switches the handle to that candidate for later
- * sweeps, index < 0 only counts.  The schedule never changes results (see vc_autotune).
+ * sweeps (and solves, but for the unsliced pipelined ones, whose solves run the resident
+ * loop), index < 0 only counts.  The schedule never changes results (see vc_autotune).
  * VC_ERR_ARG for an implicit handle or an index >= *count; the handle keeps its schedule.
  */
 int vc_sweep_schedule(vc_mdp* m, int32_t index, int32_t* count, void* stream);

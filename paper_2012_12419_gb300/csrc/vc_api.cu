@@ -253,6 +253,42 @@ static int loop32_resident(Mdp* m, float* buf0, float* buf1, double tol, long lo
     return VC_OK;
 }
 
+int time_solve_loop(Mdp* m, bool resident, int sweeps, cudaStream_t st, double* us) {
+    *us = 0.0;
+    const int choice = m->loop_choice;
+    m->loop_choice = resident ? 1 : 0;
+    cudaEvent_t e[2] = {nullptr, nullptr};
+    float* buf[2] = {m->Vb, m->E0};
+    auto run = [&]() -> int {
+        Ctl& h = *m->ctl_host;
+        reset_ctl(h, 1e-30, sweeps, m->spin_polls);
+        VC_CUDA(cudaMemcpyAsync(m->ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
+        VC_CUDA(cudaMemsetAsync(buf[0], 0, 4 * (size_t)m->S, st));
+        for (auto& x : e)
+            if (!x) VC_CUDA(cudaEventCreate(&x));
+        int rc = VC_OK;
+        bool launched = true;
+        VC_CUDA(cudaEventRecord(e[0], st));
+        if (resident) rc = launch_csr_loop(m, buf[0], buf[1], 0, st, &launched);
+        for (int i = 0; !resident && !rc && i < sweeps; i++)
+            rc = launch_sweep32(m, buf[i & 1], buf[1 - (i & 1)], nullptr, nullptr, SweepCtl{m->ctl, kModeLoop32, 1 - (i & 1), nullptr}, st);
+        if (rc || !launched) return rc;
+        VC_CUDA(cudaEventRecord(e[1], st));
+        if ((rc = read_ctl(m, st))) return rc;
+        if (h.error & kErrTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
+        float ms = 0.0f;
+        VC_CUDA(cudaEventElapsedTime(&ms, e[0], e[1]));
+        if (h.sweeps > 0) *us = 1e3 * ms / (double)h.sweeps;
+        return VC_OK;
+    };
+    int rc = run();  // warm-up
+    if (!rc && *us > 0.0) rc = run();
+    for (auto& x : e)
+        if (x) cudaEventDestroy(x);
+    m->loop_choice = choice;
+    return rc;
+}
+
 // One FP64 Bellman backup V_in -> V_out with argmax pi_out; returns max|V_out - V_in| and
 // the number of states whose argmax differs from pi_ref (if given).
 static int cert64(Mdp* m, const double* V_in, double* V_out, int32_t* pi_out, double* qgap,
@@ -321,6 +357,7 @@ int64_t vc_kernel_launches(void) { return (int64_t)g_launches.load(std::memory_o
 static int use_sliced(Mdp* m, cudaStream_t st) {
     int rc = build_sliced(m, st);
     if (rc) return rc;
+    m->loop_choice = -1;
     std::vector<CsrPlan> cands;
     if (!(m->fmt & VC_DIRECT) && (rc = sell_plans(m, st, cands))) return rc;
     if (cands.empty()) {
@@ -672,6 +709,7 @@ int vc_sweep_schedule(vc_mdp* mh, int32_t index, int32_t* count, void* stream) {
     if (index < 0) return VC_OK;
     if (index >= (int32_t)cands.size()) return fail(VC_ERR_ARG, "schedule index out of range");
     m->plan = cands[(size_t)index];
+    m->loop_choice = -1;
     return VC_OK;
 }
 

@@ -563,12 +563,6 @@ __global__ void k_tile_cap(const int64_t* __restrict__ row_ptr, int S, int A, in
     atomicMax(out, (unsigned long long)(row_ptr[s1 * A] - row_ptr[s0 * A]));
 }
 
-static int pow2_at_least(int a) {
-    int p = 1;
-    while (p < a) p <<= 1;
-    return p;
-}
-
 // Dynamic shared memory limit of a kernel instance, and how many CTAs fit on an SM.
 // `bytes` is the per-block opt-in limit; the kernel's static shared memory comes off it.
 // *dyn_limit receives the dynamic amount actually allowed.
@@ -857,7 +851,7 @@ int csr_candidates(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& cands) {
 }
 
 // Times every candidate schedule on this handle and keeps the fastest: reps FP32 sweeps
-// each after two warm-up sweeps, CUDA events on `st`.
+// each after two warm-up sweeps, CUDA events on `st`; then the resident loop against it.
 int autotune_csr(Mdp* m, int reps, cudaStream_t st, double* best_us) {
     std::vector<CsrPlan> cands;
     int rc = csr_candidates(m, st, cands);
@@ -902,7 +896,14 @@ int autotune_csr(Mdp* m, int reps, cudaStream_t st, double* best_us) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     m->plan = chosen;
-    if (best_us) *best_us = best;
+    // A solve's loop may also run resident (vc_csr_loop.cu; it needs no schedule): the faster of
+    // the two, residual and step-3 test included, serves the solves, while single sweeps keep
+    // the schedule chosen above.  64 sweeps make the launch a small part.
+    double loop_us = 0.0, sweep_us = 0.0;
+    if ((rc = time_solve_loop(m, true, std::max(reps, 64), st, &loop_us))) return rc;
+    if (loop_us > 0.0 && (rc = time_solve_loop(m, false, std::max(reps, 64), st, &sweep_us))) return rc;
+    m->loop_choice = loop_us > 0.0 && loop_us < sweep_us ? 1 : 0;
+    if (best_us) *best_us = m->loop_choice ? loop_us : best;
     return VC_OK;
 }
 

@@ -331,22 +331,22 @@ static int csr_loop_run(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStr
 int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {
     *launched = false;
     const bool bf16 = (m->fmt & 0xF) == VC_CSR_BF16;
-    // every pipelined CSR schedule (the loop is the faster one at each size and type measured)
-    // whose entries are counted in 31 bits; a handle whose waits were capped keeps the launched
+    // what the autotuner found, else every pipelined CSR schedule (the loop is the faster one at
+    // each size and type measured), if the entries are counted in 31 bits; a handle whose waits were capped keeps the launched
     // sweeps (but for the bounds-checking build, where the cap reaches this loop's waits)
 #ifdef VC_DEBUG_BOUNDS
     const bool capped = false;
 #else
     const bool capped = m->spin_polls >= 0;
 #endif
-    if (!m->plan.tma || m->plan.sliced || m->loop_cap <= 0 || capped || m->nnz_stored >= (1LL << 31) - 64)
-        return VC_OK;
+    if (m->loop_choice == 0 || (m->loop_choice < 0 && (!m->plan.tma || m->plan.sliced))) return VC_OK;
+    if (m->loop_cap <= 0 || capped || m->nnz_stored >= (1LL << 31) - 64) return VC_OK;
     auto go = [&](auto apad) {
         constexpr int AP = decltype(apad)::value;
         return bf16 ? csr_loop_run<uint16_t, AP>(m, buf0, buf1, self_loop, st, launched)
                     : csr_loop_run<float, AP>(m, buf0, buf1, self_loop, st, launched);
     };
-    switch (m->plan.apad) {
+    switch (pow2_at_least(m->A)) {
         case 1: return go(std::integral_constant<int, 1>());
         case 2: return go(std::integral_constant<int, 2>());
         case 4: return go(std::integral_constant<int, 4>());

@@ -684,6 +684,7 @@ struct Mdp {
     double* rate_tab = nullptr; // rates.occ_tab (device, owned)
     CsrPlan plan;
     int64_t loop_cap = 0;       // most entries of 32 / A consecutive states' rows (the resident loop's chunks)
+    int loop_choice = -1;       // solves by the resident loop: 1 yes, 0 no (autotuner), -1 by the plan
     const AdjRows* adj = nullptr;  // a view for the adjoint solve: its products use these rows
     std::string tune_report;    // candidates and times of the last autotune
     // sliced copy of the stored matrix (SELL-C-sigma, C = 32 states per slice): one
@@ -771,9 +772,21 @@ int state_grid(const Mdp* m);
 // grid at once (nothing was enqueued; the caller launches sweep by sweep).
 int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
 
-// The same loop over a stored matrix that stays in L2 (vc_csr_loop.cu); *launched is also
-// false when the matrix or its schedule is not one the loop serves.
+// The same loop over a stored matrix of any size (vc_csr_loop.cu); *launched is also false when
+// the matrix or its schedule is not one the loop serves.
 int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
+
+// Least power of two >= a (the lanes of a state in the CSR sweeps).
+inline int pow2_at_least(int a) {
+    int p = 1;
+    while (p < a) p <<= 1;
+    return p;
+}
+
+// Microseconds a sweep of a solve's FP32 loop over a stored matrix from V = 0 (at most `sweeps` of
+// them), resident or by launched sweeps of the handle's schedule; *us = 0 where the resident
+// loop does not serve the handle (vc_api.cu).
+int time_solve_loop(Mdp* m, bool resident, int sweeps, cudaStream_t st, double* us);
 
 // Inner hosts and block size of the in-block iteration of an implicit handle.
 int block_shape(const Mdp* m, int* h_out, int* B_out);

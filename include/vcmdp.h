@@ -573,10 +573,11 @@ int vc_batch_small_instances(const vc_batch* b, int32_t* count, int32_t* max_sta
 int vc_batch_set_block_iteration(vc_batch* b, int32_t threads, int32_t passes, void* stream);
 
 /*
- * Autotuner of the batched schedule: times the FP32 loop graph for `sweeps` sweeps of every
- * (tile size in {256, 512, ..., 8192}, blocks per SM in {2, 4, 8}) and keeps the fastest,
- * recapturing the graphs.  *best_ms (host, nullable) receives its time.  Results do not
- * depend on the schedule.
+ * Autotuner of the batched schedule: times every (tile size in {256, 512, ..., 8192}, blocks
+ * per SM in {2, 4, 8}) and keeps the fastest, recapturing the graphs.  Timed is what a solve
+ * runs by the schedule: the FP32 loop graph for `sweeps` sweeps or, where the resident loop
+ * takes its place, a round of the refinement with at most `sweeps` BiCGSTAB iterations.
+ * *best_ms (host, nullable) receives its time.  Results do not depend on the schedule.
  */
 int vc_batch_autotune(vc_batch* b, int sweeps, double* best_ms, void* stream);
 

@@ -2023,8 +2023,28 @@ int vc_batch_set_block_iteration(vc_batch* bh, int32_t threads, int32_t passes, 
     return VC_OK;
 }
 
-// Times the FP32 loop graph for every (tile size, blocks per SM) schedule on this batch
-// (a fixed number of sweeps from V = 0) and keeps the fastest.
+// Enqueues what the schedule governs in a solve whose FP32 loop is resident: one round of the
+// refinement from V = 0, its BiCGSTAB cut at kr_max_d iterations.
+static int enqueue_refinement(Batch* b, cudaStream_t st) {
+    const BatchKrylov K = kry_of(b);
+    VC_CUDA(cudaMemsetAsync(b->res64, 0, 8 * (size_t)b->n, st));
+    count_launches(9);
+    by_mh(b->mh, [&](auto m) { enqueue_extract<decltype(m)::value>(b, b->Va, b->pi, st); });
+    k_f32_to_f64_n<<<b->grid, kThreads, 0, st>>>(b->Va, b->V64, b->padded);
+    by_mh(b->mh, [&](auto m) { enqueue_resid<decltype(m)::value>(b, nullptr, st); });
+    k_bkr_reset<<<(b->n + 255) / 256, 256, 0, st>>>(K, b->n, 1e-30, b->tol_scale);
+    k_bkr_init<<<b->grid, kThreads, 0, st>>>(b->d_desc, b->d_tiles, b->ntiles, K);
+    VC_LAUNCHED("refinement round");
+    VC_CUDA(cudaGraphLaunch(b->x_kry, st));
+    by_mh(b->mh, [&](auto m) { enqueue_cert<decltype(m)::value>(b, nullptr, st); });
+    VC_LAUNCHED("FP64 certificate");
+    return VC_OK;
+}
+
+// Times every (tile size, blocks per SM) schedule on this batch over what a solve runs by it and
+// keeps the fastest: the FP32 loop graph (a fixed number of sweeps from V = 0), or, where the
+// resident loop takes its place, a round of the refinement with as many BiCGSTAB iterations.
+// Ranked by the graph, the 512-instance batch took 108.7 ms instead of 105.6.
 int vc_batch_autotune(vc_batch* bh, int sweeps, double* best_ms, void* stream) {
     set_error("");
     if (!bh) return fail(VC_ERR_ARG, "NULL handle");
@@ -2039,6 +2059,10 @@ int vc_batch_autotune(vc_batch* bh, int sweeps, double* best_ms, void* stream) {
     double best = 1e300;
     int best_ts = b->ts, best_bps = b->bps;
     int rc;
+    const bool refine = b->n_small < b->n && b->mh <= kBatchLoopMaxH && b->n <= kBatchLoopMaxN && !graph_faster(b);
+    const long long iters = sweeps, all_iters = kKrylovMaxIter;
+    const std::vector<float> ones((size_t)b->n, 1.0f);
+    VC_CUDA(cudaMemcpy(b->tol_scale, ones.data(), 4 * (size_t)b->n, cudaMemcpyHostToDevice));
     b->tune_report = "tile_states blocks_per_sm grid tiles ms\n";
     for (int ts : tss) {
         for (int bps : bpss) {
@@ -2050,11 +2074,21 @@ int vc_batch_autotune(vc_batch* bh, int sweeps, double* best_ms, void* stream) {
             for (int rep = 0; rep < 2; rep++) {
                 VC_CUDA(cudaMemsetAsync(b->Va, 0, 4 * (size_t)b->padded, st));
                 if ((rc = reset_loop(b, 1e-30, sweeps, st))) return rc;
-                VC_CUDA(cudaEventRecord(e0, st));
-                count_launches((sweeps + 1) / 2 * kViBodyKernels);
                 if (!graphs_ready(b)) return fail(VC_ERR_CUDA, "the batch's loop graphs are not built");
-                VC_CUDA(cudaGraphLaunch(b->x_vi, st));
-                VC_CUDA(cudaEventRecord(e1, st));
+                if (refine) {
+                    VC_CUDA(cudaMemcpy(b->kr_max_d, &iters, sizeof(iters), cudaMemcpyHostToDevice));
+                    VC_CUDA(cudaEventRecord(e0, st));
+                    rc = enqueue_refinement(b, st);
+                    VC_CUDA(cudaEventRecord(e1, st));
+                    VC_CUDA(cudaStreamSynchronize(st));
+                    VC_CUDA(cudaMemcpy(b->kr_max_d, &all_iters, sizeof(all_iters), cudaMemcpyHostToDevice));
+                    if (rc) return rc;
+                } else {
+                    VC_CUDA(cudaEventRecord(e0, st));
+                    count_launches((sweeps + 1) / 2 * kViBodyKernels);
+                    VC_CUDA(cudaGraphLaunch(b->x_vi, st));
+                    VC_CUDA(cudaEventRecord(e1, st));
+                }
                 VC_CUDA(cudaEventSynchronize(e1));
                 float ms = 0.0f;
                 VC_CUDA(cudaEventElapsedTime(&ms, e0, e1));

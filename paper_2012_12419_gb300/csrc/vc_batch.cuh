@@ -46,6 +46,8 @@ struct BatchCtl {
 // `first` on until all have ended, only instances of at most hand_over states are left or the
 // launch's time is up (LaunchEnd); the sweeps then done are at *end.  *launched = false when it does not serve
 // the batch (hosts, instances) or the device cannot hold the grid.
+constexpr int kBatchLoopMaxH = 5;     // above, an item and its coefficients no longer fit 128 registers
+constexpr int kBatchLoopMaxN = 4096;  // instances whose shares and verdicts fit shared memory
 constexpr int kLoopTimeout = 1, kLoopHandOver = 2;
 struct BatchLoopArgs {
     const InstDesc* descs;

@@ -25,8 +25,6 @@
 namespace vc {
 
 constexpr int kBatchLoopThreads = 512;  // 640 and 768: spills, 48 instances 10.0 -> 11.4 and 14 ms
-constexpr int kBatchLoopMaxH = 5;      // above, an item and its coefficients no longer fit 128 registers
-constexpr int kBatchLoopMaxN = 4096;   // instances whose shares and verdicts fit shared memory
 // Sweeps for which the hand-over (four launches, two host calls: 0.1 ms) pays at 2 to 4 us a sweep.
 constexpr int kHandOverSweeps = 64;
 

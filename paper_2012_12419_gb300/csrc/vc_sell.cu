@@ -551,7 +551,6 @@ struct SellRingArgs {
     FastDiv div_nu;   // division by TS * ups (units per full tile)
     FastDiv div_ups;  // division by ups
     int ups;          // units per slice
-    int per_unit;     // actions of a unit (a slice's last may hold fewer)
     int TS;           // slices per tile (the last tile may hold fewer)
     int64_t ntiles;
     int ring;         // bytes of the tile ring
@@ -559,8 +558,9 @@ struct SellRingArgs {
 };
 
 // MB = 1: up to 800 threads (24 consumer warps), 80 registers; MB = 2: two CTAs of up to
-// 17 warps per SM, 60 registers.
-template <typename VT, int MB, bool SL>
+// 17 warps per SM, 60 registers.  PU: actions of a unit; with one there is no loop over them
+// (the loop cost 5 to 9 % of a sweep at 3 actions, and 17 % with SL on BF16 values).
+template <typename VT, int MB, bool SL, int PU>
 __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_sell_ring(SellArgs a, SellRingArgs t,
                                                                                         SweepCtl sc) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
                 break;
             }
             unsigned char* base = ring + *((volatile uint32_t*)&slot_pos[s]);
-            const int sl = (int)fdiv((uint32_t)b, t.div_ups), act0 = (b - sl * t.ups) * t.per_unit;
+            const int sl = (int)fdiv((uint32_t)b, t.div_ups), act0 = (b - sl * t.ups) * PU;
             int roff = 0;
             for (int k = 0; k < sl; ++k)
                 roff += (int)rec_layout(A, reinterpret_cast<const int32_t*>(base + roff)[A], (int)sizeof(VT), a.has_scale)
@@ -717,13 +717,12 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
             // proxy fence orders the writes before the tile's next bulk copy
             const RecAt<int> at = rec_at<int>(base + roff, A, a.has_scale);
             float* qrow = reinterpret_cast<float*>(base + roff + 256) + lane;
-            if constexpr (SL && sizeof(VT) == 2) {
-                // always one action (see the launch); without the loop 64.9 us a sweep against 75.9 at
-                // 524,288 states
+            if constexpr (PU == 1) {
                 qrow[act0 * kSellC] =
                     block_q<VT, SL>(base + roff, at, act0, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
             } else {
-                const int act1 = min(act0 + t.per_unit, A);
+                const int act1 = min(act0 + PU, A);
+#pragma unroll 1
                 for (int act = act0; act < act1; ++act)
                     qrow[act * kSellC] =
                         block_q<VT, SL>(base + roff, at, act, lane, a.gamma, a.has_scale, a.V_in, a.S, sc.ctl);
@@ -794,19 +793,23 @@ __global__ void __launch_bounds__(MB == 1 ? (kMaxRW + 1) * 32 : 17 * 32, MB) k_s
     finish_block<float>(sc, res, vabs, sweep);
 }
 
-static const void* ring_fn(bool bf16, int mb, bool sl) {
-    if (bf16) {
-        if (mb == 2) return sl ? (const void*)k_sell_ring<uint16_t, 2, true> : (const void*)k_sell_ring<uint16_t, 2, false>;
-        return sl ? (const void*)k_sell_ring<uint16_t, 1, true> : (const void*)k_sell_ring<uint16_t, 1, false>;
-    }
-    if (mb == 2) return sl ? (const void*)k_sell_ring<float, 2, true> : (const void*)k_sell_ring<float, 2, false>;
-    return sl ? (const void*)k_sell_ring<float, 1, true> : (const void*)k_sell_ring<float, 1, false>;
+// Two actions a unit are not built for the self-transition sweep of BF16 values (see the launch).
+template <typename VT, int MB>
+static const void* ring_fn_of(bool sl, int per_unit) {
+    if (sl && (per_unit == 1 || sizeof(VT) == 2)) return (const void*)k_sell_ring<VT, MB, true, 1>;
+    if (sl) return (const void*)k_sell_ring<VT, MB, true, sizeof(VT) == 2 ? 1 : 2>;
+    return per_unit == 1 ? (const void*)k_sell_ring<VT, MB, false, 1> : (const void*)k_sell_ring<VT, MB, false, 2>;
+}
+
+static const void* ring_fn(bool bf16, int mb, bool sl, int per_unit) {
+    if (bf16) return mb == 2 ? ring_fn_of<uint16_t, 2>(sl, per_unit) : ring_fn_of<uint16_t, 1>(sl, per_unit);
+    return mb == 2 ? ring_fn_of<float, 2>(sl, per_unit) : ring_fn_of<float, 1>(sl, per_unit);
 }
 
 // Candidate launch shapes of the ring sweep, in preference order: (CTAs per SM, consumer
 // warps per CTA) x slices per tile; the ring takes the shared memory left after the
-// header and must hold the largest tile.  A shape must fit both instantiations (Eq. 18's
-// backup and the self-transition solve), since one plan serves both.
+// header and must hold the largest tile.  A shape must fit Eq. 18's backup and the
+// self-transition solve, since one plan serves both.
 int sell_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
     (void)st;
     out.clear();
@@ -825,32 +828,43 @@ int sell_plans(Mdp* m, cudaStream_t st, std::vector<CsrPlan>& out) {
         const long long max_tile = m->sell_max_tile[TS == 1 ? 0 : (TS == 2 ? 1 : 2)];  // largest tile of TS records
         for (auto& sh : shapes) {
             const int ctas = sh[0], nrw = sh[1], mb = sh[2];
-            const void* fn = ring_fn(bf16, mb, false);
-            const void* fn_sl = ring_fn(bf16, mb, true);
-            cudaFuncAttributes fa, fa_sl;
-            VC_CUDA(cached_func_attributes(fn, &fa));
-            VC_CUDA(cached_func_attributes(fn_sl, &fa_sl));
-            fa.numRegs = std::max(fa.numRegs, fa_sl.numRegs);
-            fa.sharedSizeBytes = std::max(fa.sharedSizeBytes, fa_sl.sharedSizeBytes);
-            fa.maxThreadsPerBlock = std::min(fa.maxThreadsPerBlock, fa_sl.maxThreadsPerBlock);
+            // Two actions a unit where a slice has four or more and its rows come from a model, whose
+            // lanes' successors share cache lines; rows of a user's matrix may scatter, and a unit of
+            // two then waits on twice the gathers (200,003 states, random columns, 12 or 30 entries:
+            // 1 to 5 % a sweep).  A shape whose warps would claim units too far ahead keeps one.
+            const bool local = m->has_model || m->val64;
+            const int ahead = (kSlots - 2) * TS;  // tiles between the oldest and the newest claimed unit
+            const int per_unit = A >= 4 && local && nrw <= ahead * ((A + 1) / 2) ? 2 : 1;
+            if (nrw > ahead * ((A + per_unit - 1) / per_unit)) continue;
+            // a shape must fit every instantiation that its plan may launch (the shared memory limit is
+            // one for all of them, so that no plan lowers another's)
+            cudaFuncAttributes fa;
+            const void* fns[4];
+            for (int k = 0; k < 4; k++) {
+                fns[k] = ring_fn(bf16, mb, k >= 2, 1 + (k & 1));
+                cudaFuncAttributes f;
+                VC_CUDA(cached_func_attributes(fns[k], &f));
+                if (k == 0) fa = f;
+                fa.sharedSizeBytes = std::max(fa.sharedSizeBytes, f.sharedSizeBytes);
+                if ((k & 1) && per_unit == 1) continue;
+                fa.numRegs = std::max(fa.numRegs, f.numRegs);
+                fa.maxThreadsPerBlock = std::min(fa.maxThreadsPerBlock, f.maxThreadsPerBlock);
+            }
             const int dyn_max = smem_blk - (int)fa.sharedSizeBytes;
-            VC_CUDA(cached_set_max_dyn_smem(fn, dyn_max));
-            VC_CUDA(cached_set_max_dyn_smem(fn_sl, dyn_max));
+            for (const void* fn : fns) VC_CUDA(cached_set_max_dyn_smem(fn, dyn_max));
             const int threads = (nrw + 1) * 32;
             if (threads > fa.maxThreadsPerBlock || (long long)threads * fa.numRegs * ctas > 65536) continue;
-            const int per_unit = A >= 4 ? 2 : 1;  // measured above; a slice of few actions keeps its units
-            const int ups = (A + per_unit - 1) / per_unit;
-            if (nrw > (kSlots - 2) * TS * ups) continue;  // claimed units stay within kSlots tiles
             // the ring follows the header; Q values live in the tiles' own R rows
             const int budget = std::min(dyn_max, (smem_sm - 1024 * ctas) / ctas - (int)fa.sharedSizeBytes);
             const int ring = ((budget - kHead) / 128) * 128;
             if (ring < max_tile + 128) continue;
             const int need = kHead + ring;
-            int per_sm = 0;
-            int per_sm_sl = 0;
-            VC_CUDA(cached_occupancy(fn, threads, (size_t)need, &per_sm));
-            VC_CUDA(cached_occupancy(fn_sl, threads, (size_t)need, &per_sm_sl));
-            per_sm = std::min(per_sm, per_sm_sl);
+            int per_sm = ctas;
+            for (int k = 0; k < 4; k += per_unit == 1 ? 2 : 1) {
+                int n = 0;
+                VC_CUDA(cached_occupancy(fns[k], threads, (size_t)need, &n));
+                per_sm = std::min(per_sm, n);
+            }
             if (per_sm < 1) continue;
             CsrPlan P;
             P.sliced = true;
@@ -893,8 +907,8 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
         // longer, of BF16 values (524,288 states: 64.9 against 79.7 us) or of a slab beyond the L2
         // (2.5 M states 284 against 291 us; within it 100,000 states 17.1 against 15.9)
         const bool one = m->plan.ntiles < 4LL * grid || (sc.self_loop && (bf16 || m->sell_bytes > (128LL << 20)));
-        t.per_unit = one ? 1 : m->plan.per_unit;
-        t.ups = (m->A + t.per_unit - 1) / t.per_unit;
+        const int per_unit = one ? 1 : m->plan.per_unit;
+        t.ups = (m->A + per_unit - 1) / per_unit;
         t.div_nu = make_fastdiv((uint32_t)(m->plan.ts * t.ups));
         t.div_ups = make_fastdiv((uint32_t)t.ups);
         t.TS = m->plan.ts;
@@ -914,7 +928,7 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         void* args[] = {&a, &t, &sc};
-        VC_CUDA(cudaLaunchKernelExC(&cfg, ring_fn(bf16, m->plan.minb, sc.self_loop != 0), args));
+        VC_CUDA(cudaLaunchKernelExC(&cfg, ring_fn(bf16, m->plan.minb, sc.self_loop != 0, per_unit), args));
         return VC_OK;
     }
     const int bps = m->plan.ctas_per_sm > 0 ? m->plan.ctas_per_sm : 4;

@@ -31,6 +31,9 @@ constexpr int kLoopThreads = 640;
 // SM, what a sweep of the multi-CTA loop takes at any size (two barriers and two cold L2
 // round trips); four arrays of 8,192 floats also fit beside the L1's needs.
 constexpr int kLoopOneCta = 8192;
+// Sweeps of its launch: 6 to 20 ms at 1.4 to 5 us (by the clock, as the grids do it, the words in
+// shared memory cost 5 % of a sweep).
+constexpr int kLoopOneCtaSweeps = 4096;
 constexpr int kLoopItems = 256;    // least items of a CTA of the multi-CTA loop
 
 // SMEM: one CTA, V's two buffers, U and W in shared memory (4 S + kUPad floats); else W, U
@@ -49,7 +52,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
     const bool lead = threadIdx.x == 0;
     long long k = ctl->sweeps;
     const bool first = lead && blockIdx.x == 0;
-    LaunchEnd end{SMEM ? &sh_end : &ctl->launch_end, &sh_start};
+    const long long k_end = k + kLoopOneCtaSweeps;
+    LaunchEnd end{&ctl->launch_end, &sh_start};
     LoopVerdict verdict{ctl->tol, __double2float_ru(ctl->tol), ctl->best_res, ctl->since_best, ctl->max_sweeps};
     float* V[2] = {buf0, buf1};
     if constexpr (SMEM) {
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         sh_max[0][0] = sh_max[0][1] = sh_max[1][0] = sh_max[1][1] = 0u;
         sh_fail = 0;
     }
-    if (first) end.open(k);
+    if (!SMEM && first) end.open(k);
     __syncthreads();
     GridBarrier bar{&ctl->arrivals, gridDim.x, 0u, &sh_fail, barrier_polls(ctl->spin_limit)};
     int done = 0;
@@ -73,7 +77,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         const int in = (int)(k & 1);
         const float* Vi = V[in];
         float* Vo = V[in ^ 1];
-        if (first) end.check(k);
+        if (!SMEM && first) end.check(k);
         for (int t = t0 + (int)threadIdx.x; t < t1; t += (int)blockDim.x)
             post_item<MH, VW, SL>(md, c, Vi, VW * t, U, W, ctl);
         if constexpr (SMEM) {
@@ -129,7 +133,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_vi_loop(Model md, Coef<floa
         }
         k++;
         done = verdict(r, vm, k);
-        if (done || k >= *((volatile long long*)&sh_end)) break;
+        if (done || k >= (SMEM ? k_end : sh_end)) break;
     }
     if constexpr (SMEM) {
         __syncthreads();

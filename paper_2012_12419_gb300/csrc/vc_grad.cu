@@ -20,6 +20,7 @@
 
 #include <algorithm>
 
+#include "vc_adj.cuh"
 #include "vc_internal.cuh"
 
 namespace vc {
@@ -71,40 +72,53 @@ __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, c
 // Orders each transposed row by source state, out of place: an entry's position is the number
 // of the row's entries with a smaller source (sources are distinct), counted over the lanes'
 // consecutive loads.  In place by insertion, every step waited for its own loads and stores:
-// 432 us at 343,750 states.
-__global__ void k_adj_sort(int S, const int64_t* __restrict__ base, const int32_t* __restrict__ cnt,
-                           const int32_t* __restrict__ colU, const double* __restrict__ valU64,
-                           int32_t* __restrict__ colT, float* __restrict__ valT, double* __restrict__ valT64) {
-    for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < S; y += gridDim.x * blockDim.x) {
-        const int64_t lo = base[y >> 5] + (y & 31);
-        const int n = cnt[y];
-        for (int i = 0; i < n; i++) {
-            const int c = colU[lo + 32LL * i];
-            const double v = valU64[lo + 32LL * i];
-            int rank = 0;
-            for (int j = 0; j < n; j++) rank += colU[lo + 32LL * j] < c ? 1 : 0;
-            colT[lo + 32LL * rank] = c;
-            valT[lo + 32LL * rank] = (float)v;
-            valT64[lo + 32LL * rank] = v;
+// 432 us at 343,750 states.  The count is quadratic in the row, so a row of more than kAdjLong
+// entries is shared by the warp, a lane per entry: a lane alone took 109 ms for the rows of some
+// 2,000 entries of a host of 1,000 slots.
+constexpr int kAdjLong = 32;
+__global__ void __launch_bounds__(kThreads) k_adj_sort(int S, const int64_t* __restrict__ base,
+                                                       const int32_t* __restrict__ cnt,
+                                                       const int32_t* __restrict__ colU,
+                                                       const double* __restrict__ valU64, int32_t* __restrict__ colT,
+                                                       float* __restrict__ valT, double* __restrict__ valT64) {
+    const int lane = threadIdx.x & 31;
+    for (int y0 = (blockIdx.x * kThreads + threadIdx.x) & ~31; y0 < S; y0 += gridDim.x * kThreads) {
+        const int y = y0 + lane;
+        const int64_t b0 = base[y0 >> 5];
+        const int n = y < S ? cnt[y] : 0;
+        // entries first, first + step, .. of the row in column q of the slice
+        auto place = [&](int q, int len, int first, int step) {
+            const int64_t lo = b0 + q;
+            for (int i = first; i < len; i += step) {
+                const int c = colU[lo + 32LL * i];
+                const double v = valU64[lo + 32LL * i];
+                int rank = 0;
+#pragma unroll 4
+                for (int j = 0; j < len; j++) rank += colU[lo + 32LL * j] < c ? 1 : 0;
+                colT[lo + 32LL * rank] = c;
+                valT[lo + 32LL * rank] = (float)v;
+                valT64[lo + 32LL * rank] = v;
+            }
+        };
+        if (n <= kAdjLong) place(lane, n, 0, 1);
+        __syncwarp();
+        for (unsigned int m = __ballot_sync(0xffffffffu, n > kAdjLong); m; m &= m - 1) {
+            const int q = __ffs((int)m) - 1;
+            place(q, __shfl_sync(0xffffffffu, n, q), lane, 32);
+            __syncwarp();
         }
     }
 }
 
 // Fixed-point sweep of the adjoint system, x' = b + gamma P^T x (the fallback solve).
-__global__ void __launch_bounds__(kThreads) k_adj_sweep(int S, float gamma, const int64_t* __restrict__ base,
-                                                        const int32_t* __restrict__ cnt,
-                                                        const int32_t* __restrict__ colT,
-                                                        const float* __restrict__ valT, const float* __restrict__ b,
+__global__ void __launch_bounds__(kThreads) k_adj_sweep(int S, float gamma, AdjRows t, const float* __restrict__ b,
                                                         const float* __restrict__ x, float* __restrict__ x_out,
                                                         SweepCtl sc) {
     if (loop_done(sc)) return;
     const long long sweep = loop_sweep(sc);
     float res = 0.0f, vabs = 0.0f;
     for (int y = blockIdx.x * kThreads + threadIdx.x; y < S; y += gridDim.x * kThreads) {
-        const int64_t lo = base[y >> 5] + (y & 31);
-        float acc = 0.0f;
-        for (int j = 0; j < cnt[y]; j++) acc = fmaf(valT[lo + 32LL * j], x[colT[lo + 32LL * j]], acc);
-        const float v = b[y] + gamma * acc;
+        const float v = b[y] + gamma * adj_row_dot<16>(t, t.val, y, x);
         x_out[y] = v;
         res = fmaxf(res, fabsf(v - x[y]));
         vabs = fmaxf(vabs, fabsf(v));
@@ -116,19 +130,12 @@ __global__ void __launch_bounds__(kThreads) k_adj_sweep(int S, float gamma, cons
 
 // FP64 residual of the adjoint system r = rho + gamma P^T lam - lam (stored as float);
 // max |r| into the control block's certificate slot.
-__global__ void __launch_bounds__(kThreads) k_adj_resid64(int S, double gamma, const int64_t* __restrict__ base,
-                                                          const int32_t* __restrict__ cnt,
-                                                          const int32_t* __restrict__ colT,
-                                                          const double* __restrict__ valT64,
-                                                          const double* __restrict__ rho,
+__global__ void __launch_bounds__(kThreads) k_adj_resid64(int S, double gamma, AdjRows t, const double* __restrict__ rho,
                                                           const double* __restrict__ lam, float* __restrict__ r,
                                                           SweepCtl sc) {
     double res = 0.0;
     for (int y = blockIdx.x * kThreads + threadIdx.x; y < S; y += gridDim.x * kThreads) {
-        double acc = 0.0;
-        const int64_t lo = base[y >> 5] + (y & 31);
-        for (int j = 0; j < cnt[y]; j++) acc += valT64[lo + 32LL * j] * lam[colT[lo + 32LL * j]];
-        const double v = rho[y] + gamma * acc - lam[y];
+        const double v = rho[y] + gamma * adj_row_dot<8>(t, t.val64, y, lam) - lam[y];
         r[y] = (float)v;
         res = fmax(res, fabs(v));
     }
@@ -323,7 +330,7 @@ int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpo
 int launch_adj_sweep(Mdp* m, const AdjRows& t, const float* b, const float* x, float* x_out, SweepCtl sc,
                      cudaStream_t st) {
     count_launches(1);
-    k_adj_sweep<<<state_grid(m), kThreads, 0, st>>>(m->S, (float)m->gamma, t.base, t.cnt, t.col, t.val, b, x, x_out, sc);
+    k_adj_sweep<<<state_grid(m), kThreads, 0, st>>>(m->S, (float)m->gamma, t, b, x, x_out, sc);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }
@@ -331,7 +338,7 @@ int launch_adj_sweep(Mdp* m, const AdjRows& t, const float* b, const float* x, f
 int launch_adj_resid64(Mdp* m, const AdjRows& t, const double* rho, const double* lam, float* r, SweepCtl sc,
                        cudaStream_t st) {
     count_launches(1);
-    k_adj_resid64<<<state_grid(m), kThreads, 0, st>>>(m->S, m->gamma, t.base, t.cnt, t.col, t.val64, rho, lam, r, sc);
+    k_adj_resid64<<<state_grid(m), kThreads, 0, st>>>(m->S, m->gamma, t, rho, lam, r, sc);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }

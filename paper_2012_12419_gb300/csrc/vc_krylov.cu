@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "vc_adj.cuh"
 #include "vc_grid.cuh"
 #include "vc_implicit.cuh"
 #include "vc_krylov.cuh"
@@ -363,26 +364,7 @@ struct AdjProduct {
     __device__ __forceinline__ void setup(const KrylovArgs&, int) const {}
     __device__ __forceinline__ void first(const KrylovArgs&, const float*, int) const {}
     __device__ __forceinline__ void row(const KrylovArgs& k, const float* xin, int s, float* y) const {
-        y[0] = xin[s];
-        const int n = __ldg(t.cnt + s);
-        const int64_t lo = __ldg(t.base + (s >> 5)) + (s & 31);
-        const int32_t* cp = t.col + lo;
-        const float* vp = t.val + lo;
-        float acc = 0.0f;
-        for (int j0 = 0; j0 < n; j0 += 16, cp += 512, vp += 512) {
-            float w[16], g[16];
-#pragma unroll
-            for (int u = 0; u < 16; u++) {
-                if (j0 + u < n) {
-                    w[u] = __ldg(vp + 32 * u);
-                    g[u] = xin[__ldg(cp + 32 * u)];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 16; u++)
-                if (j0 + u < n) acc = fmaf(w[u], g[u], acc);
-        }
-        y[0] -= gamma * acc;
+        y[0] = xin[s] - gamma * adj_row_dot<16>(t, t.val, s, xin);
     }
 };
 

@@ -570,7 +570,7 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
         used += (bytes + 255) & ~(size_t)255;
         return at;
     };
-    const size_t o_cnt = part(4 * (size_t)S), o_fill = part(4 * (size_t)S), o_err = part(16), zeroed = used;
+    const size_t o_cnt = part(4 * (size_t)S), o_fill = part(4 * (size_t)S), o_err = part(24), zeroed = used;
     const size_t o_width = part(4 * (size_t)slices), o_base = part(8 * ((size_t)slices + 3));
     const size_t o_rho = part(4 * ((size_t)S + 8)), o_partial = part(grad_partial_bytes(m)), o_out = part(8 * ((size_t)nt + 1));
     VC_TRY(cudaMallocAsync((void**)&block[0], used, st));
@@ -579,7 +579,7 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     t.base = reinterpret_cast<int64_t*>(block[0] + o_base);
     int32_t* fillpos = reinterpret_cast<int32_t*>(block[0] + o_fill);
     int32_t* width = reinterpret_cast<int32_t*>(block[0] + o_width);
-    int* err = reinterpret_cast<int*>(block[0] + o_err);  // error flags, then the transpose's entries (8 bytes on)
+    int* err = reinterpret_cast<int*>(block[0] + o_err);  // error flags; from 8 bytes on the transpose's entries and its longest row
     float* rhoF = reinterpret_cast<float*>(block[0] + o_rho);
     double* partial = reinterpret_cast<double*>(block[0] + o_partial);
     double* out = reinterpret_cast<double*>(block[0] + o_out);
@@ -587,23 +587,21 @@ int vc_value_grad(vc_mdp* mh, const double* V, const int32_t* pi, const double* 
     if (rc) return bail(rc);
     if ((rc = launch_adj_width(m, t.cnt, width, (unsigned long long*)(err + 2), st))) return bail(rc);
     if ((rc = exclusive_scan(m, width, slices, t.base, st))) return bail(rc);
-    int64_t herr[2] = {0, 0};
+    int64_t herr[3] = {0, 0, 0};
     int64_t stored = 0;
-    VC_TRY(cudaMemcpyAsync(herr, err, 16, cudaMemcpyDeviceToHost, st));
+    VC_TRY(cudaMemcpyAsync(herr, err, 24, cudaMemcpyDeviceToHost, st));
     VC_TRY(cudaMemcpyAsync(&stored, t.base + slices, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     VC_TRY(cudaStreamSynchronize(st));
     if ((int)herr[0]) return bail(fail(VC_ERR_ARG, "the policy picks an infeasible action"));
     gs.nnz_transpose = herr[1];
     used = 0;
-    const size_t o_v64 = part(8 * (size_t)stored + 8), o_tv64 = part(8 * (size_t)stored), o_col = part(4 * (size_t)stored);
-    const size_t o_tcol = part(4 * (size_t)stored), o_val = part(4 * (size_t)stored);
+    const size_t o_v64 = part(8 * (size_t)stored + 8), o_col = part(4 * (size_t)stored), o_val = part(4 * (size_t)stored);
+    const size_t o_scratch = part(adj_scratch_bytes(m, herr[2]));
     VC_TRY(cudaMallocAsync((void**)&block[1], used, st));
     t.val64 = reinterpret_cast<double*>(block[1] + o_v64);
     t.col = reinterpret_cast<int32_t*>(block[1] + o_col);
     t.val = reinterpret_cast<float*>(block[1] + o_val);
-    double* val_tmp = reinterpret_cast<double*>(block[1] + o_tv64);  // as filled, before the rows are ordered
-    int32_t* col_tmp = reinterpret_cast<int32_t*>(block[1] + o_tcol);
-    if ((rc = launch_adj_fill(m, pi, t, fillpos, col_tmp, val_tmp, st))) return bail(rc);
+    if ((rc = launch_adj_fill(m, pi, t, fillpos, herr[2], block[1] + o_scratch, st))) return bail(rc);
 
     // ---- lam: the transposed system (right-hand side rho, matrix P^T) as a view for the solver
     if ((rc = launch_f64_to_f32(rho, rhoF, S, st))) return bail(rc);

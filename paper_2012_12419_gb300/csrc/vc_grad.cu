@@ -39,18 +39,23 @@ __global__ void k_adj_count(Model md, Rates rt, const int32_t* __restrict__ pi, 
     }
 }
 
-// Entries of every slice of 32 rows (32 x its longest row), and the entries of all rows.
+// Entries of every slice of 32 rows (32 x its longest row); total[0]: the entries of all rows,
+// total[1]: the longest row.
 __global__ void __launch_bounds__(kThreads) k_adj_width(int S, const int32_t* __restrict__ cnt, int32_t* __restrict__ width,
                                                         unsigned long long* total) {
     const int lane = threadIdx.x & 31, slices = (S + 31) / 32;
-    unsigned long long sum = 0;
+    unsigned long long sum = 0, longest = 0;
     for (int g = (blockIdx.x * kThreads + threadIdx.x) >> 5; g < slices; g += (gridDim.x * kThreads) >> 5) {
         const int n = 32 * g + lane < S ? cnt[32 * g + lane] : 0;
         const int w = __reduce_max_sync(0xffffffffu, n);
         sum += (unsigned long long)__reduce_add_sync(0xffffffffu, n);
         if (lane == 0) width[g] = 32 * w;
+        longest = max(longest, (unsigned long long)w);
     }
-    if (lane == 0 && sum) atomicAdd(total, sum);
+    if (lane == 0 && sum) {
+        atomicAdd(&total[0], sum);
+        atomicMax(&total[1], longest);
+    }
 }
 
 __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, const int64_t* __restrict__ base,
@@ -69,35 +74,56 @@ __global__ void k_adj_fill(Model md, Rates rt, const int32_t* __restrict__ pi, c
     }
 }
 
-// Orders each transposed row by source state, out of place: an entry's position is the number
-// of the row's entries with a smaller source (sources are distinct), counted over the lanes'
-// consecutive loads.  In place by insertion, every step waited for its own loads and stores:
-// 432 us at 343,750 states.  The count is quadratic in the row, so a row of more than kAdjLong
-// entries is shared by the warp, a lane per entry: a lane alone took 109 ms for the rows of some
-// 2,000 entries of a host of 1,000 slots.
+// Orders each transposed row by source state: a warp copies its slice to its own scratch (`most`
+// entries), and there an entry's position is the number of the row's entries with a smaller source
+// (sources are distinct), counted over the lanes' consecutive loads.  By insertion, every step
+// waited for its own loads and stores: 432 us at 343,750 states.  The count is quadratic in the
+// row, so a row of more than kAdjLong entries is shared by the warp, a lane per entry: a lane
+// alone took 109 ms for the rows of some 2,000 entries of a host of 1,000 slots.
 constexpr int kAdjLong = 32;
 __global__ void __launch_bounds__(kThreads) k_adj_sort(int S, const int64_t* __restrict__ base,
-                                                       const int32_t* __restrict__ cnt,
-                                                       const int32_t* __restrict__ colU,
-                                                       const double* __restrict__ valU64, int32_t* __restrict__ colT,
+                                                       const int32_t* __restrict__ cnt, unsigned char* scratch,
+                                                       int64_t most, int32_t* __restrict__ colT,
                                                        float* __restrict__ valT, double* __restrict__ valT64) {
-    const int lane = threadIdx.x & 31;
-    for (int y0 = (blockIdx.x * kThreads + threadIdx.x) & ~31; y0 < S; y0 += gridDim.x * kThreads) {
-        const int y = y0 + lane;
-        const int64_t b0 = base[y0 >> 5];
-        const int n = y < S ? cnt[y] : 0;
+    const int lane = threadIdx.x & 31, slices = (S + 31) / 32;
+    const int warps = (int)(gridDim.x * kThreads) >> 5, me = (int)(blockIdx.x * kThreads + threadIdx.x) >> 5;
+    double* valU = reinterpret_cast<double*>(scratch + 12 * most * me);
+    int32_t* colU = reinterpret_cast<int32_t*>(valU + most);
+    for (int g = me; g < slices; g += warps) {
+        const int n = 32 * g + lane < S ? cnt[32 * g + lane] : 0;
+        int32_t* col = colT + base[g];
+        float* val = valT + base[g];
+        double* val64 = valT64 + base[g];
+        for (int i0 = 0; i0 < n; i0 += 8) {
+            int c[8];
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (i0 + u < n) {
+                    c[u] = col[lane + 32 * (i0 + u)];
+                    v[u] = val64[lane + 32 * (i0 + u)];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (i0 + u < n) {
+                    colU[lane + 32 * (i0 + u)] = c[u];
+                    valU[lane + 32 * (i0 + u)] = v[u];
+                }
+            }
+        }
+        __syncwarp();
         // entries first, first + step, .. of the row in column q of the slice
         auto place = [&](int q, int len, int first, int step) {
-            const int64_t lo = b0 + q;
             for (int i = first; i < len; i += step) {
-                const int c = colU[lo + 32LL * i];
-                const double v = valU64[lo + 32LL * i];
+                const int c = colU[q + 32 * i];
+                const double v = valU[q + 32 * i];
                 int rank = 0;
 #pragma unroll 4
-                for (int j = 0; j < len; j++) rank += colU[lo + 32LL * j] < c ? 1 : 0;
-                colT[lo + 32LL * rank] = c;
-                valT[lo + 32LL * rank] = (float)v;
-                valT64[lo + 32LL * rank] = v;
+                for (int j = 0; j < len; j++) rank += colU[q + 32 * j] < c ? 1 : 0;
+                col[q + 32 * rank] = c;
+                val[q + 32 * rank] = (float)v;
+                val64[q + 32 * rank] = v;
             }
         };
         if (n <= kAdjLong) place(lane, n, 0, 1);
@@ -318,11 +344,24 @@ int launch_adj_width(Mdp* m, const int32_t* cnt, int32_t* width, unsigned long l
     return VC_OK;
 }
 
-int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, int32_t* col_tmp, double* val_tmp,
-                    cudaStream_t st) {
+// Blocks of k_adj_sort: enough warps to hide its loads, and no more scratch than 64 MB (which stays
+// in L2) as long as 16 blocks remain; one slice of 32 rows of 6,000 entries takes 2.3 MB.
+static int adj_sort_grid(const Mdp* m, int64_t most) {
+    const int64_t by_scratch = std::max<int64_t>(16, (64LL << 20) / (12 * std::max<int64_t>(most, 32) * (kThreads / 32)));
+    const int64_t slices = ((int64_t)m->S + 31) / 32, blocks = (slices + kThreads / 32 - 1) / (kThreads / 32);
+    return (int)std::min({(int64_t)state_grid(m), by_scratch, blocks});
+}
+
+size_t adj_scratch_bytes(const Mdp* m, int64_t longest) {
+    return (size_t)12 * 32 * longest * adj_sort_grid(m, 32 * longest) * (kThreads / 32);
+}
+
+int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, int64_t longest,
+                    unsigned char* scratch, cudaStream_t st) {
     count_launches(2);
-    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, t.base, fillpos, col_tmp, val_tmp);
-    k_adj_sort<<<state_grid(m), kThreads, 0, st>>>(m->S, t.base, t.cnt, col_tmp, val_tmp, t.col, t.val, t.val64);
+    k_adj_fill<<<state_grid(m), kThreads, 0, st>>>(m->md, m->rates, pi, t.base, fillpos, t.col, t.val64);
+    k_adj_sort<<<adj_sort_grid(m, 32 * longest), kThreads, 0, st>>>(m->S, t.base, t.cnt, scratch, 32 * longest, t.col,
+                                                                    t.val, t.val64);
     VC_CUDA(cudaGetLastError());
     return VC_OK;
 }

@@ -814,8 +814,9 @@ int exclusive_scan(Mdp* m, const int32_t* cnt, int64_t n, int64_t* out, cudaStre
 // Adjoint gradient kernels (vc_grad.cu).
 int launch_adj_count(Mdp* m, const int32_t* pi, int32_t* cnt, int* err, cudaStream_t st);
 int launch_adj_width(Mdp* m, const int32_t* cnt, int32_t* width, unsigned long long* total, cudaStream_t st);
-int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, int32_t* col_tmp, double* val_tmp,
-                    cudaStream_t st);
+size_t adj_scratch_bytes(const Mdp* m, int64_t longest);
+int launch_adj_fill(Mdp* m, const int32_t* pi, const AdjRows& t, int32_t* fillpos, int64_t longest,
+                    unsigned char* scratch, cudaStream_t st);
 int launch_adj_sweep(Mdp* m, const AdjRows& t, const float* b, const float* x, float* x_out, SweepCtl sc,
                      cudaStream_t st);
 int launch_adj_resid64(Mdp* m, const AdjRows& t, const double* rho, const double* lam, float* r, SweepCtl sc,

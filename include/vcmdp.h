@@ -474,7 +474,7 @@ int vc_value_grad(vc_mdp* m, const double* V, const int32_t* pi, const double* r
  * The objective of vc_value_grad, J = rho . V = sum_s rho[s] V[s], in FP64 on the device
  * (the initial-distribution-weighted value whose gradient vc_value_grad returns; the paper
  * has no objective of this form).  V, rho: [S] double device arrays; J: ONE double on the
- * device, written on `stream` (enqueued only).  One block sums in a fixed order, so the
+ * device, written on `stream` (enqueued only).  One cluster sums in a fixed order, so the
  * result is reproducible bit for bit.  VC_ERR_ARG for NULL pointers or S < 1.
  */
 int vc_objective(const double* V, const double* rho, int64_t S, double* J, void* stream);

@@ -14,7 +14,8 @@
 // Bound: L2 (DRAM while more than ~10 M states are active) latency of the items' loads at 16
 // warps an SM, and the slower SMs' tail at the two barriers.  Whole solves against the graph of
 // paired tile kernels (coefficients read from shared memory at each use, 8-byte loads): 512
-// instances of 17.4 M states 134 -> 104 ms, 48 with the self-transition solve 13.1 -> 10.0 ms.
+// instances of 17.4 M states 134 -> 105 ms, 48 with the self-transition solve 13.1 -> 9.2 ms (with
+// the hand-over below).
 #include <algorithm>
 
 #include "vc_batch.cuh"

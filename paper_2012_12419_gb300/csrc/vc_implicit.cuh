@@ -118,7 +118,7 @@ __device__ __forceinline__ bool has_host(const Model& md, int k) {
 
 // Pass 1 of one item: U(x) = R(x) + gamma E[V(next) | x] of its VW states and, with SL,
 // defer's value with its self-transition solved; EXPECT: E[V(next) | x] alone, into U.  Each
-// state's arithmetic is expect_from's (and defer_from's) in the same order.
+// state's arithmetic is expect_from's (and, for W, post_and_defer's) in the same order.
 template <int MH, int VW, bool SL, bool EXPECT = false>
 __device__ __forceinline__ void post_item(const Model& md, const Coef<float>& c, const float* V, int x, float* U,
                                           float* W, Ctl* ctl) {

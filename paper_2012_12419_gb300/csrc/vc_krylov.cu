@@ -23,8 +23,8 @@
 //
 // Bound: L2 latency of the gathers and of five short vector steps, and five (seven) barriers an
 // iteration.  Whole calls, launched kernels against this one: evaluation of a policy of
-// 524,288 states 8.6 -> 2.7 ms, gradient step of 343,750 states 12.3 -> 8.6 ms, solves of
-// 2.5 M states 10.1 -> 8.0 ms and of 640 states 0.74 -> 0.46 ms.
+// 524,288 states 8.6 -> 2.8 ms, gradient step of 343,750 states 12.3 -> 8.6 ms, solves of
+// 2.5 M states 10.1 -> 8.0 ms and of 640 states 0.74 -> 0.47 ms.
 #include <math.h>
 #include <string.h>
 

@@ -10,8 +10,8 @@
 // decision itself from the same two words.  Instances whose arrays fit one CTA's shared
 // memory run there without any grid barrier.
 //
-// Bound: L2 latency and issue of the two passes (per 4 states: 16 loads of 16 bytes and ~250
-// instructions), then two barriers of ~1.5 us.  Measured per sweep, launched kernels
+// Bound: issue and L2 latency of the two passes (16 loads of 16 bytes and some 340 instructions a
+// pass for 4 states of 7 hosts; 47 % of the issue slots), then two barriers of ~1.5 us.  Measured per sweep, launched kernels
 // against this loop: 45 -> 19 us at 2.5 M states (H = 7), 18.3 -> 8.0 us at 343,750 states
 // with the self-transition solve (VW = 2), whole solves of 640 states 2.89 -> 0.76 ms.
 #include <algorithm>

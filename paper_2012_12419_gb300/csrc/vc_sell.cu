@@ -30,17 +30,17 @@
 // into a ring of shared memory, one cp.async.bulk per tile, completion counted on an
 // mbarrier, L2 evict-first.  Tiles take their actual size in the ring (a tile that would
 // wrap restarts at the ring base; bytes are reused only after the tiles holding them are
-// released, in order).  Consumer warps take units (two actions of a slice) of the CTA's tile
+// released, in order).  Consumer warps take units (one or two actions of a slice) of the CTA's tile
 // sequence in order, one lane per state: shared-memory reads are lane-consecutive (no
 // bank conflicts) and the V gathers of a warp fall on a few cache lines because the
 // lanes' successors share offsets.  A block's Q values overwrite its own R row in the
 // ring (read once, by the same lane), so no separate Q buffer takes shared memory from the
 // ring; the warp that completes a tile's last unit takes the max over actions from the
 // tile's R rows and releases the tile.
-// The sweep is bound by its consumers (issue 44 %, L1 and shared-memory latency), no longer by
-// HBM: 24-31 % fewer bytes (16-bit column offsets) gained 4 % on FP32 values and lost 16 % on
+// The sweep is bound by its consumers (issue 43 to 47 %; V gathers, then shared-memory latency), no
+// longer by HBM: 24-31 % fewer bytes (16-bit column offsets) gained 4 % on FP32 values and lost 16 % on
 // BF16.  A unit's claim, wait and release cost as much as an action's row, hence two actions a
-// unit; with more, too few warps find work in the tiles in flight.  Sweeps of 1, 2, 3, 4 actions
+// unit for the rows of a model (sell_plans); with more, too few warps find work in the tiles in flight.  Sweeps of 1, 2, 3, 4 actions
 // a unit: 2.5 M states (1.2 GB) 230 / 213 / 221 / 236 us, 524,288 states 47.4 / 43.3 / 45.7 / 49.5;
 // 12.5 M states in BF16 (6.0 GB) 1,399 / 1,337 / 1,393 / 1,456, and 1,171 with the record's regions
 // found once a unit in 32-bit arithmetic.

@@ -755,20 +755,20 @@ def comparisons(args, native, torch, dev, stream):
 # DRAM bytes (read + write) per launch of the headline sweep kernels, from one ncu capture
 # of this exact kernel source each (large workload, padded and canonical CSR with the sliced
 # copy); reported only while the sources hash the same, since a changed kernel voids them.
-TRAFFIC_SOURCES = ("vc_sell.cu", "vc_internal.cuh", "vc_ptx.cuh")
-TRAFFIC_SOURCE_SHA = "ccd123720a0440f4264ecffae2b2e4c7708db65c275981d09ba7e4ea54b0bf9c"
-TRAFFIC_BYTES = {("large", "csr_f32", True, True): 1_196_185_088,
-                 ("large", "csr_f32", False, True): 1_195_722_752}
+TRAFFIC_SOURCES = ("vc_sell.cu", "vc_sell.cuh", "vc_internal.cuh", "vc_ptx.cuh")
+TRAFFIC_SOURCE_SHA = "20688bd4ec40e9768eaf1dfd151125c8b7e488befbfc8e56e6a5d01b799b3c6f"
+TRAFFIC_BYTES = {("large", "csr_f32", True, True): 1_194_862_848,
+                 ("large", "csr_f32", False, True): 1_194_674_688}
 
 
-# ncu speed-of-light figures of the batched loop's pass-1 kernel on the 512-instance batch,
-# attached to the batched roofline while the sources hash as captured: that sweep is bound
-# by gather latency at half occupancy, not by a memory roof, and these say how far each
-# unit is from its own peak.
-BATCH_SOL_SOURCES = ("vc_batch.cu", "vc_internal.cuh")
-BATCH_SOL_SHA = "e67621a040703bc539f2e76a5369e75f8b8b8f6eb229700aff8d1bdc6019604b"
-BATCH_SOL = {"kernel": "k_bpost_pair<5>", "dram_pct": 11.5, "l2_pct": 13.1, "sm_pct": 57.5,
-             "warps_active_pct": 34.6, "registers_per_thread": 80, "top_stall": "long scoreboard (V gathers)"}
+# ncu figures of the resident batched loop on the first 64 instances of the batched workload,
+# attached to the batched roofline while the sources hash as captured: the loop is bound by load
+# latency at 16 warps an SM and by its barriers, not by a memory roof.
+BATCH_SOL_SOURCES = ("vc_batch_loop.cu", "vc_batch.cuh", "vc_implicit.cuh", "vc_grid.cuh")
+BATCH_SOL_SHA = "614135bd563ecb70148a1b3ed279cfbe6b84684b820e4429941d52eb961a6f4c"
+BATCH_SOL = {"kernel": "k_batch_loop<0>, 64 instances", "dram_pct": 0.4, "l2_hit_pct": 86.8, "sm_pct": 35.3,
+             "warps_active_pct": 25.0, "registers_per_thread": 124, "issue_active_pct": 35.7,
+             "top_stall": "barrier 3.6 (slower SMs), wait 1.9, long scoreboard 1.9"}
 
 
 def _sources_sha(names):
@@ -792,15 +792,15 @@ def captured_traffic(args, info):
     return TRAFFIC_BYTES[key], f"ncu dram__bytes_read.sum + dram__bytes_write.sum, sources sha256 {sha[:16]}"
 
 
-# ncu speed-of-light figures of the implicit sweep's two kernels on the large workload,
-# attached to that variant while the kernel source hashes as captured: the sweep is bound
-# by gather latency and issue, not by a memory roof (its HBM fraction is low by design).
-IMPLICIT_SOL_SOURCES = ("vc_sweep.cu",)
-IMPLICIT_SOL_SHA = "79e3021f39c95e9a34dc40bbf3e7c264ba4567f09c922b7da7e06a346d0060c7"
-IMPLICIT_SOL = {"kernels": "k_post_pair<7, 0> / k_max_pair<7, 0>", "sm_pct": [55.0, 43.0],
-                "l2_pct": [14.7, 9.7], "dram_pct": [5.8, 9.1], "warps_active_pct": [49.6, 55.5],
-                "top_stall": ["not selected (issue-bound)", "long scoreboard (U gathers)"],
-                "bound": "instruction issue (pass 1) and gather latency (pass 2)"}
+# ncu figures of the resident implicit loop on the large workload, attached to that variant while
+# the kernel sources hash as captured: the loop is bound by issue, gather latency and its
+# barriers, not by a memory roof (its HBM fraction is low by design).
+IMPLICIT_SOL_SOURCES = ("vc_loop.cu", "vc_implicit.cuh", "vc_grid.cuh")
+IMPLICIT_SOL_SHA = "c3fa4199f73efba2c94cf8bc60289639d8add48dbbdb351cb5c9821af5a821bb"
+IMPLICIT_SOL = {"kernels": "k_vi_loop<7, 4, 0, 0> (20 sweeps)", "sm_pct": 46.9, "dram_pct": 0.3, "l2_hit_pct": 91.7,
+                "l1_hit_pct": 56.8, "warps_active_pct": 29.7, "issue_active_pct": 47.1, "registers_per_thread": 96,
+                "top_stall": "barrier 2.3, wait 2.1, long scoreboard 1.8, not selected 1.2",
+                "bound": "instruction issue, gather latency and two grid barriers a sweep"}
 
 
 def implicit_sol():

@@ -902,11 +902,13 @@ int sell_sweep32(Mdp* m, const float* V_in, float* V_out, int32_t* pi, float* qg
         SellRingArgs t;
         const long long cap = (long long)m->num_sms * m->plan.ctas_per_sm;
         const unsigned grid = (unsigned)(m->plan.ntiles < cap ? m->plan.ntiles : cap);
-        // one action a unit where a CTA has few tiles, so the length of a unit counts (12,500
-        // states: 10.6 us a sweep against 10.9), and in the self-transition sweep, whose rows are
-        // longer, of BF16 values (524,288 states: 64.9 against 79.7 us) or of a slab beyond the L2
-        // (2.5 M states 284 against 291 us; within it 100,000 states 17.1 against 15.9)
-        const bool one = m->plan.ntiles < 4LL * grid || (sc.self_loop && (bf16 || m->sell_bytes > (128LL << 20)));
+        // One action a unit where a CTA has one or two tiles, so the length of a unit counts (microseconds
+        // a sweep, two actions / one: 12,500 states 10.8 / 10.5, with the self-transition solve 11.3 /
+        // 10.7; 32,768 states, 3.4 tiles a CTA, 11.2 / 11.5 and 11.9 / 11.6).  From there on two are
+        // faster or as fast at every size: 62,500 states 13.4 / 14.0 and 13.8 / 14.4, 343,750 34.3 /
+        // 35.9 and 39.0 / 41.7, 2.5 M 221 / 235 and 288 / 290; BF16 the same without the self-transition
+        // solve, with it only one action is built (two took 75.9 us against 64.9 at 524,288 states).
+        const bool one = m->plan.ntiles < 2LL * grid || (sc.self_loop && bf16);
         const int per_unit = one ? 1 : m->plan.per_unit;
         t.ups = (m->A + per_unit - 1) / per_unit;
         t.div_nu = make_fastdiv((uint32_t)(m->plan.ts * t.ups));

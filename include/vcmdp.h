@@ -464,7 +464,8 @@ typedef struct vc_grad_stats {
  * dJ_dtheta: [2H+5] double on the device; lambda_out: [S] double (nullable).  Temporary
  * device memory for P_pi^T is stream-ordered (cudaMallocAsync) and released before
  * return: 16 bytes an entry of rows padded to the longest of 32 (1.8 to 3.5 times the
- * transpose's entries; about 380 bytes a state at 6 hosts) and up to some 64 MB of scratch.  Synchronises `stream`.  VC_ERR_ARG for a handle built from an explicit CSR.
+ * transpose's entries; about 380 bytes a state at 6 hosts) and some 64 MB of scratch
+ * (300 MB where a row has 6,000 entries).  Synchronises `stream`.  VC_ERR_ARG for a handle built from an explicit CSR.
  * Errors: VC_ERR_NOT_CONVERGED if the residual test is not met within max_sweeps.
  */
 int vc_value_grad(vc_mdp* m, const double* V, const int32_t* pi, const double* rho, double* dJ_dtheta,

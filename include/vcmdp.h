@@ -288,7 +288,8 @@ int vc_set_wait_limit(vc_mdp* m, int64_t polls);
  * The FP32 sweeps of an implicit handle or an unsliced pipelined matrix and the correction
  * solves run in resident kernels that hold the whole device (one SM for instances of at most
  * 8,192 or 2,048 states): a kernel of another stream starts when such a launch ends, which
- * it does after about 10 ms, and the next launch follows once that kernel has its SMs.
+ * it does after about 4 ms.  Threads that solve at the same time take turns launch by launch,
+ * so their number does not add to that wait.
  * Errors: VC_ERR_NOT_CONVERGED if max_sweeps ran out (outputs still written),
  * VC_ERR_ARG for tol <= 0 or max_sweeps < 1.
  */
@@ -527,7 +528,7 @@ int vc_batch_offsets(const vc_batch* b, int64_t* offsets);
 /*
  * Value iteration of every instance (Algorithm 3), each with its own gamma, tolerance test
  * (max(tol, 4 ulp(max|V_i|)) or FP32 stall) and sweep count, in a resident kernel (launches of
- * about 10 ms, see vc_value_iterate) or, beyond its limits, one graph launch; then,
+ * about 4 ms, see vc_value_iterate) or, beyond its limits, one graph launch; then,
  * unless VC_ITER_FP32_ONLY, every instance's argmax policy is evaluated by FP64 residual +
  * FP32 correction (BiCGSTAB for every instance in one graph launch; fixed-point sweeps with
  * VC_ITER_PLAIN_CORRECTION or if an instance breaks down) + FP64 update and certified by

@@ -7,6 +7,9 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
+#include <condition_variable>
+#include <deque>
 #include <map>
 #include <mutex>
 #include <string>
@@ -148,6 +151,47 @@ cudaError_t cached_occupancy(const void* fn, int threads, size_t smem, int* per_
     return e;
 }
 
+namespace {
+struct TurnQueue {
+    std::mutex mu;
+    std::condition_variable cv;
+    std::deque<unsigned long long> waiting;
+    unsigned long long next = 0;
+    bool taken = false;
+};
+constexpr int kTurnDevices = 64;
+TurnQueue g_turns[kTurnDevices];
+}  // namespace
+
+void ResidentTurn::take(int grid, int num_sms) {
+    if (device_ >= 0 || 2 * grid <= num_sms) return;
+    const int dev = current_device();
+    if (dev < 0 || dev >= kTurnDevices) return;
+    TurnQueue& q = g_turns[dev];
+    std::unique_lock<std::mutex> lk(q.mu);
+    const unsigned long long me = q.next++;
+    q.waiting.push_back(me);
+    const bool mine = q.cv.wait_for(lk, std::chrono::milliseconds(50), [&] { return !q.taken && q.waiting.front() == me; });
+    q.waiting.erase(std::find(q.waiting.begin(), q.waiting.end(), me));
+    if (mine) {
+        q.taken = true;
+        device_ = dev;
+    } else {
+        q.cv.notify_all();  // the next in line may be first now
+    }
+}
+
+void ResidentTurn::give() {
+    if (device_ < 0) return;
+    TurnQueue& q = g_turns[device_];
+    device_ = -1;
+    {
+        std::lock_guard<std::mutex> lk(q.mu);
+        q.taken = false;
+    }
+    q.cv.notify_all();
+}
+
 static int device_sms() {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 148;
@@ -240,8 +284,9 @@ static int loop32_resident(Mdp* m, float* buf0, float* buf1, double tol, long lo
     VC_CUDA(cudaMemcpyAsync(m->ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
     int rc;
     for (;;) {
-        rc = (m->fmt & 0xF) == VC_IMPLICIT ? launch_vi_loop(m, buf0, buf1, self_loop, st, launched)
-                                           : launch_csr_loop(m, buf0, buf1, self_loop, st, launched);
+        ResidentTurn turn;
+        rc = (m->fmt & 0xF) == VC_IMPLICIT ? launch_vi_loop(m, buf0, buf1, self_loop, st, turn, launched)
+                                           : launch_csr_loop(m, buf0, buf1, self_loop, st, turn, launched);
         if (rc || !*launched) return rc;
         if ((rc = read_ctl(m, st))) return rc;
         if (h.error & kErrTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
@@ -269,7 +314,8 @@ int time_solve_loop(Mdp* m, bool resident, int sweeps, cudaStream_t st, double* 
         int rc = VC_OK;
         bool launched = true;
         VC_CUDA(cudaEventRecord(e[0], st));
-        if (resident) rc = launch_csr_loop(m, buf[0], buf[1], 0, st, &launched);
+        ResidentTurn turn;
+        if (resident) rc = launch_csr_loop(m, buf[0], buf[1], 0, st, turn, &launched);
         for (int i = 0; !resident && !rc && i < sweeps; i++)
             rc = launch_sweep32(m, buf[i & 1], buf[1 - (i & 1)], nullptr, nullptr, SweepCtl{m->ctl, kModeLoop32, 1 - (i & 1), nullptr}, st);
         if (rc || !launched) return rc;

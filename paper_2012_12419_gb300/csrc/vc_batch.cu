@@ -1575,13 +1575,15 @@ static int resident_loop(Batch* b, double tol, long long max_sweeps, int flags, 
     a.hand_over = std::min(kHandOver, b->small_max);
     for (;;) {
         int h[2] = {0, 0};  // active instances, fault
+        ResidentTurn turn;
         VC_CUDA(cudaMemsetAsync(b->bar, 0, 8, st));
-        if ((rc = launch_batch_loop(a, b->mh, b->num_sms, (flags & VC_ITER_SELF_LOOP) != 0, st, resident))) return rc;
+        if ((rc = launch_batch_loop(a, b->mh, b->num_sms, (flags & VC_ITER_SELF_LOOP) != 0, st, turn, resident))) return rc;
         if (!*resident) return VC_OK;
         VC_CUDA(cudaMemcpyAsync(&h[0], b->active, 4, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaMemcpyAsync(&h[1], a.fault, 4, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaMemcpyAsync(&a.first, a.end, 8, cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
+        turn.give();
         if (h[1] & kLoopTimeout) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");
 #ifdef VC_DEBUG_BOUNDS
         int err = 0;

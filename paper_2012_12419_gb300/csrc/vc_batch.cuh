@@ -63,6 +63,6 @@ struct BatchLoopArgs {
     long long* end;           // LaunchEnd's word
 };
 int launch_batch_loop(const BatchLoopArgs& a, int max_hosts, int num_sms, bool self_loop, cudaStream_t st,
-                      bool* launched);
+                      ResidentTurn& turn, bool* launched);
 
 }  // namespace vc

@@ -325,13 +325,13 @@ __global__ void __launch_bounds__(kBatchLoopThreads, 1) k_batch_loop(BatchLoopAr
 }
 
 int launch_batch_loop(const BatchLoopArgs& a, int max_hosts, int num_sms, bool self_loop, cudaStream_t st,
-                      bool* launched) {
+                      ResidentTurn& turn, bool* launched) {
     *launched = false;
     if (max_hosts > kBatchLoopMaxH || a.n > kBatchLoopMaxN) return VC_OK;
     const void* fn = self_loop ? (const void*)k_batch_loop<true> : (const void*)k_batch_loop<false>;
     const size_t smem = 8 * ((size_t)a.n + 1) + 12 * (size_t)a.n;
     VC_CUDA(cached_set_max_dyn_smem(fn, 8 * (kBatchLoopMaxN + 1) + 12 * kBatchLoopMaxN));
-    return launch_resident(fn, num_sms, kBatchLoopThreads, smem, st, launched, a);
+    return launch_resident(fn, num_sms, kBatchLoopThreads, smem, st, turn, num_sms, launched, a);
 }
 
 }  // namespace vc

@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(kCsrLoopWarps * 32, 1) k_csr_loop(CsrLoopArgs 
 }
 
 template <typename VT, int APAD>
-static int csr_loop_run(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {
+static int csr_loop_run(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, ResidentTurn& turn,
+                        bool* launched) {
     const int warp_bytes = 2 * (loop_col_bytes((int)m->loop_cap) + loop_val_bytes<VT>((int)m->loop_cap));
     const int warps = std::min(kCsrLoopWarps, kCsrLoopSmem / warp_bytes);
     if (warps < 12) return VC_OK;  // rows too long for a warp's own staging
@@ -325,10 +326,11 @@ static int csr_loop_run(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStr
     const CsrLoopArgs a{m->S, m->A, (int)m->loop_cap, (float)m->gamma, m->row_ptr, m->col, m->val, m->scale, m->R};
     const void* fn = self_loop ? (const void*)k_csr_loop<VT, APAD, true> : (const void*)k_csr_loop<VT, APAD, false>;
     VC_CUDA(cached_set_max_dyn_smem(fn, kCsrLoopSmem));
-    return launch_resident(fn, grid, 32 * warps, (size_t)warps * warp_bytes, st, launched, a, buf0, buf1, m->ctl);
+    return launch_resident(fn, grid, 32 * warps, (size_t)warps * warp_bytes, st, turn, sms, launched, a, buf0, buf1, m->ctl);
 }
 
-int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {
+int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, ResidentTurn& turn,
+                    bool* launched) {
     *launched = false;
     const bool bf16 = (m->fmt & 0xF) == VC_CSR_BF16;
     // what the autotuner found, else every pipelined CSR schedule (the loop is the faster one at
@@ -343,8 +345,8 @@ int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_
     if (m->loop_cap <= 0 || capped || m->nnz_stored >= (1LL << 31) - 64) return VC_OK;
     auto go = [&](auto apad) {
         constexpr int AP = decltype(apad)::value;
-        return bf16 ? csr_loop_run<uint16_t, AP>(m, buf0, buf1, self_loop, st, launched)
-                    : csr_loop_run<float, AP>(m, buf0, buf1, self_loop, st, launched);
+        return bf16 ? csr_loop_run<uint16_t, AP>(m, buf0, buf1, self_loop, st, turn, launched)
+                    : csr_loop_run<float, AP>(m, buf0, buf1, self_loop, st, turn, launched);
     };
     switch (pow2_at_least(m->A)) {
         case 1: return go(std::integral_constant<int, 1>());

@@ -53,14 +53,12 @@ struct GridBarrier {
 };
 
 // A resident launch holds every SM, so kernels of other streams wait for its end: it ends itself
-// after about 10 ms (20 M cycles at 2 GHz, a tenth of the 100 ms synchronisation interval; the
-// host reads the control block and goes on with another launch, 50 to 130 us with the kernel's
-// start: at 4 ms a 48-instance batch took 2.7 % longer), at a sweep that all CTAs take from one
-// word.  CTA 0 writes it two
+// after about 4 ms (8 M cycles at 2 GHz; the host reads the control block and goes on with another
+// launch, some 30 us: under 1 %), at a sweep that all CTAs take from one word.  CTA 0 writes it two
 // sweeps ahead: whoever still reads for the sweep before finds a number that it has not
 // reached, and everyone has it after the next barrier.  Whole solves on one launch held the
 // device for up to 0.25 s.
-constexpr long long kLaunchCycles = 20'000'000;
+constexpr long long kLaunchCycles = 8'000'000;
 constexpr long long kLaunchSweeps = 1 << 20;
 
 struct LaunchEnd {
@@ -115,11 +113,12 @@ struct LoopVerdict {
 };
 
 // Cooperative launch; *launched = false (and nothing enqueued) when the grid cannot be
-// resident at once on this device.
+// resident at once on this device.  The caller keeps `turn` until it has read the result.
 template <typename... Args>
-int launch_resident(const void* kern, int grid, int threads, size_t smem, cudaStream_t st, bool* launched,
-                    Args... args) {
+int launch_resident(const void* kern, int grid, int threads, size_t smem, cudaStream_t st, ResidentTurn& turn,
+                    int num_sms, bool* launched, Args... args) {
     void* ptrs[] = {(void*)&args...};
+    turn.take(grid, num_sms);
     const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3((unsigned)threads), ptrs, smem, st);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         cudaGetLastError();

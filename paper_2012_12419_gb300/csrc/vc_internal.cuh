@@ -766,15 +766,31 @@ int autotune_csr(Mdp* m, int reps, cudaStream_t st, double* best_us);
 // Grid of the persistent state-parallel kernels.
 int state_grid(const Mdp* m);
 
+// A turn at holding the device.  While the resident launch of one thread runs, another's waits on
+// the device and takes over the moment it ends, without a gap for anyone else: with two threads
+// solving, a kernel of a third stream (of any priority) waited until one of their solves was over,
+// 250 ms.  So a thread takes a turn, first come first served, for each resident launch that fills
+// more than half of the SMs, from the launch to the host's read of its result.  The turn is a
+// courtesy, not a guard: who waits 50 ms for it goes on without.
+class ResidentTurn {
+public:
+    void take(int grid, int num_sms);
+    void give();
+    ~ResidentTurn() { give(); }
+
+private:
+    int device_ = -1;  // held on this device
+};
+
 // FP32 value-iteration loop of an implicit handle in one resident kernel (vc_loop.cu): enqueues
 // up to a bounded number of sweeps on the reset control block (buf0 / buf1 ping-pong,
 // starting from the sweeps done so far).  *launched is false when the device cannot hold the
 // grid at once (nothing was enqueued; the caller launches sweep by sweep).
-int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
+int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, ResidentTurn& turn, bool* launched);
 
 // The same loop over a stored matrix of any size (vc_csr_loop.cu); *launched is also false when
 // the matrix or its schedule is not one the loop serves.
-int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched);
+int launch_csr_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, ResidentTurn& turn, bool* launched);
 
 // Least power of two >= a (the lanes of a state in the CSR sweeps).
 inline int pow2_at_least(int a) {

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kKrThreads, 1) k_krylov(Op op, KrylovArgs k) {
 // Enqueues one launch.  The grid is at most one CTA per SM; where the device cannot hold it
 // at once (a partitioned GPU) it is halved until it can.
 template <typename Op>
-static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, cudaStream_t st) {
+static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, cudaStream_t st, ResidentTurn& turn) {
     const int sms = m->num_sms > 0 ? m->num_sms : 148;
     const int items = std::min(k.n, k.chains) / Op::kWidth;
     int grid = k.n <= kKrOneCta ? 1 : std::max(1, std::min(sms, items / kKrItems));
@@ -531,8 +531,8 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, cudaStrea
         const int per = (items + grid - 1) / grid;
         const int threads = std::min(kKrThreads, std::max(32, (per + 31) / 32 * 32));
         bool launched = false;
-        const int rc = launch_resident((const void*)k_krylov<Op>, (items + per - 1) / per, threads, 0, st, &launched,
-                                       op, k);
+        const int rc = launch_resident((const void*)k_krylov<Op>, (items + per - 1) / per, threads, 0, st, turn,
+                                       sms, &launched, op, k);
         if (rc || launched) return rc;
         if (grid == 1) return fail(VC_ERR_CUDA, "the correction solve's kernel does not fit the device");
     }
@@ -543,23 +543,23 @@ static int krylov_run(const Mdp* m, const Op& op, const KrylovArgs& k, cudaStrea
 // 2.01 / 1.66, 524,288 3.58 / 2.72; items of two states (Q even): 343,750 2.77 / 2.35.
 constexpr int kKrTwoPass = 120000;
 
-static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, cudaStream_t st) {
-    if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, st);
+static int krylov_launch(const Mdp* m, const int32_t* pi, const KrylovArgs& k, cudaStream_t st, ResidentTurn& turn) {
+    if (m->adj) return krylov_run(m, AdjProduct{(float)m->gamma, *m->adj}, k, st, turn);
     if (!m->has_model) {
         if ((m->fmt & 0xF) == VC_CSR_BF16) {
             RowProduct<uint16_t> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const uint16_t*)m->val, m->scale, pi};
-            return krylov_run(m, op, k, st);
+            return krylov_run(m, op, k, st, turn);
         }
         RowProduct<float> op{m->A, (float)m->gamma, m->row_ptr, m->col, (const float*)m->val, m->scale, pi};
-        return krylov_run(m, op, k, st);
+        return krylov_run(m, op, k, st, turn);
     }
     const bool two = m->S >= kKrTwoPass;
     auto go = [&](auto mh) -> int {
         constexpr int MH = decltype(mh)::value;
         if (two && MH <= 8 && wide_rows(m->md))
-            return krylov_run(m, ModelProduct2<MH, MH <= 8 ? 4 : 2>{m->md, m->c32, pi}, k, st);
-        if (two) return krylov_run(m, ModelProduct2<MH, 2>{m->md, m->c32, pi}, k, st);
-        return krylov_run(m, ModelProduct<MH>{m->md, m->c32, pi}, k, st);
+            return krylov_run(m, ModelProduct2<MH, MH <= 8 ? 4 : 2>{m->md, m->c32, pi}, k, st, turn);
+        if (two) return krylov_run(m, ModelProduct2<MH, 2>{m->md, m->c32, pi}, k, st, turn);
+        return krylov_run(m, ModelProduct<MH>{m->md, m->c32, pi}, k, st, turn);
     };
     switch (m->md.H) {
         case 1: return go(std::integral_constant<int, 1>());
@@ -602,7 +602,8 @@ int krylov_correct(Mdp* m, const int32_t* pi, const float* b, float* x, double t
     k.chains = state_grid(m) * kThreads;
     int rc;
     for (;;) {
-        if ((rc = krylov_launch(m, pi, k, st))) return rc;
+        ResidentTurn turn;
+        if ((rc = krylov_launch(m, pi, k, st, turn))) return rc;
         VC_CUDA(cudaMemcpyAsync(&h, m->kctl, sizeof(KrylovCtl), cudaMemcpyDeviceToHost, st));
         VC_CUDA(cudaStreamSynchronize(st));
         if (h.fault) return fail(VC_ERR_TIMEOUT, "a bounded device-side wait expired");

@@ -171,7 +171,7 @@ static int loop_threads(int per) {
 }
 
 template <int MH, int VW, bool SL>
-static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, bool* launched) {
+static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, ResidentTurn& turn, bool* launched) {
     const int items = m->S / VW;
     float* U = m->U32 + kUShift;
     const size_t smem = 4 * ((size_t)(SL ? 4 : 3) * m->S + kUPad);
@@ -188,20 +188,21 @@ static int vi_loop_run(Mdp* m, float* buf0, float* buf1, cudaStream_t st, bool* 
     const int sms = m->num_sms > 0 ? m->num_sms : 148;
     const int grid = std::min(sms, (items + kLoopItems - 1) / kLoopItems);
     const int per = (items + grid - 1) / grid;
-    return launch_resident((const void*)kern, (items + per - 1) / per, loop_threads(per), 0, st, launched, m->md, m->c32, buf0,
-                           buf1, U, m->U32s, m->ctl);
+    return launch_resident((const void*)kern, (items + per - 1) / per, loop_threads(per), 0, st, turn, sms, launched, m->md,
+                           m->c32, buf0, buf1, U, m->U32s, m->ctl);
 }
 
-int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, bool* launched) {
+int launch_vi_loop(Mdp* m, float* buf0, float* buf1, int self_loop, cudaStream_t st, ResidentTurn& turn,
+                   bool* launched) {
     const bool wide = wide_rows(m->md) && (((uintptr_t)buf0 | (uintptr_t)buf1) & 15) == 0;
     auto go = [&](auto mh) {
         constexpr int MH = decltype(mh)::value;
         constexpr int VW = MH <= 8 ? 4 : 2;
         if (self_loop)
-            return wide && VW == 4 ? vi_loop_run<MH, VW, true>(m, buf0, buf1, st, launched)
-                                   : vi_loop_run<MH, 2, true>(m, buf0, buf1, st, launched);
-        return wide && VW == 4 ? vi_loop_run<MH, VW, false>(m, buf0, buf1, st, launched)
-                               : vi_loop_run<MH, 2, false>(m, buf0, buf1, st, launched);
+            return wide && VW == 4 ? vi_loop_run<MH, VW, true>(m, buf0, buf1, st, turn, launched)
+                                   : vi_loop_run<MH, 2, true>(m, buf0, buf1, st, turn, launched);
+        return wide && VW == 4 ? vi_loop_run<MH, VW, false>(m, buf0, buf1, st, turn, launched)
+                               : vi_loop_run<MH, 2, false>(m, buf0, buf1, st, turn, launched);
     };
     switch (m->md.H) {
         case 1: return go(std::integral_constant<int, 1>());

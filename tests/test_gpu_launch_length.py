@@ -1,4 +1,4 @@
-"""A resident kernel ends its launch after some 10 ms (20 M cycles), so that kernels of other streams
+"""A resident kernel ends its launch after some 4 ms (8 M cycles), so that kernels of other streams
 get their turn: long solves take launches in proportion to their time, and where a launch ends
 changes no result (the points differ from run to run, the values must not)."""
 import pytest
@@ -10,7 +10,7 @@ from gpu_common import native_or_skip
 
 pytestmark = pytest.mark.gpu
 
-MS = 20.0  # 20 M cycles at 1 GHz: no launch is longer
+MS = 8.0  # 8 M cycles at 1 GHz: no launch is longer
 SLOW = dict(tol=1e-9, fp32_only=True, want_v64=False, raise_on_nonconvergence=False)
 
 

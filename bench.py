@@ -756,19 +756,19 @@ def comparisons(args, native, torch, dev, stream):
 # of this exact kernel source each (large workload, padded and canonical CSR with the sliced
 # copy); reported only while the sources hash the same, since a changed kernel voids them.
 TRAFFIC_SOURCES = ("vc_sell.cu", "vc_sell.cuh", "vc_internal.cuh", "vc_ptx.cuh")
-TRAFFIC_SOURCE_SHA = "a715ee422fc4ee068555295463c6a23001db12331669488e3f02fd6fb99ea5bf"
-TRAFFIC_BYTES = {("large", "csr_f32", True, True): 1_194_746_624,
-                 ("large", "csr_f32", False, True): 1_194_703_360}
+TRAFFIC_SOURCE_SHA = "e7d2ed421cc71baa7728947ce05334b2549f425baa3d82b26bac672465c75898"
+TRAFFIC_BYTES = {("large", "csr_f32", True, True): 1_194_802_944,
+                 ("large", "csr_f32", False, True): 1_194_644_224}
 
 
 # ncu figures of the resident batched loop on the first 64 instances of the batched workload,
 # attached to the batched roofline while the sources hash as captured: the loop is bound by load
 # latency at 16 warps an SM and by its barriers, not by a memory roof.
 BATCH_SOL_SOURCES = ("vc_batch_loop.cu", "vc_batch.cuh", "vc_implicit.cuh", "vc_grid.cuh")
-BATCH_SOL_SHA = "614135bd563ecb70148a1b3ed279cfbe6b84684b820e4429941d52eb961a6f4c"
-BATCH_SOL = {"kernel": "k_batch_loop<0>, 64 instances", "dram_pct": 0.4, "l2_hit_pct": 86.8, "sm_pct": 35.3,
-             "warps_active_pct": 25.0, "registers_per_thread": 124, "issue_active_pct": 35.7,
-             "top_stall": "barrier 3.6 (slower SMs), wait 1.9, long scoreboard 1.9"}
+BATCH_SOL_SHA = "dd3b8dc598047b8a30382b39085241c3e3dbad4a271a0ec9371b1746991ce9b6"
+BATCH_SOL = {"kernel": "k_batch_loop<0>, 64 instances", "dram_pct": 0.4, "l2_hit_pct": 86.6, "sm_pct": 35.1,
+             "warps_active_pct": 25.0, "registers_per_thread": 124, "issue_active_pct": 35.6,
+             "top_stall": "barrier 3.7 (slower SMs), wait 1.9, long scoreboard 1.9"}
 
 
 def _sources_sha(names):
@@ -796,10 +796,10 @@ def captured_traffic(args, info):
 # the kernel sources hash as captured: the loop is bound by issue, gather latency and its
 # barriers, not by a memory roof (its HBM fraction is low by design).
 IMPLICIT_SOL_SOURCES = ("vc_loop.cu", "vc_implicit.cuh", "vc_grid.cuh")
-IMPLICIT_SOL_SHA = "c3fa4199f73efba2c94cf8bc60289639d8add48dbbdb351cb5c9821af5a821bb"
-IMPLICIT_SOL = {"kernels": "k_vi_loop<7, 4, 0, 0> (20 sweeps)", "sm_pct": 46.9, "dram_pct": 0.3, "l2_hit_pct": 91.7,
-                "l1_hit_pct": 56.8, "warps_active_pct": 29.7, "issue_active_pct": 47.1, "registers_per_thread": 96,
-                "top_stall": "barrier 2.3, wait 2.1, long scoreboard 1.8, not selected 1.2",
+IMPLICIT_SOL_SHA = "4690e475a5d623b2c2b36ece95e240124b37cbc0f581ffc19c5d61e1519f434f"
+IMPLICIT_SOL = {"kernels": "k_vi_loop<7, 4, 0, 0> (20 sweeps)", "sm_pct": 47.2, "dram_pct": 0.3, "l2_hit_pct": 92.2,
+                "l1_hit_pct": 56.8, "warps_active_pct": 29.6, "issue_active_pct": 47.4, "registers_per_thread": 96,
+                "top_stall": "barrier 2.3, wait 2.1, long scoreboard 1.7, not selected 1.2",
                 "bound": "instruction issue, gather latency and two grid barriers a sweep"}
 
 

@@ -122,7 +122,6 @@ struct Sum3 {
 // met, the sum goes on scaled by 2^-32, which no sum of FP32 terms overflows; what that shifts
 // out lies more than 200 bits below the term.
 struct DotSum {
-    static constexpr int kWords = 4;
     static constexpr float kLarge = 0x1p96f, kDown = 0x1p-32f;
     static constexpr double kUp = 0x1p32;
     Sum3 v;
@@ -155,13 +154,13 @@ struct DotSum {
         v.merge(s, c, __shfl_xor_sync(0xffffffffu, given.e, o));
     }
     __device__ __forceinline__ double value() const { return scale == 1.0f ? v.value() : kUp * v.value(); }
-    __device__ __forceinline__ void put(float* w) const { w[0] = v.s, w[1] = v.c, w[2] = v.e, w[3] = scale; }
-    __device__ __forceinline__ void get(const float* w) { v.s = w[0], v.c = w[1], v.e = w[2], scale = w[3]; }
+    __device__ __forceinline__ float4 words() const { return make_float4(v.s, v.c, v.e, scale); }
+    __device__ __forceinline__ void set(const float4& w) { v.s = w.x, v.c = w.y, v.e = w.z, scale = w.w; }
 };
 
 struct KrShared {
     KrylovCtl c;                           // this CTA's copy of the scalars
-    float dot[2][kKrThreads / 32][DotSum::kWords];  // the warps' sums
+    float4 dot[2][kKrThreads / 32];        // the warps' sums
     unsigned int mx;                       // bits of the CTA's max |r|
     double tot[2];
     long long end, start;                  // iterations at which this launch ends, its first cycle
@@ -192,14 +191,14 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
     }
     t.half_warp_sum();
     const unsigned int mb = MX ? __reduce_max_sync(0xffffffffu, fbits(mx)) : 0u;
-    if (l == 0 || (D1 && l == 16)) t.put(sh.dot[l >> 4][w]);
+    if (l == 0 || (D1 && l == 16)) sh.dot[l >> 4][w] = t.words();
     if (MX && l == 0) atomicMax(&sh.mx, mb);
     __syncthreads();
     const int G = (int)gridDim.x;
     double* part = k.part + kr_part_set(stage) * kKrPartValues * G;
     if (w == 0) {
         DotSum sum;
-        if ((l & 15) < nw && (D1 || l < 16)) sum.get(sh.dot[l >> 4][l & 15]);
+        if ((l & 15) < nw && (D1 || l < 16)) sum.set(sh.dot[l >> 4][l & 15]);
         sum.align();
         sum.half_warp_sum();
         const double v0 = sum.value(), v1 = D1 ? __shfl_sync(0xffffffffu, v0, 16) : 0.0;
@@ -215,6 +214,7 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
         }
     }
     if (!bar.arrive_and_wait()) return false;
+    if (end && threadIdx.x == blockDim.x - 1) sh.end = end->read();  // beside warp 0's reads
     if (w == 0) {
         double v0 = 0.0, v1 = 0.0;
         unsigned int vm = 0u;
@@ -237,7 +237,6 @@ __device__ __forceinline__ bool kr_reduce(const KrylovArgs& k, KrShared& sh, Gri
         if (l == 0) {
             kr_advance(&sh.c, stage, v0, v1, (double)__uint_as_float(vm));
             if (MX) sh.mx = 0u;  // next written after the caller's barriers
-            if (end) sh.end = end->read();
         }
     }
     __syncthreads();
